@@ -7,10 +7,11 @@
 //                        rows are decided, and Algorithm 1's scan run, by
 //                        decide_rows, a second launch.
 //   fuse_verify_row      (kernel_row.cuh) the same decomposition with no
-//                        slice in shared memory (pass 1 from HBM, pass 2 from
-//                        the L2, four CTAs per SM) and the lean per-entry
-//                        arithmetic: the production program of the
-//                        stochastic JSD step (no debug outputs, delta = a - b).
+//                        slice in shared memory (pass 1 from HBM, four CTAs
+//                        per SM; a second pass from the L2 only for rows whose
+//                        decision needs it): the production programs of the
+//                        stochastic step (no per-row outputs, delta = a - b).
+//                        Its rows are decided by decide_blocks.
 //   fuse_verify_generic  (kernel_generic.cuh) one cluster per row, any
 //                        element-aligned input; folds the scan into the same
 //                        launch through a per-element ticket in the workspace.
@@ -48,17 +49,13 @@ struct Plan {
   long long ctas;  // grid size
   bool vector_path;
   bool row;          // the production row kernel (fuse_verify_row) runs
+  bool stoch, edge;  // its mode; its form for rows off the 16-byte boundaries
   int nt;            // threads per CTA (kRowThreads or kTThreads)
   int grid_y;        // the row kernel's grid is (C (K+1), B): grid_y = B (1 otherwise)
 };
 
-// Shared memory one SM offers its CTAs, and what each CTA costs beyond its
-// own allocation.
-constexpr int kSmemPerSm = 228 * 1024;
-constexpr int kSmemPerCta = 1024;
-
-const void* row_kernel(int dtype) {
-  return dtype == ASYMSPEC_FP32 ? row_kernel_f32() : row_kernel_bf16();
+const void* row_kernel(int dtype, bool stoch, bool edge) {
+  return dtype == ASYMSPEC_FP32 ? row_kernel_f32(stoch, edge) : row_kernel_bf16(stoch, edge);
 }
 
 
@@ -114,19 +111,19 @@ bool plan_tma(int V, int elt, int forced_C, Plan* pl) {
   return false;
 }
 
-// The production row kernel.  Pass 2 re-reads each row from the L2, so the
-// rows in flight (one per resident cluster) must stay well inside it, while
+// The production row kernel.  A second pass re-reads its row from the L2, so
+// the rows in flight (one per resident cluster) must stay well inside it, while
 // fewer CTAs per row give each warp a longer block over which the fixed
 // costs of a CTA (its launch, the first loads, the exchange of the pass-1
 // records) are spread.  With at least one wave of clusters of 8 (rows x 8 >=
 // 4 CTAs x SMs): the smallest C of kRowClusters whose resident clusters
-// hold at most kRowL2Budget of rows.  Measured on GB300 (kernel time, rows
-// in flight):
+// hold at most kRowL2Budget of rows.  Measured on GB300 with a second pass on
+// every row (kernel time, rows in flight):
 //   B=64, K=7, V=128256 bf16:  C=5 103.4 us (90 MB), C=6 97.3 us (75 MB), C=8 102.4 us (57 MB)
 //   B=32, K=8, V=151936 bf16:  C=6 70.7 us (88 MB), C=7 71.7 us (74 MB), C=8 75.8 us (67 MB)
 //   B=128, K=4, V=151936 fp32: C=12 207.9 us (84 MB), C=16 247.8 us (60 MB)
 // Smaller batches take C = 8.  A warp's block takes at most kWalkRounds
-// steps (the decision kernel's walk loads a whole block at once).  Only the
+// steps (the decision kernel's draw takes one vector of a block per thread).  Only the
 // pass-1 records live in shared memory.  forced_C: the caller's
 // asymspec_launch_opts.
 constexpr int kRowClusters[] = {4, 5, 6, 7, 8, 10, 12, 16};
@@ -148,17 +145,15 @@ DeviceShape device_shape() {
   return d;
 }
 
-const void* row_kernel(int dtype);
 cudaError_t prepare_kernel(const void* fn, int device);
 cudaError_t active_clusters(const void* fn, const Plan& pl, int device, int* out);
 
-bool plan_row(int V, int dtype, int forced_C, long long rows, Plan* pl) {
+bool plan_row(int V, int dtype, bool stoch, bool edge, int forced_C, long long rows, Plan* pl) {
   const int elt = elt_size(dtype);
   const int VE = 16 / elt;
-  auto width = [&](int C) {
-    const long long per = (static_cast<long long>(V) + C - 1) / C;
-    return round_up_ll(per, VE);
-  };
+  // (a row off the 16-byte boundaries may touch one vector more than it fills)
+  const long long span = edge ? static_cast<long long>(V) + VE - 1 : V;
+  auto width = [&](int C) { return round_up_ll((span + C - 1) / C, VE); };
   auto fits = [&](int C) {
     return width(C) / VE <= static_cast<long long>(kWalkRounds) * kRowThreads;
   };
@@ -172,7 +167,7 @@ bool plan_row(int V, int dtype, int forced_C, long long rows, Plan* pl) {
     if (rows * 8 < slots) {
       if (fits(8)) C = 8;
     } else {
-      const void* fn = row_kernel(dtype);
+      const void* fn = row_kernel(dtype, stoch, edge);
       const bool query = dev.ok && prepare_kernel(fn, dev.device) == cudaSuccess;
       for (int c : kRowClusters) {
         if (!fits(c)) continue;
@@ -205,6 +200,8 @@ bool plan_row(int V, int dtype, int forced_C, long long rows, Plan* pl) {
   pl->smem = row_shared_bytes(C) + kRingBytes;
   pl->group_stride = kGroupsMax;
   pl->nt = kRowThreads;
+  pl->stoch = stoch;
+  pl->edge = edge;
   return true;
 }
 
@@ -242,10 +239,17 @@ TmaLayout tma_layout(int B, int K, int C, int group_stride = kGroupsMax) {
   return L;
 }
 
-// prod_row: the call is the production stochastic JSD step (no debug
-// outputs, no per-row tokens, delta = a - b), which fuse_verify_row runs.
+// What the streaming row kernel could take of a call: its mode if it is a
+// production program (no per-row outputs, delta = a - b).
+enum RowProgram { kRowNone, kRowGreedy, kRowStochastic };
+
+RowProgram row_program(const asymspec_gate_params& gp) {
+  if ((gp.flags & ASYMSPEC_FLAG_DELTA_MASK) != ASYMSPEC_DELTA_AB) return kRowNone;
+  return gp.mode == ASYMSPEC_MODE_STOCHASTIC ? kRowStochastic : kRowGreedy;
+}
+
 int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, bool vec_ok,
-              size_t ws_bytes, bool prod_row, Plan* pl) {
+              size_t ws_bytes, RowProgram prog, Plan* pl) {
   const int elt = elt_size(dtype);
   const int forced_C = (opts && opts->cluster_size > 0) ? opts->cluster_size : 0;
   const int forced_kernel = opts ? opts->kernel : 0;
@@ -261,8 +265,9 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
   if (ws_bytes < cluster_ws_bytes(B, K)) return ASYMSPEC_ERR_WORKSPACE;
   bool ok = false;
   // (its grid is (C (K+1), B): B up to 65535)
-  if (forced_kernel != ASYMSPEC_KERNEL_GENERIC && vec_ok && prod_row && B <= 65535 &&
-      plan_row(V, dtype, forced_C, static_cast<long long>(B) * (K + 1), pl)) {
+  if (forced_kernel != ASYMSPEC_KERNEL_GENERIC && vec_ok && prog == kRowStochastic &&
+      B <= 65535 &&
+      plan_row(V, dtype, true, false, forced_C, static_cast<long long>(B) * (K + 1), pl)) {
     if (ws_bytes >= tma_layout(B, K, pl->C).total) {
       pl->kernel = ASYMSPEC_KERNEL_TMA;
       pl->VE = 16 / elt;
@@ -302,13 +307,16 @@ using KernelFn = const void*;  // a __global__ function taking KParams (or SPara
 
 // sel: the TMA kernel's program set (tma_program_set; 0 = run-time dispatch)
 KernelFn pick_kernel(const Plan& pl, int dtype, bool stoch, int sel = 0) {
-  if (pl.row) return row_kernel(dtype);
+  if (pl.row) return row_kernel(dtype, pl.stoch, pl.edge);
   if (pl.kernel == ASYMSPEC_KERNEL_TMA)
     return dtype == ASYMSPEC_FP32 ? tma_kernel_f32(stoch, sel) : tma_kernel_bf16(stoch, sel);
   return generic_kernel(dtype, pl.vector_path, stoch);
 }
 
-KernelFn pick_decide(int dtype, bool stoch) {
+KernelFn pick_decide(const Plan& pl, int dtype, bool stoch) {
+  if (pl.row)
+    return dtype == ASYMSPEC_FP32 ? decide_blocks_f32(stoch, pl.edge)
+                                  : decide_blocks_bf16(stoch, pl.edge);
   return dtype == ASYMSPEC_FP32 ? decide_kernel_f32(stoch) : decide_kernel_bf16(stoch);
 }
 
@@ -342,8 +350,7 @@ cudaError_t prepare_kernel(KernelFn fn, int device) {
 }
 
 // A kernel without clusters whose dynamic shared memory may reach max_bytes
-// (the decision kernel's walk staging: what its static records leave of the
-// per-CTA limit; the gather's restricted row of t).
+// (the gather's restricted row of t).
 cudaError_t prepare_plain_kernel(KernelFn fn, int device, int max_bytes) {
   std::lock_guard<std::mutex> lock(g_mu);
   const void* f = fn;
@@ -570,11 +577,8 @@ int asymspec_plan(int B, int K, int V, int dtype, const asymspec_gate_params* ga
   if (st) return st;
   const bool vec_ok = (static_cast<long long>(V) * elt_size(dtype)) % 16 == 0;
   Plan pl = {};
-  const bool stoch_p = gp.mode == ASYMSPEC_MODE_STOCHASTIC;
   st = make_plan(B, K, V, dtype, opts, vec_ok, asymspec_workspace_bytes(B, K, V),
-                 stoch_p && gp.divergence == ASYMSPEC_DIV_JSD &&
-                     (gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB,
-                 &pl);
+                 row_program(gp), &pl);
   if (st) return st;
   out->cluster_size = pl.C;
   out->block_threads = pl.kernel == ASYMSPEC_KERNEL_GENERIC ? kThreads : pl.nt;
@@ -637,10 +641,9 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   const bool vec_ok = (static_cast<long long>(V) * elt) % 16 == 0 && aligned(logits_full, 16) &&
                       aligned(logits_comp, 16) && aligned(logits_ver, 16);
   Plan pl = {};
-  const bool prod_row = stoch && gp.divergence == ASYMSPEC_DIV_JSD && !out_row_stats &&
-                        !out_fused_logprobs && !out_row_tokens &&
-                        (gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB;
-  st = make_plan(B, K, V, dtype, opts, vec_ok, workspace_bytes, prod_row, &pl);
+  const bool per_row_out = out_row_stats || out_fused_logprobs || out_row_tokens;
+  st = make_plan(B, K, V, dtype, opts, vec_ok, workspace_bytes,
+                 per_row_out ? kRowNone : row_program(gp), &pl);
   if (st) return st;
 
   KParams P;
@@ -682,9 +685,8 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   P.pass2_rec = nullptr;
   P.group_mass = nullptr;
   P.tma_threads = pl.nt;
-  P.row_blocks = pl.row ? 1 : 0;
+  P.head0 = static_cast<int>((reinterpret_cast<uintptr_t>(logits_full) % 16) / elt);
   // the chunk waits of the TMA kernel: bounded, or (test hook) giving up at once
-  P.walk_stage = 0;
   P.copy_wait_ns =
       (opts && (opts->test_flags & ASYMSPEC_TEST_COPY_GIVE_UP)) ? 0ull : kCopyTimeoutNs;
   P.tickets = reinterpret_cast<unsigned int*>(static_cast<char*>(workspace) +
@@ -719,27 +721,14 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
     // the rows' decisions and Algorithm 1's scan: one CTA per batch element
     // as a programmatic dependent launch: its launch overlaps the row
     // kernel's last CTAs, and it waits (griddepcontrol.wait) for that kernel
-    int warps = std::min(K + 1, kDecideThreads / 32);
-    // rows of the production row kernel: each warp stages the vectors of the
-    // inverse-CDF group it walks (at most one warp block: 3 streams x 32
-    // vectors per step) in shared memory
-    P.walk_stage = 0;
-    if (pl.row) {
-      const int nv = pl.W / pl.VE;
-      const int steps = (row_block_vectors(nv, pl.nt / 32) + 31) / 32;
-      P.walk_stage = 3 * steps * 32 * 16;
-      warps = std::min(warps, (kMaxSmem - kDecideSmemRows * 16) / P.walk_stage);
-    }
-    const KernelFn dfn = pick_decide(dtype, stoch);
-    e = prepare_plain_kernel(dfn, device, kMaxSmem - kDecideSmemRows * 16);
-    if (e != cudaSuccess) return cuda_fail(e);
+    const int threads = pl.row ? kDrawThreads : 32 * std::min(K + 1, kDecideThreads / 32);
+    const KernelFn dfn = pick_decide(pl, dtype, stoch);
     cudaLaunchConfig_t dcfg = {};
     cudaLaunchAttribute dattr[1];
     dattr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     dattr[0].val.programmaticStreamSerializationAllowed = 1;
     dcfg.gridDim = dim3(static_cast<unsigned>(B));
-    dcfg.blockDim = dim3(32 * warps);
-    dcfg.dynamicSmemBytes = static_cast<size_t>(warps) * P.walk_stage;
+    dcfg.blockDim = dim3(threads);
     dcfg.stream = static_cast<cudaStream_t>(stream);
     dcfg.attrs = dattr;
     dcfg.numAttrs = 1;

@@ -435,9 +435,8 @@ struct KParams {
   float* group_mass;    // [B(K+1)][C][group_stride] inverse-CDF group masses (stochastic)
   int group_stride;     // floats per row and CTA in group_mass (one per warp and round)
   int tma_threads;      // threads per CTA of the row kernel (its group layout)
-  int row_blocks;       // 1: fuse_verify_row's layout, one inverse-CDF group per warp block
   unsigned long long copy_wait_ns;  // limit of each bulk-copy wait (0: give up at once)
-  int walk_stage;       // decide_rows on fuse_verify_row's rows: staging bytes per warp
+  int head0;            // fuse_verify_row, EDGE: elements from a 16-byte boundary to the logits
 };
 
 // What pass 1 leaves for the decision of a row: the normalisers, the
@@ -448,7 +447,7 @@ struct __align__(16) RowStat {
   unsigned bad;
   int dtok;
   float da, db, dt;
-  float pad;
+  int path;  // fuse_verify_row: what its second pass did (kPath*)
 };
 
 
@@ -490,10 +489,12 @@ __device__ __forceinline__ RowScalars load_row_scalars(const KParams& P, int bi,
 // acceptance test of Eq. 4 (or its stochastic counterpart), the emitted
 // candidate, and the optional per-row outputs.  Returns the 16-byte row
 // record (accept bit, candidate, ASYMSPEC_DATA_* bits).
-// dtok/ad/bd/td: the draft token of this row and its three logits.
+// dtok/ad/bd/td: the draft token of this row and its three logits.  report:
+// this thread writes the row's errors (a warp may compute one row's record
+// in every lane; such callers ask for no per-row outputs).
 template <bool STOCH>
 __device__ int4 row_record(const KParams& P, long long row, int k, const RowResult& r, int dtok,
-                           float ad, float bd, float td, const RowScalars& sc) {
+                           float ad, float bd, float td, const RowScalars& sc, bool report = true) {
   const int V = P.V, K = P.K;
   const bool bonus = (k == K);
   unsigned err = 0;
@@ -573,7 +574,7 @@ __device__ int4 row_record(const KParams& P, long long row, int k, const RowResu
     P.row_tokens[static_cast<size_t>(row) * 2] = (r.is == INT_MAX) ? -1 : r.is;
     P.row_tokens[static_cast<size_t>(row) * 2 + 1] = cand;
   }
-  if (err && P.err_word) atomicOr(P.err_word, err);
+  if (report && err && P.err_word) atomicOr(P.err_word, err);
   return make_int4(accept, cand, static_cast<int>(err), 0);
 }
 

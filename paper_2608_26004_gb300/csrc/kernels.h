@@ -16,11 +16,13 @@ const void* tma_kernel_bf16_any_stoch();  // k_tma_bf16_any_s.cu
 const void* tma_kernel_f32_any_stoch();   // k_tma_f32_any_s.cu
 const void* tma_kernel_bf16(bool stoch, int sel);
 const void* tma_kernel_f32(bool stoch, int sel);
-// fuse_verify_row<T>, the production kernel of the stochastic JSD step
-// (k_row_bf16.cu, k_row_f32.cu)
-const void* row_kernel_bf16();
-const void* row_kernel_f32();
-// decide_rows<T, STOCH>, launched after fuse_verify_tma or fuse_verify_row (k_tma_*.cu)
+// fuse_verify_row<T, STOCH, EDGE>, the production programs, and
+// decide_blocks<T, STOCH, EDGE>, launched after it (k_row_bf16.cu, k_row_f32.cu)
+const void* row_kernel_bf16(bool stoch, bool edge);
+const void* row_kernel_f32(bool stoch, bool edge);
+const void* decide_blocks_bf16(bool stoch, bool edge);
+const void* decide_blocks_f32(bool stoch, bool edge);
+// decide_rows<T, STOCH>, launched after fuse_verify_tma (k_tma_*.cu)
 const void* decide_kernel_bf16(bool stoch);
 const void* decide_kernel_f32(bool stoch);
 // draft_kernel<T, VE, STOCH>, the drafter's draw (k_draft.cu)
