@@ -141,9 +141,10 @@ typedef struct {
 /* Kernels (asymspec_launch_opts.kernel, asymspec_launch_info.kernel). */
 #define ASYMSPEC_KERNEL_GENERIC 1  /* one cluster per row; any element-aligned input */
 #define ASYMSPEC_KERNEL_TMA 2      /* one cluster per row, then a decision kernel; rows
-                                      16-byte aligned.  The stochastic step without per-row
-                                      outputs and with delta = a - b runs the production row
-                                      kernel (slices read from HBM, and again from the L2 for
+                                      16-byte aligned.  The step without per-row outputs
+                                      and with delta = a - b runs the production row
+                                      kernel (in greedy mode unless this kernel or a test
+                                      hook is asked for; slices read from HBM, and again from the L2 for
                                       rows whose decision needs a second pass; C chosen so
                                       that the rows in flight stay within an L2 budget once a
                                       batch fills a wave of clusters of 8); every other
@@ -162,8 +163,8 @@ typedef struct {
   int32_t launches;        /* kernel launches of one call: 1 (the generic kernel) or 2
                               (a cluster row kernel and its decision kernel) */
   int32_t row_kernel;      /* 1 if ASYMSPEC_KERNEL_TMA runs its production row kernel
-                              (fuse_verify_row: the stochastic step without per-row
-                              outputs, delta = a - b), 0 otherwise */
+                              (fuse_verify_row: the step without per-row outputs,
+                              delta = a - b) in stochastic mode, 0 otherwise */
 } asymspec_launch_info;
 
 /* Fills *p with the paper's defaults: gamma 0.5, beta 1.0, lambda 0.1,

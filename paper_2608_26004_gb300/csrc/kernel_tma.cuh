@@ -1,6 +1,6 @@
 // Staged fuse-and-verify kernel for 16-byte aligned rows (every program
-// but the production stochastic JSD step, which fuse_verify_row in
-// kernel_row.cuh runs), and the decision kernel both row kernels feed.
+// but the production ones, which fuse_verify_row in kernel_row.cuh runs), and
+// its decision kernel.
 //
 // One cluster of C CTAs per row triple (one launch of the cluster per row;
 // the hardware hands out rows as clusters finish).  CTA r owns vocabulary
@@ -341,8 +341,7 @@ __device__ __forceinline__ void vec_masses(const f2 (&xa)[NP], const f2 (&xb)[NP
                                            f2 (&p)[NP], f2 (&qf)[NP], f2 (&r)[NP],
                                            f2 (&la2)[NP]) {
   // delta = a - b: the fused score in log2 units as t log2 e + (beta log2 e)(a - b),
-  // the form the production kernel (kernel_row.cuh) uses, so that a walk over
-  // either kernel's group masses sees identical vector masses
+  // the form fuse_verify_row (kernel_row.cuh) uses too
   const f2 bL2 = mul2(beta2, L2);
 #pragma unroll
   for (int h = 0; h < NP; ++h) {
