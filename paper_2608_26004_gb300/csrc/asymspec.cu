@@ -11,8 +11,9 @@
 //                        slice in shared memory (pass 1 from HBM, four CTAs
 //                        per SM; a second pass from the L2 only for rows whose
 //                        decision needs it): the production programs (no
-//                        per-row outputs, delta = a - b).  Its rows are
-//                        decided by decide_blocks.
+//                        per-row outputs, delta = a - b), also for rows off
+//                        the 16-byte boundaries.  Its rows are decided by
+//                        decide_blocks.
 //   fuse_verify_generic  (kernel_generic.cuh) one cluster per row, any
 //                        element-aligned input; folds the scan into the same
 //                        launch through a per-element ticket in the workspace.
@@ -249,7 +250,17 @@ RowProgram row_program(const asymspec_gate_params& gp) {
   return gp.mode == ASYMSPEC_MODE_STOCHASTIC ? kRowStochastic : kRowGreedy;
 }
 
-int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, bool vec_ok,
+// Rows off the 16-byte boundaries stream too: the generic kernel reads them
+// element by element (greedy bf16, K=4: 98 us at B=32, V=100003 against 23
+// streaming; 16 against 7 at B=8, V=16385, the shortest measured).  Shorter
+// rows keep the generic kernel's single launch.
+constexpr int kEdgeMinV = 16384;
+
+// How a call's rows lie in memory: every row on a 16-byte boundary; a, b and t
+// at the same offset from one; or neither.
+enum RowAlign { kRowsAligned, kRowsShifted, kRowsScattered };
+
+int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, RowAlign align,
               size_t ws_bytes, RowProgram prog, Plan* pl) {
   const int elt = elt_size(dtype);
   const int forced_C = (opts && opts->cluster_size > 0) ? opts->cluster_size : 0;
@@ -258,6 +269,7 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
   if (forced_kernel != 0 && forced_kernel != ASYMSPEC_KERNEL_GENERIC &&
       forced_kernel != ASYMSPEC_KERNEL_TMA)
     return ASYMSPEC_ERR_INVALID_ARG;
+  const bool vec_ok = align == kRowsAligned;
   pl->rows = static_cast<long long>(B) * (K + 1);
   pl->vector_path = vec_ok;
   pl->row = false;
@@ -271,9 +283,10 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
   // the test hook shortens, so a call that sets it, or asks for
   // ASYMSPEC_KERNEL_TMA in greedy mode, keeps the staged kernel.
   const bool stoch = prog == kRowStochastic;
+  const bool edge = align == kRowsShifted && V >= kEdgeMinV && !forced_kernel;
   const bool streams = stoch || (prog == kRowGreedy && !forced_kernel && !(opts && opts->test_flags));
-  if (forced_kernel != ASYMSPEC_KERNEL_GENERIC && vec_ok && streams && B <= 65535 &&
-      plan_row(V, dtype, stoch, false, forced_C, static_cast<long long>(B) * (K + 1), pl)) {
+  if (forced_kernel != ASYMSPEC_KERNEL_GENERIC && (vec_ok || edge) && streams && B <= 65535 &&
+      plan_row(V, dtype, stoch, edge, forced_C, pl->rows, pl)) {
     if (ws_bytes >= tma_layout(B, K, pl->C).total) {
       pl->kernel = ASYMSPEC_KERNEL_TMA;
       pl->VE = 16 / elt;
@@ -285,7 +298,7 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
     }
   }
   if (ok) {
-    // the production row kernel
+    // the streaming row kernel
   } else if (forced_kernel != ASYMSPEC_KERNEL_GENERIC && vec_ok && plan_tma(V, elt, forced_C, pl)) {
     // the TMA kernel leaves each row's results in the workspace; the generic
     // kernel, which needs only the records and tickets, runs when it is short
@@ -583,8 +596,8 @@ int asymspec_plan(int B, int K, int V, int dtype, const asymspec_gate_params* ga
   if (st) return st;
   const bool vec_ok = (static_cast<long long>(V) * elt_size(dtype)) % 16 == 0;
   Plan pl = {};
-  st = make_plan(B, K, V, dtype, opts, vec_ok, asymspec_workspace_bytes(B, K, V),
-                 row_program(gp), &pl);
+  st = make_plan(B, K, V, dtype, opts, vec_ok ? kRowsAligned : kRowsShifted,
+                 asymspec_workspace_bytes(B, K, V), row_program(gp), &pl);
   if (st) return st;
   out->cluster_size = pl.C;
   out->block_threads = pl.kernel == ASYMSPEC_KERNEL_GENERIC ? kThreads : pl.nt;
@@ -644,11 +657,15 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
       (out_error_word && !aligned(out_error_word, 4)))
     return ASYMSPEC_ERR_MISALIGNED;
   if (!workspace || !aligned(workspace, 16)) return ASYMSPEC_ERR_WORKSPACE;
-  const bool vec_ok = (static_cast<long long>(V) * elt) % 16 == 0 && aligned(logits_full, 16) &&
-                      aligned(logits_comp, 16) && aligned(logits_ver, 16);
+  const auto offset = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16; };
+  const RowAlign align =
+      offset(logits_full) != offset(logits_comp) || offset(logits_full) != offset(logits_ver)
+          ? kRowsScattered
+      : (static_cast<long long>(V) * elt) % 16 == 0 && !offset(logits_full) ? kRowsAligned
+                                                                            : kRowsShifted;
   Plan pl = {};
   const bool per_row_out = out_row_stats || out_fused_logprobs || out_row_tokens;
-  st = make_plan(B, K, V, dtype, opts, vec_ok, workspace_bytes,
+  st = make_plan(B, K, V, dtype, opts, align, workspace_bytes,
                  per_row_out ? kRowNone : row_program(gp), &pl);
   if (st) return st;
 
@@ -691,7 +708,7 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   P.pass2_rec = nullptr;
   P.group_mass = nullptr;
   P.tma_threads = pl.nt;
-  P.head0 = static_cast<int>((reinterpret_cast<uintptr_t>(logits_full) % 16) / elt);
+  P.head0 = static_cast<int>(offset(logits_full) / elt);
   // the chunk waits of the TMA kernel: bounded, or (test hook) giving up at once
   P.copy_wait_ns =
       (opts && (opts->test_flags & ASYMSPEC_TEST_COPY_GIVE_UP)) ? 0ull : kCopyTimeoutNs;

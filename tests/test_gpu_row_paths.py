@@ -1,5 +1,6 @@
-"""The production row kernel's second pass runs only for rows whose decision
-needs it; every outcome of that choice against the oracle.
+"""The streaming row kernel: its second pass runs only for rows whose decision
+needs it, and rows may start off the 16-byte boundaries; every outcome of both
+against the oracle.
 
 A row that passes its acceptance test at D = 0, or fails it at the gate's
 largest D, is decided by its normalisers alone; the others need the divergence,
@@ -17,8 +18,8 @@ pytestmark = pytest.mark.gpu
 GREEDY, STOCH = A.MODE_GREEDY, A.MODE_STOCHASTIC
 
 
-@pytest.fixture(scope="module")
-def torch():
+@pytest.fixture(scope="module", name="torch")
+def torch_():
     import torch as _torch
     assert _torch.cuda.is_available(), "the gpu tests need a CUDA device"
     from paper_2608_26004_gb300 import build
@@ -129,3 +130,79 @@ def test_more_rows_than_the_decision_kernel_keeps_on_chip(torch):
             o = run_oracle(batch, mode=STOCH, gamma=gamma, logprobs=False)
             assert err == 0
             check_decisions(batch, np.arange(3), L, N, o, STOCH)
+
+
+# ---------------------------------------------------------------- rows off the 16-byte boundaries
+
+def shifted(x, offset, torch):
+    """The logits in buffers that start `offset` elements after a 16-byte boundary."""
+    out = dict(x)
+    for key in "abt":
+        buf = torch.full((x[key].numel() + offset + 16,), float("nan"), dtype=x[key].dtype,
+                         device="cuda")
+        assert buf.data_ptr() % 16 == 0
+        view = buf[offset:offset + x[key].numel()]
+        view.copy_(x[key].reshape(-1))
+        out[key] = view.view(x[key].shape)
+    return out
+
+
+@pytest.mark.parametrize("mode", [GREEDY, STOCH])
+@pytest.mark.parametrize("dtype", [synth.BF16, synth.FP32])
+@pytest.mark.parametrize("V", [16384, 16385, 16387, 16391, 33333])
+def test_rows_at_odd_addresses(torch, V, dtype, mode):
+    # every offset of a row inside its first vector: odd V moves it from row to
+    # row, an offset base moves all rows; the buffers around the rows hold NaN
+    batch, _ = batch_over_the_threshold(4, 3, V, dtype, 40 + V, torch, mode)
+    o = run_oracle(batch, mode=mode, logprobs=False)
+    x = device_inputs(batch, torch)
+    for offset in (0, 1, 2, 3, 5) if dtype == synth.BF16 else (0, 1, 3):
+        g = run_gpu(batch, torch, mode=mode, full="row", inputs=shifted(x, offset, torch))
+        assert int(g["error_word"][0]) == 0
+        check_decisions(batch, np.arange(4), g["accept_len"], g["next_token"], o, mode)
+
+
+@pytest.mark.parametrize("mode", [GREEDY, STOCH])
+@pytest.mark.parametrize("dtype", [synth.BF16, synth.FP32])
+def test_edges_hold_the_answer(torch, dtype, mode):
+    # the emitted token, the draft token and the spike of every row among the
+    # first or last elements of the row, which no whole vector holds
+    B, K, V = 6, 2, 16391
+    for at in (0, 1, 2, V - 3, V - 2, V - 1):
+        batch, _ = batch_over_the_threshold(B, K, V, dtype, 7000 + at, torch, mode)
+        bits = np.float32(30.0)
+        big = (bits.view(np.uint32) >> 16).astype(np.uint16) if dtype == synth.BF16 else bits
+        batch.logits_ver[..., at] = big
+        batch.draft_tokens[::2] = at
+        for cluster in (0, 5, 16):
+            g = run_gpu(batch, torch, mode=mode, full="row", cluster_size=cluster)
+            o = run_oracle(batch, mode=mode, logprobs=False)
+            assert int(g["error_word"][0]) == 0
+            check_decisions(batch, np.arange(B), g["accept_len"], g["next_token"], o, mode)
+        batch.logits_full[1, 0, at] = np.float32("nan").view(np.uint32) >> 16 \
+            if dtype == synth.BF16 else np.nan
+        g = run_gpu(batch, torch, mode=mode, full="row")
+        assert g["accept_len"][1] == -1 and (np.delete(g["accept_len"], 1) >= 0).all()
+
+
+def test_an_overflowing_sum_beside_an_edge(torch):
+    batch, _ = batch_over_the_threshold(3, 2, 16391, synth.FP32, 8, torch, STOCH)
+    for arr in (batch.logits_full, batch.logits_comp, batch.logits_ver):
+        arr[0, 1, 0] = 150.0
+        arr[1, 0, 16390] = 150.0
+        arr[2, 2, 9000] = 150.0
+    for mode in (GREEDY, STOCH):
+        L, N, err = accept_and_next(batch, torch, mode)
+        o = run_oracle(batch, mode=mode, logprobs=False)
+        assert err == 0
+        check_decisions(batch, np.arange(3), L, N, o, mode)
+
+
+def test_rows_at_different_offsets_take_the_generic_kernel(torch):
+    batch, _ = batch_over_the_threshold(2, 2, 16385, synth.BF16, 12, torch, STOCH)
+    x = device_inputs(batch, torch)
+    y = shifted(x, 3, torch)
+    x["b"] = y["b"]
+    g = run_gpu(batch, torch, mode=STOCH, full="row", inputs=x)
+    o = run_oracle(batch, mode=STOCH, logprobs=False)
+    check_decisions(batch, np.arange(2), g["accept_len"], g["next_token"], o, STOCH)
