@@ -231,15 +231,25 @@ struct Streams {
   const T *a, *b, *t;
 };
 
+// 16 bytes global -> shared, skipped (without a branch) unless `on`.
+__device__ __forceinline__ void cp_async16_if(void* smem, const void* gmem, bool on) {
+  asm volatile(
+      "{ .reg .pred p; setp.ne.s32 p, %2, 0; @p cp.async.cg.shared.global [%0], [%1], 16; }" ::"r"(
+          smem_u32(smem)),
+      "l"(gmem), "r"(static_cast<int>(on))
+      : "memory");
+}
+
 // The lane's vector at element offset o of the streams into ring slot `slot`.
 template <typename T, bool AB, bool TT>
-__device__ __forceinline__ void ring_issue(uint4* ring, int slot, const Streams<T>& g, size_t o) {
+__device__ __forceinline__ void ring_issue(uint4* ring, int slot, const Streams<T>& g, size_t o,
+                                           bool on) {
   uint4* d = ring + slot * 96 + (threadIdx.x & 31);
   if (AB) {
-    cp_async16(d, g.a + o);
-    cp_async16(d + 32, g.b + o);
+    cp_async16_if(d, g.a + o, on);
+    cp_async16_if(d + 32, g.b + o, on);
   }
-  if (TT) cp_async16(d + 64, g.t + o);
+  if (TT) cp_async16_if(d + 64, g.t + o, on);
 }
 template <typename T, bool AB, bool TT>
 __device__ __forceinline__ void ring_read(const uint4* ring, int slot, RawVec<T>& va,
@@ -252,29 +262,50 @@ __device__ __forceinline__ void ring_read(const uint4* ring, int slot, RawVec<T>
   }
   if (TT) vt.v = d[64];
 }
-// Before step r (r >= 1) reads its slot: step r + kRing - 1 into the slot
-// step r - 1 used (slot `slot`, a constant once the loops are unrolled).
-// That slot's values were consumed by instructions this thread has already
-// issued, so the copy cannot overwrite unread data.  g: the lane's vector of
-// step 0 (vector i0 of the slice) of each stream.
-template <typename T, bool AB, bool TT>
-__device__ __forceinline__ void ring_refill(uint4* ring, int slot, const Streams<T>& g, int i0,
-                                            int v1, int r) {
-  constexpr int VE = 16 / static_cast<int>(sizeof(T));
-  const int q = r + kRing - 1;
-  if (i0 + 32 * q < v1) ring_issue<T, AB, TT>(ring, slot, g, static_cast<size_t>(q) * 32 * VE);
-  cp_async_commit();
-}
 // The first kRing steps of a pass into the ring (one group each, empty past
-// the block's end).
+// the block's end).  g: the lane's vector of step 0 (vector i0 of the slice)
+// of each stream.
 template <typename T, bool AB, bool TT>
 __device__ __forceinline__ void ring_prologue(uint4* ring, const Streams<T>& g, int i0, int v1) {
   constexpr int VE = 16 / static_cast<int>(sizeof(T));
 #pragma unroll
   for (int q = 0; q < kRing; ++q) {
-    if (i0 + 32 * q < v1) ring_issue<T, AB, TT>(ring, q, g, static_cast<size_t>(q) * 32 * VE);
+    ring_issue<T, AB, TT>(ring, q, g, static_cast<size_t>(q) * 32 * VE, i0 + 32 * q < v1);
     cp_async_commit();
   }
+}
+// use(r, va, vb, vt) for every step r of vectors [v0, v1) the lane has a
+// vector in, after the prologue.  kRing whole steps at a time with constant
+// slots and no branch: step r + kRing goes into the slot step r was just used
+// from (its values were consumed by instructions this thread has already
+// issued, so the copy cannot overwrite unread data).  At most kRing steps
+// remain after those, all of them already issued.
+template <typename T, bool AB, bool TT, typename Use>
+__device__ __forceinline__ void ring_steps(uint4* ring, const Streams<T>& g, int v0, int v1,
+                                           Use&& use) {
+  constexpr int VE = 16 / static_cast<int>(sizeof(T));
+  const int i0 = v0 + static_cast<int>(threadIdx.x & 31);
+  const int whole = (v1 - v0) / 32;
+  RawVec<T> va, vb, vt;
+  int r = 0;
+  for (; r + kRing <= whole; r += kRing) {
+#pragma unroll
+    for (int u = 0; u < kRing; ++u) {
+      cp_async_wait<kRing - 1>();
+      ring_read<T, AB, TT>(ring, u, va, vb, vt);
+      use(r + u, va, vb, vt);
+      ring_issue<T, AB, TT>(ring, u, g, static_cast<size_t>(r + u + kRing) * 32 * VE,
+                            i0 + 32 * (r + u + kRing) < v1);
+      cp_async_commit();
+    }
+  }
+  cp_async_wait<0>();
+#pragma unroll 1
+  for (int u = 0; i0 + 32 * r < v1; ++r, ++u) {
+    ring_read<T, AB, TT>(ring, u, va, vb, vt);
+    use(r, va, vb, vt);
+  }
+  __syncwarp();
 }
 
 // ---------------------------------------------------------------- pass 1
@@ -317,8 +348,8 @@ __device__ __forceinline__ float vmax_nan(const f2 (&x)[NP]) {
   }
 }
 
-// Pass 1 over vectors [v0, v1) of the slice (R steps; g: the lane's vector
-// v0 + lane of each stream), read through the warp's ring (the caller issued
+// Pass 1 over vectors [v0, v1) of the slice (g: the lane's vector v0 + lane
+// of each stream), read through the warp's ring (the caller issued
 // the prologue), with one fixed reference per warp and stream: the largest
 // of the first pairs of the lanes' first vectors.  vec0: the row's index of
 // vector v0 + lane; lastvec: the row's last vector.  chk: a non-finite a or b
@@ -327,7 +358,7 @@ __device__ __forceinline__ float vmax_nan(const f2 (&x)[NP]) {
 // finite (the warp then redoes its block with running maxima).  Every lane
 // ends with the warp's record.
 template <typename T, int PROG, bool EDGE>
-__device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int v0, int v1, int R,
+__device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int v0, int v1,
                                           float beta, bool chk, const EdgeVals& ed, int vec0,
                                           int lastvec, W1& e) {
   constexpr int NP = RawVec<T>::NP;
@@ -341,8 +372,8 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
   const int i0 = v0 + static_cast<int>(threadIdx.x & 31);
   float ra0 = -INFINITY, rb0 = -INFINITY, r30 = -INFINITY;
   cp_async_wait<kRing - 1>();  // step 0 (this lane's own copies)
-  RawVec<T> va, vb, vt;
   if (i0 < v1) {
+    RawVec<T> va, vb, vt;
     ring_read<T, AB, true>(ring, 0, va, vb, vt);
     if (SUM3) {
       const f2 t2 = vt.pair(0);
@@ -373,46 +404,34 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
   f2 acc_a = 0ull, acc_b = 0ull, acc_3 = 0ull, fin = 0ull;
   float best = -INFINITY;
   int rbest = -1;
-  // unrolled by the ring's depth, so that every slot is a constant
-  for (int r0 = 0; r0 < R; r0 += kRing) {
+  ring_steps<T, AB, true>(ring, g, v0, v1, [&](int r, const RawVec<T>& va, const RawVec<T>& vb,
+                                               const RawVec<T>& vt) {
+    f2 sc[NP];  // the argmax's scores
 #pragma unroll
-    for (int u = 0; u < kRing; ++u) {
-      const int r = r0 + u;
-      if (r >= R) break;
-      if (r > 0) {
-        ring_refill<T, AB, true>(ring, (u + kRing - 1) % kRing, g, i0, v1, r);
-        cp_async_wait<kRing - 1>();
-      }
-      if (i0 + 32 * r < v1) {
-        if (r > 0) ring_read<T, AB, true>(ring, u, va, vb, vt);
-        f2 sc[NP];  // the argmax's scores
-#pragma unroll
-        for (int h = 0; h < NP; ++h) {
-          const f2 t2 = vt.pair(h);
-          if (AB) {
-            const f2 a2 = va.pair(h), b2 = vb.pair(h);
-            const f2 amb = sub2(a2, b2);
-            if (DRAFT) {
-              acc_a = add2(acc_a, ex2_2(fma2(a2, L2, nA2)));
-              acc_b = add2(acc_b, ex2_2(fma2(b2, L2, nB2)));
-              fin = fma2(amb, 0ull, fin);  // 0 x (non-finite) is NaN
-            }
-            if (STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, fma2(bL2, amb, n32))));
-            if (ARG) sc[h] = fma2(beta2, amb, t2);
-          } else {
-            sc[h] = t2;
-          }
-          if (SUM3 && !STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, n32)));
+    for (int h = 0; h < NP; ++h) {
+      const f2 t2 = vt.pair(h);
+      if (AB) {
+        const f2 a2 = va.pair(h), b2 = vb.pair(h);
+        const f2 amb = sub2(a2, b2);
+        if (DRAFT) {
+          acc_a = add2(acc_a, ex2_2(fma2(a2, L2, nA2)));
+          acc_b = add2(acc_b, ex2_2(fma2(b2, L2, nB2)));
+          fin = fma2(amb, 0ull, fin);  // 0 x (non-finite) is NaN
         }
-        if (ARG) {
-          // strictly larger wins, so the lane's earliest vector keeps a tie
-          const float c = vmax_nan(sc);
-          rbest = c > best ? r : rbest;
-          best = max_nan(best, c);
-        }
+        if (STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, fma2(bL2, amb, n32))));
+        if (ARG) sc[h] = fma2(beta2, amb, t2);
+      } else {
+        sc[h] = t2;
       }
+      if (SUM3 && !STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, n32)));
     }
-  }
+    if (ARG) {
+      // strictly larger wins, so the lane's earliest vector keeps a tie
+      const float c = vmax_nan(sc);
+      rbest = c > best ? r : rbest;
+      best = max_nan(best, c);
+    }
+  });
   if (EDGE && ed.own) {
     const float amb = ed.a - ed.b;
     if (DRAFT) {
@@ -526,12 +545,11 @@ enum : int { kDivNone = 0, kDivJsd = 1, kDivKl = 2 };
 // warp's sums (every lane ends with them): msum is the mass of the warp's
 // inverse-CDF group.
 template <typename T, int DIV, bool RES, bool EDGE>
-__device__ __forceinline__ void row_pass2(uint4* ring, const Streams<T>& g, int v0, int v1, int R,
+__device__ __forceinline__ void row_pass2(uint4* ring, const Streams<T>& g, int v0, int v1,
                                           const ResConst& k, const EdgeVals& ed, float& jsum,
                                           float& msum) {
   constexpr int NP = RawVec<T>::NP;
   f2 jacc = 0ull, macc = 0ull;
-  const int i0 = v0 + static_cast<int>(threadIdx.x & 31);
   auto take = [&](f2 a2, f2 b2, f2 t2) {
     f2 amb, p;
     if (RES) {
@@ -545,21 +563,11 @@ __device__ __forceinline__ void row_pass2(uint4* ring, const Streams<T>& g, int 
     if (DIV == kDivJsd) jacc = jsd_pair(amb, p, k, jacc);
     if (DIV == kDivKl) jacc = kl_pair(amb, p, k, jacc);
   };
-  for (int r0 = 0; r0 < R; r0 += kRing) {
+  ring_steps<T, true, RES>(ring, g, v0, v1, [&](int, const RawVec<T>& va, const RawVec<T>& vb,
+                                                const RawVec<T>& vt) {
 #pragma unroll
-    for (int u = 0; u < kRing; ++u) {
-      const int r = r0 + u;
-      if (r >= R) break;
-      if (r > 0) ring_refill<T, true, RES>(ring, (u + kRing - 1) % kRing, g, i0, v1, r);
-      cp_async_wait<kRing - 1>();
-      if (i0 + 32 * r < v1) {
-        RawVec<T> va, vb, vt;
-        ring_read<T, true, RES>(ring, u, va, vb, vt);
-#pragma unroll
-        for (int h = 0; h < NP; ++h) take(va.pair(h), vb.pair(h), RES ? vt.pair(h) : 0ull);
-      }
-    }
-  }
+    for (int h = 0; h < NP; ++h) take(va.pair(h), vb.pair(h), RES ? vt.pair(h) : 0ull);
+  });
   if (EDGE && ed.own) take(pk(ed.a, kEdgeNone), pk(ed.b, kEdgeNone), pk(ed.t, kEdgeNone));
   float j = hsum2(jacc), m = hsum2(macc), z0 = 0.f, z1 = 0.f;
   if (DIV == kDivKl) j = -j;
@@ -730,7 +738,6 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
   // the block's whole vectors [v0, v1)
   const int v0 = EDGE ? max(b0, cut.in0 - s0) : b0;
   const int v1 = EDGE ? max(v0, min(b1, cut.in1 - s0)) : b1;
-  const int R = (v1 - v0 + 31) / 32;
   const int i0 = v0 + lane;
   Streams<T> g;  // the lane's first vector
   {
@@ -786,7 +793,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
   W1 e;
   auto pass1 = [&](auto prog) {
     constexpr int PROG = decltype(prog)::value;
-    const bool ovf = row_pass1<T, PROG, EDGE>(ring, g, v0, v1, R, P.beta, chk, ed, s0 + i0,
+    const bool ovf = row_pass1<T, PROG, EDGE>(ring, g, v0, v1, P.beta, chk, ed, s0 + i0,
                                               cut.nvec - 1, e);
     if (PROG != kGreedyBonusT && PROG != kGreedyBonusS && __any_sync(0xffffffffu, ovf)) {
       // an entry far above the warp's reference (or non-finite data): redo
@@ -887,9 +894,9 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
     ring_prologue<T, true, STOCH>(ring, g, i0, v1);
     const bool jsd = P.divergence == ASYMSPEC_DIV_JSD;
     if (STOCH && path == kPathReject)
-      row_pass2<T, kDivNone, STOCH, EDGE>(ring, g, v0, v1, R, kc, ed, jsum, msum);
-    else if (jsd) row_pass2<T, kDivJsd, STOCH, EDGE>(ring, g, v0, v1, R, kc, ed, jsum, msum);
-    else row_pass2<T, kDivKl, STOCH, EDGE>(ring, g, v0, v1, R, kc, ed, jsum, msum);
+      row_pass2<T, kDivNone, STOCH, EDGE>(ring, g, v0, v1, kc, ed, jsum, msum);
+    else if (jsd) row_pass2<T, kDivJsd, STOCH, EDGE>(ring, g, v0, v1, kc, ed, jsum, msum);
+    else row_pass2<T, kDivKl, STOCH, EDGE>(ring, g, v0, v1, kc, ed, jsum, msum);
     cp_async_wait<0>();
     if (jsd && path == kPathFull && !(fabsf(jsum) <= 3.402823466e38f))
       jsum = row_jsd_wide<T, EDGE>(g, v0, v1, A2, B2, ed);
