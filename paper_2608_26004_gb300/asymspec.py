@@ -11,6 +11,7 @@ or fails to load, every call raises.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -309,7 +310,15 @@ def version() -> int:
 # ----------------------------------------------------------------- PyTorch
 
 def _ptr(t):
-    return 0 if t is None else int(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
+
+
+def _stream(torch, dev) -> int:
+    """The handle of the current stream of a tensor's device.  The raw-handle
+    query costs 0.1 us where building torch.cuda.current_stream's object takes
+    2.3 us of a 16 us call (B=1, K=4, V=32000)."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(dev.index) if raw else torch.cuda.current_stream(dev).cuda_stream
 
 
 class FuseVerify:
@@ -346,20 +355,21 @@ class FuseVerify:
                  fused_logprobs=False, cluster_size=0, kernel=KERNEL_AUTO, out=None,
                  delta_source=DELTA_AB, test_flags=0, block_threads=0):
         import torch
-        B, K1, V = logits_full.shape
+        shape, kind = logits_full.shape, logits_full.dtype
+        B, K1, V = shape
         K = K1 - 1
         if K != self.K or B > self.B_max:
             raise ValueError("batch does not fit this workspace")
-        self._ensure(V)
-        if logits_full.dtype == torch.float32:
+        if self.workspace is None or V > self.V_ws:
+            self._ensure(V)
+        if kind == torch.float32:
             dtype = FP32
-        elif logits_full.dtype == torch.bfloat16:
+        elif kind == torch.bfloat16:
             dtype = BF16
         else:
             raise TypeError("logits must be float32 or bfloat16")
         for x in (logits_full, logits_comp, logits_ver):
-            if not x.is_cuda or not x.is_contiguous() or x.dtype != logits_full.dtype \
-                    or tuple(x.shape) != (B, K1, V):
+            if not x.is_cuda or not x.is_contiguous() or x.dtype != kind or x.shape != shape:
                 raise ValueError("logits must be contiguous CUDA tensors of one shape and dtype")
         dev = logits_full.device
         res = out if out is not None else {}
@@ -376,15 +386,14 @@ class FuseVerify:
         gate = gate_params(gamma, beta, lam, mode, divergence, fuse_bonus, delta_source)
         opts = (LaunchOpts(cluster_size, block_threads, kernel, test_flags)
                 if (cluster_size or kernel or test_flags or block_threads) else None)
-        stream = torch.cuda.current_stream(dev).cuda_stream
         st = fuse_verify_ex(
-            _ptr(logits_full), _ptr(logits_comp), _ptr(logits_ver), _ptr(draft_tokens),
-            _ptr(draft_probs), _ptr(uniforms), B, K, V, dtype, gate,
-            _ptr(res["accept_len"]), _ptr(res["next_token"]), _ptr(self.workspace),
-            self.nbytes, _ptr(res.get("row_stats") if row_stats else None),
-            _ptr(res.get("row_tokens") if row_tokens else None),
-            _ptr(res.get("fused_logprobs") if fused_logprobs else None),
-            _ptr(res["error_word"]), opts, stream)
+            logits_full.data_ptr(), logits_comp.data_ptr(), logits_ver.data_ptr(),
+            _ptr(draft_tokens), _ptr(draft_probs), _ptr(uniforms), B, K, V, dtype, gate,
+            _ptr(res["accept_len"]), _ptr(res["next_token"]), self.workspace.data_ptr(),
+            self.nbytes, _ptr(res["row_stats"]) if row_stats else 0,
+            _ptr(res["row_tokens"]) if row_tokens else 0,
+            _ptr(res["fused_logprobs"]) if fused_logprobs else 0,
+            _ptr(res["error_word"]), opts, _stream(torch, dev))
         if st != OK:
             raise AsymSpecError(st, "asymspec_fuse_verify_ex")
         return res
@@ -404,10 +413,8 @@ def draft_tokens(logits, uniforms=None, *, mode=MODE_GREEDY, cluster_size=0, out
         raise TypeError("logits must be float32 or bfloat16")
     if not logits.is_cuda or not logits.is_contiguous():
         raise ValueError("logits must be a contiguous CUDA tensor")
-    lead, V = tuple(logits.shape[:-1]), int(logits.shape[-1])
-    rows = 1
-    for n in lead:
-        rows *= n
+    *lead, V = logits.shape
+    rows = math.prod(lead)
     if mode == MODE_STOCHASTIC:
         if uniforms is None or uniforms.dtype != torch.float32 or not uniforms.is_cuda \
                 or not uniforms.is_contiguous() or uniforms.numel() != rows:
@@ -416,10 +423,9 @@ def draft_tokens(logits, uniforms=None, *, mode=MODE_GREEDY, cluster_size=0, out
     tokens, probs = out if out is not None else (
         torch.empty(lead, dtype=torch.int32, device=dev),
         torch.empty(lead, dtype=torch.float32, device=dev))
-    stream = torch.cuda.current_stream(dev).cuda_stream
-    st = draft_sample(_ptr(logits), rows, V, dtype, mode,
+    st = draft_sample(logits.data_ptr(), rows, V, dtype, mode,
                       _ptr(uniforms) if mode == MODE_STOCHASTIC else 0,
-                      _ptr(tokens), _ptr(probs), cluster_size, stream)
+                      _ptr(tokens), _ptr(probs), cluster_size, _stream(torch, dev))
     if st != OK:
         raise AsymSpecError(st, "asymspec_draft_sample")
     return tokens, probs
