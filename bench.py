@@ -37,9 +37,10 @@ WORKLOAD_CFG = 2
 FALLBACK_HBM_GBS = 6800.0
 CSRC = os.path.join(ROOT, "paper_2608_26004_gb300", "csrc")
 KERNEL_SRCS = ("asymspec.cu", "device_common.cuh", "kernel_generic.cuh", "kernel_tma.cuh",
-               "kernel_row.cuh", "kernels.h", "k_generic.cu", "k_tma_bf16.cu", "k_tma_f32.cu",
+               "kernel_row.cuh", "kernel_full.cuh", "kernels.h", "k_generic.cu", "k_tma_bf16.cu", "k_tma_f32.cu",
                "k_tma_bf16_prod.cu", "k_tma_f32_prod.cu", "k_tma_bf16_any_s.cu",
-               "k_tma_f32_any_s.cu", "k_row_bf16.cu", "k_row_f32.cu")
+               "k_tma_f32_any_s.cu", "k_row_bf16.cu", "k_row_f32.cu", "k_full_bf16.cu",
+               "k_full_f32.cu")
 N_SETS = 4          # resident input sets rotated between steps (4 x 394 MB, each > L2)
 DIST_MIN_S = 1.0    # the per-step distribution loop runs at least this long
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "fuse_verify_B64_K7_V128256_bf16_traffic.txt")

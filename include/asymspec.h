@@ -31,8 +31,9 @@
  *    library never frees or retains them.  Logit tensors are [B, K+1, V]
  *    row-major in the dtype given (fp32, or bf16 as 16-bit words).  Any
  *    element-aligned pointer works.  Rows on 16-byte boundaries take the fast
- *    path; so do, for the step without per-row outputs, rows of at least
- *    16384 entries off them, if a, b and t lie at the same offset from one.
+ *    path; so do (but for the row tokens alone, or another delta source) rows
+ *    of at least 16384 entries off them, if a, b and t lie at the same offset
+ *    from one.
  *  - All work is enqueued on `stream` (a cudaStream_t; NULL = legacy default
  *    stream) and is asynchronous: results are valid once the stream has
  *    completed.  Calls on different streams are independent and may run
@@ -142,11 +143,13 @@ typedef struct {
 /* Kernels (asymspec_launch_opts.kernel, asymspec_launch_info.kernel). */
 #define ASYMSPEC_KERNEL_GENERIC 1  /* one cluster per row; any element-aligned input */
 #define ASYMSPEC_KERNEL_TMA 2      /* one cluster per row, then a decision kernel; rows
-                                      16-byte aligned.  The step without per-row outputs
-                                      and with delta = a - b runs the production row
-                                      kernel (in greedy mode unless this kernel or a test
-                                      hook is asked for; chosen automatically also for rows
-                                      of 16384 entries and more off the boundaries; slices read from HBM, and again from the L2 for
+                                      16-byte aligned.  With delta = a - b the step without
+                                      per-row outputs, and the step that records row
+                                      statistics or log-probabilities, run streaming row
+                                      kernels (greedy and recorded steps unless this kernel
+                                      or a test hook is asked for; chosen automatically also
+                                      for rows of 16384 entries and more off the boundaries;
+                                      slices read from HBM, and again from the L2 for
                                       rows whose decision needs a second pass; C chosen so
                                       that the rows in flight stay within an L2 budget once a
                                       batch fills a wave of clusters of 8); every other

@@ -26,6 +26,7 @@
 #include "kernel_generic.cuh"
 #include "kernel_tma.cuh"
 #include "kernel_row.cuh"
+#include "kernel_full.cuh"
 #include "kernel_draft.cuh"
 #include "kernel_xvocab.cuh"
 #include "kernels.h"
@@ -52,11 +53,13 @@ struct Plan {
   bool vector_path;
   bool row;          // the production row kernel (fuse_verify_row) runs
   bool stoch, edge;  // its mode; its form for rows off the 16-byte boundaries
+  bool full;         // the recording row kernel (fuse_verify_full) instead
   int nt;            // threads per CTA (kRowThreads or kTThreads)
   int grid_y;        // the row kernel's grid is (C (K+1), B): grid_y = B (1 otherwise)
 };
 
-const void* row_kernel(int dtype, bool stoch, bool edge) {
+const void* row_kernel(int dtype, bool stoch, bool edge, bool full) {
+  if (full) return dtype == ASYMSPEC_FP32 ? full_kernel_f32(stoch, edge) : full_kernel_bf16(stoch, edge);
   return dtype == ASYMSPEC_FP32 ? row_kernel_f32(stoch, edge) : row_kernel_bf16(stoch, edge);
 }
 
@@ -150,7 +153,8 @@ DeviceShape device_shape() {
 cudaError_t prepare_kernel(const void* fn, int device);
 cudaError_t active_clusters(const void* fn, const Plan& pl, int device, int* out);
 
-bool plan_row(int V, int dtype, bool stoch, bool edge, int forced_C, long long rows, Plan* pl) {
+bool plan_row(int V, int dtype, bool stoch, bool edge, bool full, int forced_C, long long rows,
+              Plan* pl) {
   const int elt = elt_size(dtype);
   const int VE = 16 / elt;
   // (a row off the 16-byte boundaries may touch one vector more than it fills)
@@ -159,17 +163,21 @@ bool plan_row(int V, int dtype, bool stoch, bool edge, int forced_C, long long r
   auto fits = [&](int C) {
     return width(C) / VE <= static_cast<long long>(kWalkRounds) * kRowThreads;
   };
+  auto smem = [&](int C) {
+    // the warps' rings follow the fixed state and the pushed records
+    return (full ? full_shared_bytes(C) : row_shared_bytes(C)) + kRingBytes;
+  };
   int C = 0;
   if (forced_C) {
     if (fits(forced_C)) C = forced_C;
   } else {
     const DeviceShape dev = device_shape();
-    const long long slots = static_cast<long long>(dev.sms) * kRowMinBlocks;
+    const long long slots = static_cast<long long>(dev.sms) * (full ? kFullMinBlocks : kRowMinBlocks);
     const double row_bytes = 3.0 * V * elt;
     if (rows * 8 < slots) {
       if (fits(8)) C = 8;
     } else {
-      const void* fn = row_kernel(dtype, stoch, edge);
+      const void* fn = row_kernel(dtype, stoch, edge, full);
       const bool query = dev.ok && prepare_kernel(fn, dev.device) == cudaSuccess;
       for (int c : kRowClusters) {
         if (!fits(c)) continue;
@@ -177,7 +185,7 @@ bool plan_row(int V, int dtype, bool stoch, bool edge, int forced_C, long long r
         long long resident = slots / c;
         Plan q = *pl;
         q.C = c;
-        q.smem = row_shared_bytes(c) + kRingBytes;
+        q.smem = smem(c);
         q.nt = kRowThreads;
         q.kernel = ASYMSPEC_KERNEL_TMA;
         q.grid_y = 1;
@@ -198,12 +206,13 @@ bool plan_row(int V, int dtype, bool stoch, bool edge, int forced_C, long long r
   if (!C) return false;
   pl->C = C;
   pl->W = static_cast<int>(width(C));
-  pl->sh_off = row_shared_bytes(C);  // the warps' rings follow the fixed state
-  pl->smem = row_shared_bytes(C) + kRingBytes;
+  pl->smem = smem(C);
+  pl->sh_off = pl->smem - kRingBytes;
   pl->group_stride = kGroupsMax;
   pl->nt = kRowThreads;
   pl->stoch = stoch;
   pl->edge = edge;
+  pl->full = full;
   return true;
 }
 
@@ -241,13 +250,16 @@ TmaLayout tma_layout(int B, int K, int C, int group_stride = kGroupsMax) {
   return L;
 }
 
-// What the streaming row kernel could take of a call: its mode if it is a
-// production program (no per-row outputs, delta = a - b).
-enum RowProgram { kRowNone, kRowGreedy, kRowStochastic };
+// What the streaming row kernels could take of a call: delta = a - b, and no
+// per-row outputs (fuse_verify_row) or all of what they need (fuse_verify_full);
+// the row tokens alone stay with the staged kernel.
+struct RowProgram {
+  bool ok, stoch, full;
+};
 
-RowProgram row_program(const asymspec_gate_params& gp) {
-  if ((gp.flags & ASYMSPEC_FLAG_DELTA_MASK) != ASYMSPEC_DELTA_AB) return kRowNone;
-  return gp.mode == ASYMSPEC_MODE_STOCHASTIC ? kRowStochastic : kRowGreedy;
+RowProgram row_program(const asymspec_gate_params& gp, bool full, bool tokens) {
+  return {(gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB && (full || !tokens),
+          gp.mode == ASYMSPEC_MODE_STOCHASTIC, full};
 }
 
 // Rows off the 16-byte boundaries stream too: the generic kernel reads them
@@ -278,15 +290,16 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
   if (ws_bytes < cluster_ws_bytes(B, K)) return ASYMSPEC_ERR_WORKSPACE;
   bool ok = false;
   // (its grid is (C (K+1), B): B up to 65535)
-  // Greedy steps stream too: 114 us of staged kernel at B=64, K=7, V=128256
-  // bf16 against 65 us streaming.  The staged kernel's copy waits are what
-  // the test hook shortens, so a call that sets it, or asks for
-  // ASYMSPEC_KERNEL_TMA in greedy mode, keeps the staged kernel.
-  const bool stoch = prog == kRowStochastic;
+  // Greedy and recorded steps stream too (B=64, K=7, V=128256 bf16 greedy:
+  // 114 us of staged kernel against 65 us; B=8, K=5, V=151936 bf16 greedy with
+  // every row recorded: 48 us a step against 28).  The staged kernel's copy waits are
+  // what the test hook shortens, so such calls that set it, or ask for
+  // ASYMSPEC_KERNEL_TMA, keep the staged kernel.
   const bool edge = align == kRowsShifted && V >= kEdgeMinV && !forced_kernel;
-  const bool streams = stoch || (prog == kRowGreedy && !forced_kernel && !(opts && opts->test_flags));
+  const bool streams = prog.ok && ((prog.stoch && !prog.full) ||
+                                   (!forced_kernel && !(opts && opts->test_flags)));
   if (forced_kernel != ASYMSPEC_KERNEL_GENERIC && (vec_ok || edge) && streams && B <= 65535 &&
-      plan_row(V, dtype, stoch, edge, forced_C, pl->rows, pl)) {
+      plan_row(V, dtype, prog.stoch, edge, prog.full, forced_C, pl->rows, pl)) {
     if (ws_bytes >= tma_layout(B, K, pl->C).total) {
       pl->kernel = ASYMSPEC_KERNEL_TMA;
       pl->VE = 16 / elt;
@@ -326,13 +339,16 @@ using KernelFn = const void*;  // a __global__ function taking KParams (or SPara
 
 // sel: the TMA kernel's program set (tma_program_set; 0 = run-time dispatch)
 KernelFn pick_kernel(const Plan& pl, int dtype, bool stoch, int sel = 0) {
-  if (pl.row) return row_kernel(dtype, pl.stoch, pl.edge);
+  if (pl.row) return row_kernel(dtype, pl.stoch, pl.edge, pl.full);
   if (pl.kernel == ASYMSPEC_KERNEL_TMA)
     return dtype == ASYMSPEC_FP32 ? tma_kernel_f32(stoch, sel) : tma_kernel_bf16(stoch, sel);
   return generic_kernel(dtype, pl.vector_path, stoch);
 }
 
 KernelFn pick_decide(const Plan& pl, int dtype, bool stoch) {
+  if (pl.row && pl.full)
+    return dtype == ASYMSPEC_FP32 ? decide_full_f32(stoch, pl.edge)
+                                  : decide_full_bf16(stoch, pl.edge);
   if (pl.row)
     return dtype == ASYMSPEC_FP32 ? decide_blocks_f32(stoch, pl.edge)
                                   : decide_blocks_bf16(stoch, pl.edge);
@@ -597,7 +613,7 @@ int asymspec_plan(int B, int K, int V, int dtype, const asymspec_gate_params* ga
   const bool vec_ok = (static_cast<long long>(V) * elt_size(dtype)) % 16 == 0;
   Plan pl = {};
   st = make_plan(B, K, V, dtype, opts, vec_ok ? kRowsAligned : kRowsShifted,
-                 asymspec_workspace_bytes(B, K, V), row_program(gp), &pl);
+                 asymspec_workspace_bytes(B, K, V), row_program(gp, false, false), &pl);
   if (st) return st;
   out->cluster_size = pl.C;
   out->block_threads = pl.kernel == ASYMSPEC_KERNEL_GENERIC ? kThreads : pl.nt;
@@ -664,9 +680,8 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
       : (static_cast<long long>(V) * elt) % 16 == 0 && !offset(logits_full) ? kRowsAligned
                                                                             : kRowsShifted;
   Plan pl = {};
-  const bool per_row_out = out_row_stats || out_fused_logprobs || out_row_tokens;
   st = make_plan(B, K, V, dtype, opts, align, workspace_bytes,
-                 per_row_out ? kRowNone : row_program(gp), &pl);
+                 row_program(gp, out_row_stats || out_fused_logprobs, out_row_tokens), &pl);
   if (st) return st;
 
   KParams P;
@@ -709,6 +724,7 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   P.group_mass = nullptr;
   P.tma_threads = pl.nt;
   P.head0 = static_cast<int>(offset(logits_full) / elt);
+  P.lp_vec = P.head0 == 0 && aligned(out_fused_logprobs, 16) ? 1 : 0;
   // the chunk waits of the TMA kernel: bounded, or (test hook) giving up at once
   P.copy_wait_ns =
       (opts && (opts->test_flags & ASYMSPEC_TEST_COPY_GIVE_UP)) ? 0ull : kCopyTimeoutNs;
@@ -742,15 +758,18 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   if (e != cudaSuccess) return cuda_fail(e);
   if (pl.kernel == ASYMSPEC_KERNEL_TMA) {
     // the rows' decisions and Algorithm 1's scan: one CTA per batch element
-    // as a programmatic dependent launch: its launch overlaps the row
+    // (per row after the recording kernel), as a programmatic dependent launch: its launch overlaps the row
     // kernel's last CTAs, and it waits (griddepcontrol.wait) for that kernel
-    const int threads = pl.row ? kDrawThreads : 32 * std::min(K + 1, kDecideThreads / 32);
+    const int threads = !pl.row              ? 32 * std::min(K + 1, kDecideThreads / 32)
+                        : pl.full && !stoch ? 32
+                                            : kDrawThreads;
     const KernelFn dfn = pick_decide(pl, dtype, stoch);
     cudaLaunchConfig_t dcfg = {};
     cudaLaunchAttribute dattr[1];
     dattr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     dattr[0].val.programmaticStreamSerializationAllowed = 1;
-    dcfg.gridDim = dim3(static_cast<unsigned>(B));
+    dcfg.gridDim = pl.row && pl.full ? dim3(static_cast<unsigned>(K + 1), static_cast<unsigned>(B))
+                                     : dim3(static_cast<unsigned>(B));
     dcfg.blockDim = dim3(threads);
     dcfg.stream = static_cast<cudaStream_t>(stream);
     dcfg.attrs = dattr;

@@ -274,8 +274,9 @@ __device__ __forceinline__ void ring_prologue(uint4* ring, const Streams<T>& g, 
     cp_async_commit();
   }
 }
-// use(r, va, vb, vt) for every step r of vectors [v0, v1) the lane has a
-// vector in, after the prologue.  kRing whole steps at a time with constant
+// use(r, va, vb, vt, whole) for every step r of vectors [v0, v1) the lane has
+// a vector in, after the prologue (whole: std::true_type where every lane of
+// the warp has one).  kRing whole steps at a time with constant
 // slots and no branch: step r + kRing goes into the slot step r was just used
 // from (its values were consumed by instructions this thread has already
 // issued, so the copy cannot overwrite unread data).  At most kRing steps
@@ -293,7 +294,7 @@ __device__ __forceinline__ void ring_steps(uint4* ring, const Streams<T>& g, int
     for (int u = 0; u < kRing; ++u) {
       cp_async_wait<kRing - 1>();
       ring_read<T, AB, TT>(ring, u, va, vb, vt);
-      use(r + u, va, vb, vt);
+      use(r + u, va, vb, vt, std::true_type{});
       ring_issue<T, AB, TT>(ring, u, g, static_cast<size_t>(r + u + kRing) * 32 * VE,
                             i0 + 32 * (r + u + kRing) < v1);
       cp_async_commit();
@@ -303,7 +304,7 @@ __device__ __forceinline__ void ring_steps(uint4* ring, const Streams<T>& g, int
 #pragma unroll 1
   for (int u = 0; i0 + 32 * r < v1; ++r, ++u) {
     ring_read<T, AB, TT>(ring, u, va, vb, vt);
-    use(r, va, vb, vt);
+    use(r, va, vb, vt, std::false_type{});
   }
   __syncwarp();
 }
@@ -328,8 +329,42 @@ constexpr float kEdgeNone = -1e30f;
 struct EdgeVals {
   bool own;           // the warp owns a partial vector
   bool head, tail;    // this lane holds an element of vector 0 / of the last vector
+  int at;             // its index in the row (-1: none)
   float a, b, t;
 };
+
+// The edge elements of the warp whose block is vectors [b0, b1) of the slice
+// that starts at vector s0; ab: a and b are wanted too.
+template <typename T, bool EDGE>
+__device__ __forceinline__ EdgeVals load_edges(const KParams& P, const RowCut<T, EDGE>& cut,
+                                               unsigned row, int s0, int b0, int b1, bool ab) {
+  constexpr int VE = 16 / static_cast<int>(sizeof(T));
+  EdgeVals ed{false, false, false, -1, kEdgeNone, kEdgeNone, kEdgeNone};
+  if constexpr (EDGE) {
+    const int lane = static_cast<int>(threadIdx.x & 31);
+    const bool h = cut.in0 > 0 && s0 == 0 && b0 == 0 && b1 > 0;
+    const bool l = cut.in1 < cut.nvec && b1 > b0 && s0 + b1 == cut.nvec;
+    ed.own = h || l;
+    if (h && lane < VE && lane >= cut.head) {
+      ed.head = true;
+      ed.at = lane - cut.head;
+    }
+    const int el = cut.in1 * VE - cut.head + lane - 8;
+    if (l && lane >= 8 && lane < 8 + VE && el < P.V) {
+      ed.tail = true;
+      ed.at = el;
+    }
+    if (ed.at >= 0) {
+      const size_t o = static_cast<size_t>(row) * P.V + ed.at;
+      ed.t = elem_ldg(static_cast<const T*>(P.t) + o);
+      if (ab) {
+        ed.a = elem_ldg(static_cast<const T*>(P.a) + o);
+        ed.b = elem_ldg(static_cast<const T*>(P.b) + o);
+      }
+    }
+  }
+  return ed;
+}
 
 // Larger of three with NaN winning (non-finite scores are flagged at the end).
 __device__ __forceinline__ float max3_nan(float a, float b, float c) {
@@ -405,7 +440,7 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
   float best = -INFINITY;
   int rbest = -1;
   ring_steps<T, AB, true>(ring, g, v0, v1, [&](int r, const RawVec<T>& va, const RawVec<T>& vb,
-                                               const RawVec<T>& vt) {
+                                               const RawVec<T>& vt, auto) {
     f2 sc[NP];  // the argmax's scores
 #pragma unroll
     for (int h = 0; h < NP; ++h) {
@@ -564,7 +599,7 @@ __device__ __forceinline__ void row_pass2(uint4* ring, const Streams<T>& g, int 
     if (DIV == kDivKl) jacc = kl_pair(amb, p, k, jacc);
   };
   ring_steps<T, true, RES>(ring, g, v0, v1, [&](int, const RawVec<T>& va, const RawVec<T>& vb,
-                                                const RawVec<T>& vt) {
+                                                const RawVec<T>& vt, auto) {
 #pragma unroll
     for (int h = 0; h < NP; ++h) take(va.pair(h), vb.pair(h), RES ? vt.pair(h) : 0ull);
   });
@@ -578,7 +613,8 @@ __device__ __forceinline__ void row_pass2(uint4* ring, const Streams<T>& g, int 
 
 // The warp's JSD sum term by term, for a block where e = q/p overflowed
 // (finite logits with b - a above about 88): p and q from their own
-// exponents, an entry of no mass contributing nothing.
+// exponents, an entry of no mass contributing nothing.  NaN where a or b is
+// not finite.
 template <typename T, bool EDGE>
 __device__ __noinline__ float row_jsd_wide(const Streams<T>& g, int v0, int v1, float A2, float B2,
                                            const EdgeVals& ed) {
@@ -591,6 +627,7 @@ __device__ __noinline__ float row_jsd_wide(const Streams<T>& g, int v0, int v1, 
     const float lm = lg2(p + q) - 1.f;  // log2 of the mean
     if (p > 0.f) j += p * (la - lm);
     if (q > 0.f) j += q * (lb - lm);
+    j = fmaf(a - b, 0.f, j);
   };
   const int lane = static_cast<int>(threadIdx.x & 31);
   for (int i = v0 + lane, q = 0; i < v1; i += 32, ++q) {
@@ -759,30 +796,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
   cluster_arrive_relaxed();
   if (only_t) ring_prologue<T, false, true>(ring, g, i0, v1);
   else ring_prologue<T, true, true>(ring, g, i0, v1);
-  EdgeVals ed{false, false, false, kEdgeNone, kEdgeNone, kEdgeNone};
-  if constexpr (EDGE) {
-    const bool h = cut.in0 > 0 && s0 == 0 && b0 == 0 && b1 > 0;
-    const bool l = cut.in1 < cut.nvec && b1 > b0 && s0 + b1 == cut.nvec;
-    ed.own = h || l;
-    int at = -1;  // this lane's element of the row
-    if (h && lane < VE && lane >= cut.head) {
-      ed.head = true;
-      at = lane - cut.head;
-    }
-    const int el = cut.in1 * VE - cut.head + lane - 8;
-    if (l && lane >= 8 && lane < 8 + VE && el < P.V) {
-      ed.tail = true;
-      at = el;
-    }
-    if (at >= 0) {
-      const size_t o = static_cast<size_t>(row32) * P.V + at;
-      ed.t = elem_ldg(static_cast<const T*>(P.t) + o);
-      if (!only_t) {
-        ed.a = elem_ldg(static_cast<const T*>(P.a) + o);
-        ed.b = elem_ldg(static_cast<const T*>(P.b) + o);
-      }
-    }
-  }
+  const EdgeVals ed = load_edges<T, EDGE>(P, cut, row32, s0, b0, b1, !only_t);
   // every CTA's barrier is initialised before any push (the CTAs of a
   // cluster start together; this wait overlaps the first loads)
   cluster_wait();
@@ -967,15 +981,16 @@ struct Draw {
   int last, use_r;
 };
 
-// By one warp: the records of the row's C x NW groups (lane l holds groups
-// 4l .. 4l + 3, in index order).
+// By one warp: the draw's group from the masses of the row's C x NW groups
+// (lane l holds groups 4l .. 4l + 3, in index order); total: the row's mass.
 __device__ __forceinline__ Draw select_group(const float (&Rm)[4], const float (&Qm)[4], bool bonus,
-                                             float u_last) {
+                                             float u_last, float& total) {
   const int lane = threadIdx.x & 31;
   const float Rl = (Rm[0] + Rm[1]) + (Rm[2] + Rm[3]), Ql = (Qm[0] + Qm[1]) + (Qm[2] + Qm[3]);
   const float R_all = warp_sum(Rl), Q_all = warp_sum(Ql);
   const bool r_ok = !bonus && R_all > 0.f;
-  const float ml = r_ok ? Rl : Ql, total = r_ok ? R_all : Q_all;
+  const float ml = r_ok ? Rl : Ql;
+  total = r_ok ? R_all : Q_all;
   const float tau = u_last * total;
   Draw d{-1, 0.f, 0, r_ok ? 1 : 0};
   float incl = ml;
@@ -1019,21 +1034,161 @@ __device__ __forceinline__ Draw select_group(const float (&Rm)[4], const float (
   return d;
 }
 
-template <typename T, bool STOCH, bool EDGE>
-__global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
+// A row's statistics and its warps' records, as decided from (one warp; one
+// trip to the L2): the divergence sum (every lane) and the masses of groups
+// 4 lane .. 4 lane + 3.
+struct RowRecords {
+  RowStat st;
+  float j, R[4], Q[4];
+};
+
+__device__ __forceinline__ RowRecords load_records(const KParams& P, long long row) {
+  RowRecords x;
+  const int lane = threadIdx.x & 31, ng = P.C * (kRowThreads / 32);
+  const float4* src = reinterpret_cast<const float4*>(static_cast<const RowStat*>(P.row_stat) + row);
+  float4* dst = reinterpret_cast<float4*>(&x.st);
+  dst[0] = __ldcg(src);
+  dst[1] = __ldcg(src + 1);
+  dst[2] = __ldcg(src + 2);
+  float j = 0.f;
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const int q = 4 * lane + h;
+    x.R[h] = x.Q[h] = 0.f;
+    if (q < ng) {  // record q: warp q % NW of CTA q / NW
+      const float4 v = __ldcg(
+          reinterpret_cast<const float4*>(P.pass2_rec + (static_cast<size_t>(row) * ng + q) * 8));
+      j += v.x;
+      x.R[h] = v.y;
+      x.Q[h] = v.z;
+    }
+  }
+  x.j = warp_sum(j);
+  return x;
+}
+
+// The divergence from its sum: 2 JSD, or KL, in bits.
+__device__ __forceinline__ float divergence_nats(const KParams& P, float j) {
+  return P.divergence == ASYMSPEC_DIV_JSD ? 0.5f * kLn2 * j
+         : P.divergence == ASYMSPEC_DIV_KL ? kLn2 * j
+                                           : 0.f;
+}
+
+// The draw inside a group by the whole CTA (kDrawThreads threads): the
+// smallest index whose cumulative mass exceeds the target, the masses formed
+// exactly as the row kernel forms them; every thread returns it (-1: no
+// mass).
+template <typename T, bool EDGE>
+__device__ __forceinline__ int block_draw(const KParams& P, long long row, const Draw& dr, float A2,
+                                          float S2) {
   constexpr int VE = 16 / static_cast<int>(sizeof(T));
   constexpr int NP = VE / 2;
   constexpr int NW = kRowThreads / 32;
+  __shared__ float wtot[kDrawWarps];
+  __shared__ int wfirst[kDrawWarps], wlast[kDrawWarps], s_pick;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const RowCut<T, EDGE> cut(P, row);
+  const int Wv = P.W / VE, rk = max(dr.g, 0) / NW, w = max(dr.g, 0) - rk * NW;
+  const int s0 = rk * Wv, nv = max(0, min(Wv, cut.nvec - s0)), bw = row_block_vectors(nv, NW);
+  const int g0 = s0 + min(nv, w * bw), g1 = s0 + min(nv, w * bw + bw);
+  const int i = g0 + static_cast<int>(threadIdx.x);  // this thread's vector of the row
+  const ResConst kc = res_const(P.beta, A2, 0.f, S2);
+  f2 m2[NP];
+#pragma unroll
+  for (int h = 0; h < NP; ++h) m2[h] = 0ull;
+  if (dr.g >= 0 && i < g1) {
+    const T *pa = cut.base(P.a), *pb = cut.base(P.b), *pt = cut.base(P.t);
+    const size_t o = static_cast<size_t>(i) * VE;
+    f2 xa[NP], xb[NP], xt[NP];
+    if (!EDGE || (i >= cut.in0 && i < cut.in1)) {
+      const RawVec<T> va = raw_ldg(pa + o), vb = raw_ldg(pb + o), vt = raw_ldg(pt + o);
+#pragma unroll
+      for (int h = 0; h < NP; ++h) {
+        xa[h] = va.pair(h);
+        xb[h] = vb.pair(h);
+        xt[h] = vt.pair(h);
+      }
+    } else {
+      const int el0 = i * VE - cut.head;
+#pragma unroll
+      for (int h = 0; h < NP; ++h) {
+        float x[6];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const bool in = el0 + 2 * h + q >= 0 && el0 + 2 * h + q < P.V;
+          const size_t oe = o + 2 * h + q;
+          x[q] = in ? elem_ldg(pa + oe) : kEdgeNone;
+          x[2 + q] = in ? elem_ldg(pb + oe) : kEdgeNone;
+          x[4 + q] = in ? elem_ldg(pt + oe) : kEdgeNone;
+        }
+        xa[h] = pk(x[0], x[1]);
+        xb[h] = pk(x[2], x[3]);
+        xt[h] = pk(x[4], x[5]);
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
+      f2 amb, p, qf, r;
+      res_pair(xa[h], xb[h], xt[h], kc, amb, p, qf, r);
+      m2[h] = dr.use_r ? r : qf;
+    }
+  }
+  const float mv = vsum(m2);
+  float vin = mv;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const float x = __shfl_up_sync(0xffffffffu, vin, off);
+    if (lane >= off) vin += x;
+  }
+  if (lane == 31) wtot[warp] = vin;
+  __syncthreads();
+  float before = 0.f;
+  for (int q = 0; q < warp; ++q) before += wtot[q];
+  const unsigned over = __ballot_sync(0xffffffffu, !dr.last && mv > 0.f && before + vin > dr.rem);
+  const unsigned pos = __ballot_sync(0xffffffffu, mv > 0.f);
+  if (lane == 0) {
+    wfirst[warp] = over ? __ffs(over) - 1 : -1;
+    wlast[warp] = pos ? 31 - __clz(pos) : -1;
+  }
+  if (threadIdx.x == 0) s_pick = -1;
+  __syncthreads();
+  int first = -1, last = -1;
+#pragma unroll
+  for (int q = kDrawWarps - 1; q >= 0; --q) {
+    if (wfirst[q] >= 0) first = 32 * q + wfirst[q];
+    if (last < 0 && wlast[q] >= 0) last = 32 * q + wlast[q];
+  }
+  const int pick = first >= 0 ? first : last;  // the thread that holds the vector
+  if (static_cast<int>(threadIdx.x) == pick) {
+    const float rem = fmaxf(dr.rem - (before + (vin - mv)), 0.f);
+    float cum = 0.f;
+    int el = -1, lastel = -1;
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float m = q == 0 ? lo_of(m2[h]) : hi_of(m2[h]);
+        if (m > 0.f) lastel = 2 * h + q;
+        cum += m;
+        if (first >= 0 && el < 0 && cum > rem) el = 2 * h + q;
+      }
+    }
+    if (el < 0) el = lastel;
+    s_pick = i * VE + el - cut.head;
+  }
+  __syncthreads();
+  return s_pick;
+}
+
+template <typename T, bool STOCH, bool EDGE>
+__global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
   __shared__ int4 srec[kDecideSmemRows];   // the element's records (accept, candidate, error bits)
   __shared__ Draw sdraw[kDecideSmemRows];  // where each row's draw lies
   __shared__ float slse[kDecideSmemRows][2];  // LSE(a), LSE(s) of each row
-  __shared__ int s_len, s_err, s_next;
-  __shared__ float wtot[kDrawWarps];
-  __shared__ int wfirst[kDrawWarps], wlast[kDrawWarps];
+  __shared__ int s_len, s_err;
   const int bi = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int K = P.K, K1 = K + 1, C = P.C, ng = C * NW;
-  const bool jsd = P.divergence == ASYMSPEC_DIV_JSD;
+  const int K = P.K, K1 = K + 1;
   const bool in_smem = K1 <= kDecideSmemRows;
   // the kernel inputs of this warp's first row, loaded before the wait
   RowInputs pre{-1, 0.f, 0.f, 0.f, RowScalars{0.f, 0.f, 0.f}};
@@ -1046,38 +1201,14 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
   auto decide = [&](int k, const RowInputs& din, Draw& dr, float (&lse_as)[2]) {
     const long long row = static_cast<long long>(bi) * K1 + k;
     const bool bonus = k == K;
-    RowStat st;
-    {
-      const float4* src =
-          reinterpret_cast<const float4*>(static_cast<const RowStat*>(P.row_stat) + row);
-      float4* dst = reinterpret_cast<float4*>(&st);
-      dst[0] = __ldcg(src);
-      dst[1] = __ldcg(src + 1);
-      dst[2] = __ldcg(src + 2);
-    }
-    float j = 0.f, Rm[4], Qm[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int q = 4 * lane + h;
-      Rm[h] = Qm[h] = 0.f;
-      if (q < ng) {  // record q: warp q % NW of CTA q / NW
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(
-            P.pass2_rec + (static_cast<size_t>(row) * ng + q) * 8));
-        j += x.x;
-        Rm[h] = x.y;
-        Qm[h] = x.z;
-      }
-    }
+    const RowRecords x = load_records(P, row);
+    const RowStat& st = x.st;
     RowResult rr;
     rr.lse_a = bonus ? NAN : st.lse[0];
     rr.lse_b = bonus ? NAN : st.lse[1];
     rr.lse_t = st.lse[2];
     rr.lse_s = st.lse[3];
-    rr.D = 0.f;
-    if (!bonus && st.path == kPathFull) {
-      const float js = warp_sum(j);
-      rr.D = jsd ? 0.5f * kLn2 * js : kLn2 * js;  // 2 JSD, or KL, in bits
-    }
+    rr.D = !bonus && st.path == kPathFull ? divergence_nats(P, x.j) : 0.f;
     rr.is = st.is;
     rr.it = st.it;
     rr.sample = 0;  // the stop row's draw follows the scan
@@ -1089,7 +1220,10 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
     if (!bonus && st.path == kPathReject) rec.x = 0;
     lse_as[0] = st.lse[0];
     lse_as[1] = st.lse[3];
-    if (STOCH && (bonus || rec.x == 0)) dr = select_group(Rm, Qm, bonus, din.sc.u_last);
+    if (STOCH && (bonus || rec.x == 0)) {
+      float total;
+      dr = select_group(x.R, x.Q, bonus, din.sc.u_last, total);
+    }
     return rec;
   };
   for (int k = warp; k < K1; k += nw) {
@@ -1139,7 +1273,6 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
     if (lane == 0) {
       s_len = len;
       s_err = any_err;
-      s_next = next;
       if (!STOCH || any_err) {
         P.out_len[bi] = any_err ? -1 : len;
         P.out_next[bi] = any_err ? -1 : next;
@@ -1149,109 +1282,15 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
   if constexpr (STOCH) {
     __syncthreads();
     if (s_err) return;
-    // the draw at row len: the smallest index whose cumulative mass exceeds
-    // the target, the masses formed exactly as the row kernel forms them
-    const int len = s_len;
-    const Draw dr = sdraw[in_smem ? len : 0];
-    const float A2 = slse[in_smem ? len : 0][0] * kLog2e, S2 = slse[in_smem ? len : 0][1] * kLog2e;
-    const long long row = static_cast<long long>(bi) * K1 + len;
-    const RowCut<T, EDGE> cut(P, row);
-    const int Wv = P.W / VE, rk = max(dr.g, 0) / NW, w = max(dr.g, 0) - rk * NW;
-    const int s0 = rk * Wv, nv = max(0, min(Wv, cut.nvec - s0)), bw = row_block_vectors(nv, NW);
-    const int g0 = s0 + min(nv, w * bw), g1 = s0 + min(nv, w * bw + bw);
-    const int i = g0 + static_cast<int>(threadIdx.x);  // this thread's vector of the row
-    const ResConst kc = res_const(P.beta, A2, 0.f, S2);
-    f2 m2[NP];
-#pragma unroll
-    for (int h = 0; h < NP; ++h) m2[h] = 0ull;
-    if (dr.g >= 0 && i < g1) {
-      const T *pa = cut.base(P.a), *pb = cut.base(P.b), *pt = cut.base(P.t);
-      const size_t o = static_cast<size_t>(i) * VE;
-      f2 xa[NP], xb[NP], xt[NP];
-      if (!EDGE || (i >= cut.in0 && i < cut.in1)) {
-        const RawVec<T> va = raw_ldg(pa + o), vb = raw_ldg(pb + o), vt = raw_ldg(pt + o);
-#pragma unroll
-        for (int h = 0; h < NP; ++h) {
-          xa[h] = va.pair(h);
-          xb[h] = vb.pair(h);
-          xt[h] = vt.pair(h);
-        }
-      } else {
-        const int el0 = i * VE - cut.head;
-#pragma unroll
-        for (int h = 0; h < NP; ++h) {
-          float x[6];
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const bool in = el0 + 2 * h + q >= 0 && el0 + 2 * h + q < P.V;
-            const size_t oe = o + 2 * h + q;
-            x[q] = in ? elem_ldg(pa + oe) : kEdgeNone;
-            x[2 + q] = in ? elem_ldg(pb + oe) : kEdgeNone;
-            x[4 + q] = in ? elem_ldg(pt + oe) : kEdgeNone;
-          }
-          xa[h] = pk(x[0], x[1]);
-          xb[h] = pk(x[2], x[3]);
-          xt[h] = pk(x[4], x[5]);
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < NP; ++h) {
-        f2 amb, p, qf, r;
-        res_pair(xa[h], xb[h], xt[h], kc, amb, p, qf, r);
-        m2[h] = dr.use_r ? r : qf;
-      }
+    const int len = s_len, at = in_smem ? len : 0;
+    const int tok = block_draw<T, EDGE>(P, static_cast<long long>(bi) * K1 + len, sdraw[at],
+                                        slse[at][0] * kLog2e, slse[at][1] * kLog2e);
+    if (threadIdx.x == 0) {
+      // (no mass at all: non-finite data that the normalisers did not show)
+      P.out_len[bi] = tok < 0 ? -1 : len;
+      P.out_next[bi] = tok;
+      if (tok < 0 && P.err_word) atomicOr(P.err_word, ASYMSPEC_DATA_NONFINITE);
     }
-    const float mv = vsum(m2);
-    float vin = mv;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const float x = __shfl_up_sync(0xffffffffu, vin, off);
-      if (lane >= off) vin += x;
-    }
-    if (lane == 31) wtot[warp] = vin;
-    __syncthreads();
-    float before = 0.f;
-    for (int q = 0; q < warp; ++q) before += wtot[q];
-    const unsigned over = __ballot_sync(0xffffffffu, !dr.last && mv > 0.f && before + vin > dr.rem);
-    const unsigned pos = __ballot_sync(0xffffffffu, mv > 0.f);
-    if (lane == 0) {
-      wfirst[warp] = over ? __ffs(over) - 1 : -1;
-      wlast[warp] = pos ? 31 - __clz(pos) : -1;
-    }
-    __syncthreads();
-    int first = -1, last = -1;
-#pragma unroll
-    for (int q = kDrawWarps - 1; q >= 0; --q) {
-      if (wfirst[q] >= 0) first = 32 * q + wfirst[q];
-      if (last < 0 && wlast[q] >= 0) last = 32 * q + wlast[q];
-    }
-    const int pick = first >= 0 ? first : last;  // the thread that holds the vector
-    if (pick < 0) {
-      // no mass at all (non-finite data that the normalisers did not show)
-      if (threadIdx.x == 0) {
-        P.out_len[bi] = -1;
-        P.out_next[bi] = -1;
-        if (P.err_word) atomicOr(P.err_word, ASYMSPEC_DATA_NONFINITE);
-      }
-      return;
-    }
-    if (static_cast<int>(threadIdx.x) != pick) return;
-    const float rem = fmaxf(dr.rem - (before + (vin - mv)), 0.f);
-    float cum = 0.f;
-    int el = -1, lastel = -1;
-#pragma unroll
-    for (int h = 0; h < NP; ++h) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float m = q == 0 ? lo_of(m2[h]) : hi_of(m2[h]);
-        if (m > 0.f) lastel = 2 * h + q;
-        cum += m;
-        if (first >= 0 && el < 0 && cum > rem) el = 2 * h + q;
-      }
-    }
-    if (el < 0) el = lastel;
-    P.out_len[bi] = len;
-    P.out_next[bi] = i * VE + el - cut.head;
   }
 }
 

@@ -22,6 +22,12 @@ const void* row_kernel_bf16(bool stoch, bool edge);
 const void* row_kernel_f32(bool stoch, bool edge);
 const void* decide_blocks_bf16(bool stoch, bool edge);
 const void* decide_blocks_f32(bool stoch, bool edge);
+// fuse_verify_full<T, STOCH, EDGE>, every row recorded, and
+// decide_full<T, STOCH, EDGE>, launched after it (k_full_bf16.cu, k_full_f32.cu)
+const void* full_kernel_bf16(bool stoch, bool edge);
+const void* full_kernel_f32(bool stoch, bool edge);
+const void* decide_full_bf16(bool stoch, bool edge);
+const void* decide_full_f32(bool stoch, bool edge);
 // decide_rows<T, STOCH>, launched after fuse_verify_tma (k_tma_*.cu)
 const void* decide_kernel_bf16(bool stoch);
 const void* decide_kernel_f32(bool stoch);

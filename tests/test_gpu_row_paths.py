@@ -11,7 +11,7 @@ import pytest
 
 from paper_2608_26004_gb300 import asymspec as A
 from paper_2608_26004_gb300 import synth
-from tests._parity import check_decisions, device_inputs, run_gpu, run_oracle
+from tests._parity import D_TOL, check_decisions, compare, device_inputs, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -206,3 +206,27 @@ def test_rows_at_different_offsets_take_the_generic_kernel(torch):
     g = run_gpu(batch, torch, mode=STOCH, full="row", inputs=x)
     o = run_oracle(batch, mode=STOCH, logprobs=False)
     check_decisions(batch, np.arange(2), g["accept_len"], g["next_token"], o, STOCH)
+
+
+# ---------------------------------------------------------------- every row recorded
+
+@pytest.mark.parametrize("mode", [GREEDY, STOCH])
+@pytest.mark.parametrize("B,K,V,dtype,offset,cluster", [
+    (3, 2, 40000, synth.BF16, 0, 0), (2, 2, 12288, synth.FP32, 0, 1), (2, 3, 8200, synth.BF16, 0, 16),
+    (3, 2, 16391, synth.BF16, 0, 0), (2, 2, 16391, synth.BF16, 3, 5), (2, 2, 16385, synth.FP32, 1, 0),
+    (2, 1, 16, synth.BF16, 0, 0), (1, 70, 1024, synth.FP32, 0, 0)])
+def test_recorded_rows(torch, B, K, V, dtype, offset, cluster, mode):
+    # statistics, tokens and log-probabilities of every row, on and off the
+    # 16-byte boundaries (16-byte and single stores of the log-probabilities)
+    batch, _ = batch_over_the_threshold(B, K, V, dtype, 60 + V, torch, mode)
+    x = shifted(device_inputs(batch, torch), offset, torch)
+    for div in (A.DIV_JSD, A.DIV_KL, A.DIV_LAMBDA):
+        g = run_gpu(batch, torch, mode=mode, divergence=div, inputs=x, cluster_size=cluster)
+        o = run_oracle(batch, mode=mode, divergence=div)
+        assert int(g["error_word"][0]) == 0
+        # KL is not bounded by ln 2: its error grows with it, each p carrying the
+        # rounding of its exponent (2^-23 |log2 p|, up to about 30 of them: 2.5e-6
+        # of the sum in relative terms)
+        compare(batch, g, o, mode=mode, check_stats=div != A.DIV_KL)
+        err = np.abs(g["row_stats"][..., 4] - o.D)
+        assert np.all(err <= D_TOL * np.maximum(1.0, np.abs(o.D)))
