@@ -339,7 +339,7 @@ def draft_timing(torch, A, sets, B, K, V, mode, dev, steps):
 
 
 def xvocab_timing(torch, A, synth, mode, dev, steps, timed, stream):
-    """The cross-family step (asymspec_fuse_verify_xvocab: gather, step,
+    """The cross-family step (asymspec_fuse_verify_xvocab: map check, row kernel,
     emission) on the bench workload's batch shape over a Qwen3-sized drafter
     vocabulary, a Llama-3-sized verifier vocabulary and the paper's shared set,
     and its gather (asymspec_xvocab_gather) alone; CUDA events on the stream."""
@@ -402,7 +402,7 @@ def xvocab_timing(torch, A, synth, mode, dev, steps, timed, stream):
     return {"mode": "stochastic" if mode == A.MODE_STOCHASTIC else "greedy",
             "B": B, "K": K, "S": S, "V_d": V_d, "V_v": V_v, "rows": rows,
             "ms_per_step": ms_step, "rows_per_s": rows / (ms_step * 1e-3),
-            "launches_per_step": 6,
+            "launches_per_step": 4,
             "gather": {"kernel": "xvocab_gather", "us_per_launch": ms_gather * 1e3,
                        "algorithmic_bytes_per_launch": touched + written,
                        "algorithmic_bytes": "the 32-byte sectors of a, b and t holding paired "

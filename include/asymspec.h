@@ -400,9 +400,11 @@ int asymspec_draft_sample(const void* logits, int rows, int V, int dtype, int mo
  *   ASYMSPEC_ERR_WORKSPACE (scratch unaligned or too small),
  *   ASYMSPEC_ERR_TOO_LARGE (rows above 524,280).
  *
- * asymspec_fuse_verify_xvocab: map check, gather, step and emission, up to
- *   seven launches on `stream` (the gather's four, the step's one or two,
- *   the emission): logits_full, logits_comp
+ * asymspec_fuse_verify_xvocab: the step on the restricted rows.  Where a
+ *   restricted row fits the shared memory of four CTAs (and delta = a - b), the
+ *   map check, a row kernel on the rows as they are and a decision kernel: four
+ *   launches on `stream`; otherwise map check, gather, step and emission, up to
+ *   seven (the gather's four, the step's one or two, the emission): logits_full, logits_comp
  *   [B, K+1, V_d]; logits_ver [B, K+1, V_v]; draft_index [B, K] int32 pair indices; draft_probs,
  *   uniforms, gate_params as for asymspec_fuse_verify (draft_probs[b][k] is
  *   the drafter's probability of pair draft_index[b][k] under the restricted
@@ -414,10 +416,8 @@ int asymspec_draft_sample(const void* logits, int rows, int V, int dtype, int mo
  *   (asymspec_workspace_reset; every call that completes leaves it fit for
  *   the next); out_error_word as for asymspec_fuse_verify_ex.  A map entry
  *   outside its vocabulary or a token in two pairs makes every batch element
- *   a data error (accept_len = next_token = -1, ASYMSPEC_DATA_BAD_MAP).  The
- *   restricted rows are laid out with a stride of S entries, so the fast
- *   step kernel runs when S * element size is a multiple of 16 and the
- *   generic one otherwise.  Status codes are those of
+ *   a data error (accept_len = next_token = -1, ASYMSPEC_DATA_BAD_MAP).
+ *   Status codes are those of
  *   asymspec_fuse_verify_ex and asymspec_xvocab_gather; a pair index outside
  *   [0, S) is the data error ASYMSPEC_DATA_BAD_TOKEN of that element.
  */

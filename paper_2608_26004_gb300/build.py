@@ -19,10 +19,11 @@ CSRC = os.path.join(HERE, "csrc")
 CUDA_SRC = [os.path.join(CSRC, f) for f in (
     "asymspec.cu", "k_generic.cu", "k_tma_bf16.cu", "k_tma_f32.cu", "k_tma_bf16_prod.cu",
     "k_tma_f32_prod.cu", "k_tma_bf16_any_s.cu", "k_tma_f32_any_s.cu", "k_row_bf16.cu",
-    "k_row_f32.cu", "k_full_bf16.cu", "k_full_f32.cu", "k_draft.cu", "k_xvocab.cu")]
+    "k_row_f32.cu", "k_full_bf16.cu", "k_full_f32.cu", "k_xrow_bf16.cu",
+    "k_xrow_f32.cu", "k_draft.cu", "k_xvocab.cu")]
 CUDA_HEADERS = [os.path.join(CSRC, f) for f in (
     "device_common.cuh", "kernel_generic.cuh", "kernel_tma.cuh", "kernel_row.cuh",
-    "kernel_full.cuh", "kernel_draft.cuh", "kernel_xvocab.cuh", "kernels.h")]
+    "kernel_full.cuh", "kernel_xrow.cuh", "kernel_draft.cuh", "kernel_xvocab.cuh", "kernels.h")]
 CUDA_LIB = os.path.join(HERE, "libasymspec.so")
 GENCODE = "arch=compute_103a,code=sm_103a"
 

@@ -29,6 +29,7 @@
 #include "kernel_full.cuh"
 #include "kernel_draft.cuh"
 #include "kernel_xvocab.cuh"
+#include "kernel_xrow.cuh"
 #include "kernels.h"
 
 namespace {
@@ -470,6 +471,28 @@ int check_opts(const asymspec_launch_opts* opts) {
   return ASYMSPEC_OK;
 }
 
+// The call's inputs and gate.
+void set_inputs(KParams* P, const void* a, const void* b, const void* t, const int32_t* tokens,
+                const float* probs, const float* unif, int B, int K, int V,
+                const asymspec_gate_params& gp) {
+  P->a = a;
+  P->b = b;
+  P->t = t;
+  P->tokens = tokens;
+  P->dprobs = probs;
+  P->unif = unif;
+  P->B = B;
+  P->K = K;
+  P->V = V;
+  P->gamma = gp.gamma;
+  P->beta = gp.beta;
+  P->lambda = gp.lambda;
+  P->ln_gamma = logf(gp.gamma);
+  P->divergence = gp.divergence;
+  P->delta_src = gp.flags & ASYMSPEC_FLAG_DELTA_MASK;
+  P->fuse_bonus = gp.fuse_bonus ? 1 : 0;
+}
+
 // The caller's timing events around the fused row kernel (asymspec_launch_opts).
 cudaError_t record_timing(const asymspec_launch_opts* opts, bool begin, cudaStream_t s) {
   if (!opts || !opts->timing_begin) return cudaSuccess;
@@ -684,26 +707,12 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
                  row_program(gp, out_row_stats || out_fused_logprobs, out_row_tokens), &pl);
   if (st) return st;
 
-  KParams P;
-  P.a = logits_full;
-  P.b = logits_comp;
-  P.t = logits_ver;
-  P.tokens = draft_tokens;
-  P.dprobs = draft_probs;
-  P.unif = uniforms;
-  P.B = B;
-  P.K = K;
-  P.V = V;
+  KParams P = {};
+  set_inputs(&P, logits_full, logits_comp, logits_ver, draft_tokens, draft_probs, uniforms, B, K, V,
+             gp);
   P.C = pl.C;
   P.W = pl.W;
   P.sh_off = pl.sh_off;
-  P.gamma = gp.gamma;
-  P.beta = gp.beta;
-  P.lambda = gp.lambda;
-  P.ln_gamma = logf(gp.gamma);
-  P.divergence = gp.divergence;
-  P.delta_src = gp.flags & ASYMSPEC_FLAG_DELTA_MASK;
-  P.fuse_bonus = gp.fuse_bonus ? 1 : 0;
   P.need_lse_s = (stoch || out_fused_logprobs || out_row_stats) ? 1 : 0;
   P.need_pass2 = (stoch || out_fused_logprobs || gp.divergence == ASYMSPEC_DIV_JSD ||
                   gp.divergence == ASYMSPEC_DIV_KL)
@@ -719,9 +728,6 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   P.logprobs = out_fused_logprobs;
   P.err_word = out_error_word;
   P.recs = static_cast<int4*>(workspace);
-  P.row_stat = nullptr;
-  P.pass2_rec = nullptr;
-  P.group_mass = nullptr;
   P.tma_threads = pl.nt;
   P.head0 = static_cast<int>(offset(logits_full) / elt);
   P.lp_vec = P.head0 == 0 && aligned(out_fused_logprobs, 16) ? 1 : 0;
@@ -1037,6 +1043,124 @@ XLayout xvocab_layout(int B, int K, int S, int V_d, int V_v, int dtype) {
   return L;
 }
 
+// The map check: inverse maps built with atomicCAS, the map-error word.
+cudaError_t map_check(const int32_t* md, const int32_t* mv, int S, int Vd, int Vv, char* scratch,
+                      uint32_t* ew, cudaStream_t st) {
+  const XScratch XL = xvocab_scratch_layout(Vd, Vv);
+  int* inv_d = reinterpret_cast<int*>(scratch + XL.inv_d);
+  int* inv_v = reinterpret_cast<int*>(scratch + XL.inv_v);
+  unsigned* merr = reinterpret_cast<unsigned*>(scratch + XL.err);
+  void* fargs[] = {&inv_d, &Vd, &inv_v, &Vv, &merr};
+  const int vmax = std::max(Vd, Vv);
+  const cudaError_t e =
+      cudaLaunchKernel(xvocab_inv_fill_ptr(), dim3((vmax + 255) / 256), dim3(256), fargs, 0, st);
+  if (e != cudaSuccess) return e;
+  void* bargs[] = {&md, &mv, &S, &inv_d, &Vd, &inv_v, &Vv, &merr, &ew};
+  return cudaLaunchKernel(xvocab_inv_build_ptr(), dim3((S + 255) / 256), dim3(256), bargs, 0, st);
+}
+
+// The one-kernel cross-family step: clusters of C <= 4 CTAs (128 warp records
+// a row), one CTA an SM, each with its share of a restricted row of t in
+// shared memory.  C by the time of rows C CTAs in waves of one an SM: a CTA's
+// is about 0.4 + 0.6 / C of a whole row's (every CTA reads the whole row of t
+// and the inverse map), and 1.4 times that when its share leaves the L1 less
+// than about 60 KB.  Measured (us a step; C = 1, 2, 3, 4):
+//   512 rows, S=109568 bf16: 215 187 247 285    160 rows, S=93793 bf16: 79 83 94 100
+//   320 rows, S=105622 fp32: - 185 144 157       80 rows: - 94 60 67
+//    20 rows, S=93793 bf16: 41 29 26 25           5 rows, S=64000: 27 21 20 19
+// False: the gather and the step on its output run instead.
+bool plan_xrow(int S, int elt, long long rows, int sms, Plan* pl) {
+  double best = 0.0;
+  for (int C = 1; C <= 4; ++C) {
+    const int W = static_cast<int>(round_up_ll((static_cast<long long>(S) + C - 1) / C, kXVec));
+    const long long smem = xrow_shared_bytes(C) + static_cast<long long>(W) * elt;
+    // (a warp's block of pairs is at most what the decision kernel's draw takes)
+    if (smem > kMaxSmem ||
+        row_block_vectors(W / kXVec, kXRowWarps) > kDrawThreads)
+      continue;
+    const double waves = static_cast<double>((rows * C + sms - 1) / sms);
+    const double cost = waves * (0.4 + 0.6 / C) * (smem > 160 * 1024 ? 1.4 : 1.0);
+    if (best > 0.0 && cost >= best) continue;
+    best = cost;
+    pl->C = C;
+    pl->W = W;
+    pl->sh_off = xrow_shared_bytes(C);
+    pl->smem = static_cast<int>(smem);
+    pl->nt = kXRowThreads;
+  }
+  return best > 0.0;
+}
+
+// The map check, the row kernel (a programmatic dependent: it fetches its
+// rows into the L2 meanwhile) and the decision kernel.  step_ws: a workspace
+// of the step for S entries.
+int run_xrow(const Plan& pl, const void* a, const void* b, int V_d, const void* t, int V_v,
+             const int32_t* map_d, const int32_t* map_v, int S, const int32_t* draft_index,
+             const float* probs, const float* unif, int B, int K, int dtype,
+             const asymspec_gate_params& gp, int32_t* out_len, int32_t* out_next, int32_t* out_index,
+             char* scratch, char* step_ws, uint32_t* err_word, cudaStream_t st) {
+  int device = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return cuda_fail(e);
+  const bool stoch = gp.mode == ASYMSPEC_MODE_STOCHASTIC;
+  const KernelFn fn =
+      dtype == ASYMSPEC_FP32 ? xrow_kernel_f32(stoch) : xrow_kernel_bf16(stoch);
+  const KernelFn dfn = dtype == ASYMSPEC_FP32 ? decide_xrow_f32(stoch) : decide_xrow_bf16(stoch);
+  e = prepare_kernel(fn, device);
+  if (e != cudaSuccess) return cuda_fail(e);
+  const TmaLayout TL = tma_layout(B, K, 16);
+  const XScratch XL = xvocab_scratch_layout(V_d, V_v);
+  KParams P = {};
+  set_inputs(&P, a, b, t, draft_index, probs, unif, B, K, S, gp);
+  P.C = pl.C;
+  P.W = pl.W;
+  P.sh_off = pl.sh_off;
+  P.rows = static_cast<long long>(B) * (K + 1);
+  P.out_len = out_len;
+  P.out_next = out_next;
+  P.err_word = err_word;
+  P.recs = reinterpret_cast<int4*>(step_ws);
+  P.row_stat = step_ws + TL.stat;
+  P.pass2_rec = reinterpret_cast<float*>(step_ws + TL.p2rec);
+  XRowParams X;
+  X.map_d = map_d;
+  X.map_v = map_v;
+  X.inv_v = reinterpret_cast<const int*>(scratch + XL.inv_v);
+  X.map_err = reinterpret_cast<const unsigned*>(scratch + XL.err);
+  X.out_index = out_index;
+  X.V_d = V_d;
+  X.V_v = V_v;
+  X.t_vec = aligned(t, 16) && (static_cast<size_t>(V_v) * elt_size(dtype)) % 16 == 0 ? 1 : 0;
+  X.idx2 = aligned(map_d, 8) ? 1 : 0;
+  e = map_check(map_d, map_v, S, V_d, V_v, scratch, err_word, st);
+  if (e != cudaSuccess) return cuda_fail(e);
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = pl.C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(pl.C * (K + 1)), static_cast<unsigned>(B));
+  cfg.blockDim = dim3(pl.nt);
+  cfg.dynamicSmemBytes = pl.smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  void* args[] = {&P, &X};
+  e = cudaLaunchKernelExC(&cfg, fn, args);
+  if (e != cudaSuccess) return cuda_fail(e);
+  cudaLaunchConfig_t dcfg = {};
+  dcfg.gridDim = dim3(static_cast<unsigned>(B));
+  dcfg.blockDim = dim3(kDrawThreads);
+  dcfg.stream = st;
+  dcfg.attrs = attr + 1;
+  dcfg.numAttrs = 1;
+  e = cudaLaunchKernelExC(&dcfg, dfn, args);
+  return e == cudaSuccess ? ASYMSPEC_OK : cuda_fail(e);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1075,21 +1199,7 @@ int asymspec_xvocab_gather(const void* logits_full, const void* logits_comp, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
   if (scratch) {
-    // the map check: inverse maps built with atomicCAS, the map-error word
-    char* base = static_cast<char*>(scratch);
-    int* inv_d = reinterpret_cast<int*>(base + XL.inv_d);
-    int* inv_v = reinterpret_cast<int*>(base + XL.inv_v);
-    unsigned* merr = reinterpret_cast<unsigned*>(base + XL.err);
-    int Vd = V_d, Vv = V_v, S_ = S;
-    void* fargs[] = {&inv_d, &Vd, &inv_v, &Vv, &merr};
-    const int vmax = std::max(V_d, V_v);
-    e = cudaLaunchKernel(xvocab_inv_fill_ptr(), dim3((vmax + 255) / 256), dim3(256), fargs, 0, st);
-    if (e != cudaSuccess) return cuda_fail(e);
-    const int32_t* md = map_d;
-    const int32_t* mv = map_v;
-    uint32_t* ew = out_error_word;
-    void* bargs[] = {&md, &mv, &S_, &inv_d, &Vd, &inv_v, &Vv, &merr, &ew};
-    e = cudaLaunchKernel(xvocab_inv_build_ptr(), dim3((S + 255) / 256), dim3(256), bargs, 0, st);
+    e = map_check(map_d, map_v, S, V_d, V_v, static_cast<char*>(scratch), out_error_word, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   XGatherParams P;
@@ -1177,11 +1287,27 @@ int asymspec_fuse_verify_xvocab(const void* logits_full, const void* logits_comp
   if (!workspace || !aligned(workspace, 256) || workspace_bytes < L.total)
     return ASYMSPEC_ERR_WORKSPACE;
   char* base = static_cast<char*>(workspace);
+  int32_t* idx = out_next_index ? out_next_index : reinterpret_cast<int32_t*>(base + L.idx);
+  const long long rows = static_cast<long long>(B) * (K + 1);
+  const int elt = elt_size(dtype);
+  Plan pl = {};
+  if ((gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB && B <= 65535 && rows <= 8LL * 65535 &&
+      plan_xrow(S, elt, rows, device_shape().sms, &pl)) {
+    if (!logits_full || !logits_comp || !logits_ver || !map_d || !map_v) return ASYMSPEC_ERR_INVALID_ARG;
+    if (!aligned(logits_full, elt) || !aligned(logits_comp, elt) || !aligned(logits_ver, elt) ||
+        !aligned(map_d, 4) || !aligned(map_v, 4) || (out_error_word && !aligned(out_error_word, 4)) ||
+        !aligned(draft_index, 4) || (draft_probs && !aligned(draft_probs, 4)) ||
+        (uniforms && !aligned(uniforms, 4)))
+      return ASYMSPEC_ERR_MISALIGNED;
+    return run_xrow(pl, logits_full, logits_comp, V_d, logits_ver, V_v, map_d, map_v, S,
+                    draft_index, draft_probs, uniforms, B, K, dtype, gp, out_accept_len,
+                    out_next_token, idx, base + L.scratch, base + L.step, out_error_word,
+                    static_cast<cudaStream_t>(stream));
+  }
   st = asymspec_xvocab_gather(logits_full, logits_comp, V_d, logits_ver, V_v, map_d, map_v, S,
                               B * (K + 1), dtype, base + L.ga, base + L.gb, base + L.gt,
                               out_error_word, base + L.scratch, L.scratch_bytes, stream);
   if (st) return st;
-  int32_t* idx = out_next_index ? out_next_index : reinterpret_cast<int32_t*>(base + L.idx);
   st = asymspec_fuse_verify_ex(base + L.ga, base + L.gb, base + L.gt, draft_index, draft_probs,
                                uniforms, B, K, S, dtype, &gp, out_accept_len, idx,
                                base + L.step, L.step_bytes, nullptr, nullptr, nullptr,

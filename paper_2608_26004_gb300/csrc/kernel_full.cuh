@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(STOCH ? kDrawThreads : 32) decide_full(const K
   rr.sample = -1;
   rr.mass = NAN;
   if (warp == 0) {
-    const RowRecords x = load_records(P, row);
+    const RowRecords x = load_records(P, row, P.C * (kRowThreads / 32));
     rr.lse_a = x.st.lse[0];
     rr.lse_b = x.st.lse[1];
     rr.lse_t = x.st.lse[2];

@@ -1042,9 +1042,9 @@ struct RowRecords {
   float j, R[4], Q[4];
 };
 
-__device__ __forceinline__ RowRecords load_records(const KParams& P, long long row) {
+__device__ __forceinline__ RowRecords load_records(const KParams& P, long long row, int ng) {
   RowRecords x;
-  const int lane = threadIdx.x & 31, ng = P.C * (kRowThreads / 32);
+  const int lane = threadIdx.x & 31;
   const float4* src = reinterpret_cast<const float4*>(static_cast<const RowStat*>(P.row_stat) + row);
   float4* dst = reinterpret_cast<float4*>(&x.st);
   dst[0] = __ldcg(src);
@@ -1055,7 +1055,7 @@ __device__ __forceinline__ RowRecords load_records(const KParams& P, long long r
   for (int h = 0; h < 4; ++h) {
     const int q = 4 * lane + h;
     x.R[h] = x.Q[h] = 0.f;
-    if (q < ng) {  // record q: warp q % NW of CTA q / NW
+    if (q < ng) {  // record q: warp q % NW of CTA q / NW (ng = C NW)
       const float4 v = __ldcg(
           reinterpret_cast<const float4*>(P.pass2_rec + (static_cast<size_t>(row) * ng + q) * 8));
       j += v.x;
@@ -1074,19 +1074,71 @@ __device__ __forceinline__ float divergence_nats(const KParams& P, float j) {
                                            : 0.f;
 }
 
-// The draw inside a group by the whole CTA (kDrawThreads threads): the
-// smallest index whose cumulative mass exceeds the target, the masses formed
-// exactly as the row kernel forms them; every thread returns it (-1: no
-// mass).
+// The draw inside a group by the whole CTA (kDrawThreads threads), thread i
+// holding the masses of the group's entries [2 NP i, 2 NP (i + 1)): the
+// smallest entry whose cumulative mass exceeds the target; every thread
+// returns it (-1: no mass).
+template <int NP>
+__device__ __forceinline__ int block_pick(const f2 (&m2)[NP], const Draw& dr) {
+  __shared__ float wtot[kDrawWarps];
+  __shared__ int wfirst[kDrawWarps], wlast[kDrawWarps], s_pick;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float mv = vsum(m2);
+  float vin = mv;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const float x = __shfl_up_sync(0xffffffffu, vin, off);
+    if (lane >= off) vin += x;
+  }
+  if (lane == 31) wtot[warp] = vin;
+  __syncthreads();
+  float before = 0.f;
+  for (int q = 0; q < warp; ++q) before += wtot[q];
+  const unsigned over = __ballot_sync(0xffffffffu, !dr.last && mv > 0.f && before + vin > dr.rem);
+  const unsigned pos = __ballot_sync(0xffffffffu, mv > 0.f);
+  if (lane == 0) {
+    wfirst[warp] = over ? __ffs(over) - 1 : -1;
+    wlast[warp] = pos ? 31 - __clz(pos) : -1;
+  }
+  if (threadIdx.x == 0) s_pick = -1;
+  __syncthreads();
+  int first = -1, last = -1;
+#pragma unroll
+  for (int q = kDrawWarps - 1; q >= 0; --q) {
+    if (wfirst[q] >= 0) first = 32 * q + wfirst[q];
+    if (last < 0 && wlast[q] >= 0) last = 32 * q + wlast[q];
+  }
+  const int pick = first >= 0 ? first : last;  // the thread that holds the entry
+  if (static_cast<int>(threadIdx.x) == pick) {
+    const float rem = fmaxf(dr.rem - (before + (vin - mv)), 0.f);
+    float cum = 0.f;
+    int el = -1, lastel = -1;
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float m = q == 0 ? lo_of(m2[h]) : hi_of(m2[h]);
+        if (m > 0.f) lastel = 2 * h + q;
+        cum += m;
+        if (first >= 0 && el < 0 && cum > rem) el = 2 * h + q;
+      }
+    }
+    if (el < 0) el = lastel;
+    s_pick = pick * 2 * NP + el;
+  }
+  __syncthreads();
+  return s_pick;
+}
+
+// The row's draw: the masses of the group's vectors, one per thread, formed
+// exactly as the row kernel forms them; every thread returns the token (-1:
+// no mass).
 template <typename T, bool EDGE>
 __device__ __forceinline__ int block_draw(const KParams& P, long long row, const Draw& dr, float A2,
                                           float S2) {
   constexpr int VE = 16 / static_cast<int>(sizeof(T));
   constexpr int NP = VE / 2;
   constexpr int NW = kRowThreads / 32;
-  __shared__ float wtot[kDrawWarps];
-  __shared__ int wfirst[kDrawWarps], wlast[kDrawWarps], s_pick;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const RowCut<T, EDGE> cut(P, row);
   const int Wv = P.W / VE, rk = max(dr.g, 0) / NW, w = max(dr.g, 0) - rk * NW;
   const int s0 = rk * Wv, nv = max(0, min(Wv, cut.nvec - s0)), bw = row_block_vectors(nv, NW);
@@ -1133,55 +1185,17 @@ __device__ __forceinline__ int block_draw(const KParams& P, long long row, const
       m2[h] = dr.use_r ? r : qf;
     }
   }
-  const float mv = vsum(m2);
-  float vin = mv;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const float x = __shfl_up_sync(0xffffffffu, vin, off);
-    if (lane >= off) vin += x;
-  }
-  if (lane == 31) wtot[warp] = vin;
-  __syncthreads();
-  float before = 0.f;
-  for (int q = 0; q < warp; ++q) before += wtot[q];
-  const unsigned over = __ballot_sync(0xffffffffu, !dr.last && mv > 0.f && before + vin > dr.rem);
-  const unsigned pos = __ballot_sync(0xffffffffu, mv > 0.f);
-  if (lane == 0) {
-    wfirst[warp] = over ? __ffs(over) - 1 : -1;
-    wlast[warp] = pos ? 31 - __clz(pos) : -1;
-  }
-  if (threadIdx.x == 0) s_pick = -1;
-  __syncthreads();
-  int first = -1, last = -1;
-#pragma unroll
-  for (int q = kDrawWarps - 1; q >= 0; --q) {
-    if (wfirst[q] >= 0) first = 32 * q + wfirst[q];
-    if (last < 0 && wlast[q] >= 0) last = 32 * q + wlast[q];
-  }
-  const int pick = first >= 0 ? first : last;  // the thread that holds the vector
-  if (static_cast<int>(threadIdx.x) == pick) {
-    const float rem = fmaxf(dr.rem - (before + (vin - mv)), 0.f);
-    float cum = 0.f;
-    int el = -1, lastel = -1;
-#pragma unroll
-    for (int h = 0; h < NP; ++h) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float m = q == 0 ? lo_of(m2[h]) : hi_of(m2[h]);
-        if (m > 0.f) lastel = 2 * h + q;
-        cum += m;
-        if (first >= 0 && el < 0 && cum > rem) el = 2 * h + q;
-      }
-    }
-    if (el < 0) el = lastel;
-    s_pick = i * VE + el - cut.head;
-  }
-  __syncthreads();
-  return s_pick;
+  const int pick = block_pick(m2, dr);
+  return pick < 0 ? -1 : g0 * VE + pick - cut.head;
 }
 
-template <typename T, bool STOCH, bool EDGE>
-__global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
+// One batch element, by one CTA.  Rows: where the rows' inputs lie,
+//   groups(P): warp records per row;  refused(P, bi): the whole call is a data
+//   error (its outputs are written);  inputs(P, bi, k): load_row_inputs;
+//   draw(P, row, dr, A2, S2): block_draw;  emit(P, bi, len, next): the
+//   element's outputs (thread 0; next < 0 on a data error).
+template <bool STOCH, typename Rows>
+__device__ __forceinline__ void decide_element(const KParams& P, const Rows& rows) {
   __shared__ int4 srec[kDecideSmemRows];   // the element's records (accept, candidate, error bits)
   __shared__ Draw sdraw[kDecideSmemRows];  // where each row's draw lies
   __shared__ float slse[kDecideSmemRows][2];  // LSE(a), LSE(s) of each row
@@ -1192,16 +1206,17 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
   const bool in_smem = K1 <= kDecideSmemRows;
   // the kernel inputs of this warp's first row, loaded before the wait
   RowInputs pre{-1, 0.f, 0.f, 0.f, RowScalars{0.f, 0.f, 0.f}};
-  if (warp < K1) pre = load_row_inputs<T, STOCH>(P, bi, warp);
+  if (warp < K1) pre = rows.inputs(P, bi, warp);
   // launched as a programmatic dependent of the row kernel: its CTAs may
   // start early; nothing of the workspace is read before that kernel is done
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (rows.refused(P, bi)) return;
   // Decides row k (one warp).  The group records are loaded with the row's
   // statistics (one trip) and used only where the row left some.
   auto decide = [&](int k, const RowInputs& din, Draw& dr, float (&lse_as)[2]) {
     const long long row = static_cast<long long>(bi) * K1 + k;
     const bool bonus = k == K;
-    const RowRecords x = load_records(P, row);
+    const RowRecords x = load_records(P, row, rows.groups(P));
     const RowStat& st = x.st;
     RowResult rr;
     rr.lse_a = bonus ? NAN : st.lse[0];
@@ -1227,7 +1242,7 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
     return rec;
   };
   for (int k = warp; k < K1; k += nw) {
-    const RowInputs din = (k == warp) ? pre : load_row_inputs<T, STOCH>(P, bi, k);
+    const RowInputs din = (k == warp) ? pre : rows.inputs(P, bi, k);
     Draw dr{-1, 0.f, 0, 0};
     float las[2];
     const int4 rec = decide(k, din, dr, las);
@@ -1263,7 +1278,7 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
     if (STOCH && !in_smem && !any_err) {  // the stop row's group was not kept
       Draw dr{-1, 0.f, 0, 0};
       float las[2];
-      decide(len, load_row_inputs<T, STOCH>(P, bi, len), dr, las);
+      decide(len, rows.inputs(P, bi, len), dr, las);
       if (lane == 0) {
         sdraw[0] = dr;
         slse[0][0] = las[0];
@@ -1273,25 +1288,45 @@ __global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
     if (lane == 0) {
       s_len = len;
       s_err = any_err;
-      if (!STOCH || any_err) {
-        P.out_len[bi] = any_err ? -1 : len;
-        P.out_next[bi] = any_err ? -1 : next;
-      }
+      if (any_err) rows.emit(P, bi, -1, -1);
+      else if (!STOCH) rows.emit(P, bi, len, next);
     }
   }
   if constexpr (STOCH) {
     __syncthreads();
     if (s_err) return;
     const int len = s_len, at = in_smem ? len : 0;
-    const int tok = block_draw<T, EDGE>(P, static_cast<long long>(bi) * K1 + len, sdraw[at],
-                                        slse[at][0] * kLog2e, slse[at][1] * kLog2e);
+    const int tok = rows.draw(P, static_cast<long long>(bi) * K1 + len, sdraw[at],
+                              slse[at][0] * kLog2e, slse[at][1] * kLog2e);
     if (threadIdx.x == 0) {
       // (no mass at all: non-finite data that the normalisers did not show)
-      P.out_len[bi] = tok < 0 ? -1 : len;
-      P.out_next[bi] = tok;
+      rows.emit(P, bi, tok < 0 ? -1 : len, tok);
       if (tok < 0 && P.err_word) atomicOr(P.err_word, ASYMSPEC_DATA_NONFINITE);
     }
   }
+}
+
+// Rows [B, K+1, V] of one vocabulary.
+template <typename T, bool STOCH, bool EDGE>
+struct PlainRows {
+  __device__ __forceinline__ int groups(const KParams& P) const { return P.C * (kRowThreads / 32); }
+  __device__ __forceinline__ bool refused(const KParams&, int) const { return false; }
+  __device__ __forceinline__ RowInputs inputs(const KParams& P, int bi, int k) const {
+    return load_row_inputs<T, STOCH>(P, bi, k);
+  }
+  __device__ __forceinline__ int draw(const KParams& P, long long row, const Draw& dr, float A2,
+                                      float S2) const {
+    return block_draw<T, EDGE>(P, row, dr, A2, S2);
+  }
+  __device__ __forceinline__ void emit(const KParams& P, int bi, int len, int next) const {
+    P.out_len[bi] = len;
+    P.out_next[bi] = next;
+  }
+};
+
+template <typename T, bool STOCH, bool EDGE>
+__global__ void __launch_bounds__(kDrawThreads) decide_blocks(const KParams P) {
+  decide_element<STOCH>(P, PlainRows<T, STOCH, EDGE>{});
 }
 
 }  // namespace asymspec_impl

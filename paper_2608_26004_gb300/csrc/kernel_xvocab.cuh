@@ -57,6 +57,10 @@ struct XGatherParams {
 
 constexpr int kXInvThreads = 512;
 
+// The map check's error word: a token claimed by two pairs; an entry outside
+// its vocabulary (whose logits read as NaN).
+constexpr unsigned kMapTwice = 1u, kMapOutside = 2u;
+
 template <typename T>
 __device__ __forceinline__ T x_nan();
 template <>
@@ -241,20 +245,19 @@ __global__ void __launch_bounds__(256) xvocab_inv_build(const I* __restrict__ ma
                                                         I* __restrict__ inv_v, int V_v,
                                                         unsigned* __restrict__ map_err,
                                                         uint32_t* __restrict__ err_word) {
+  // fuse_verify_xrow, a programmatic dependent, may start fetching its rows;
+  // it waits for this kernel before it uses the maps
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= S) return;
   const I md = map_d[j], mv = map_v[j];
-  bool bad = false;
-  if (static_cast<unsigned>(md) < static_cast<unsigned>(V_d))
-    bad |= atomicCAS(inv_d + md, I(-1), I(j)) != I(-1);
-  else
-    bad = true;
-  if (static_cast<unsigned>(mv) < static_cast<unsigned>(V_v))
-    bad |= atomicCAS(inv_v + mv, I(-1), I(j)) != I(-1);
-  else
-    bad = true;
+  unsigned bad = 0u;
+  if (static_cast<unsigned>(md) >= static_cast<unsigned>(V_d)) bad |= kMapOutside;
+  else if (atomicCAS(inv_d + md, I(-1), I(j)) != I(-1)) bad |= kMapTwice;
+  if (static_cast<unsigned>(mv) >= static_cast<unsigned>(V_v)) bad |= kMapOutside;
+  else if (atomicCAS(inv_v + mv, I(-1), I(j)) != I(-1)) bad |= kMapTwice;
   if (bad) {
-    atomicOr(map_err, 1u);
+    atomicOr(map_err, bad);
     if (err_word) atomicOr(err_word, ASYMSPEC_DATA_BAD_MAP);
   }
 }

@@ -31,6 +31,12 @@ const void* decide_full_f32(bool stoch, bool edge);
 // decide_rows<T, STOCH>, launched after fuse_verify_tma (k_tma_*.cu)
 const void* decide_kernel_bf16(bool stoch);
 const void* decide_kernel_f32(bool stoch);
+// fuse_verify_xrow<T, STOCH> and decide_xrow<T, STOCH>, the cross-family step
+// (k_xrow_bf16.cu, k_xrow_f32.cu)
+const void* xrow_kernel_bf16(bool stoch);
+const void* xrow_kernel_f32(bool stoch);
+const void* decide_xrow_bf16(bool stoch);
+const void* decide_xrow_f32(bool stoch);
 // draft_kernel<T, VE, STOCH>, the drafter's draw (k_draft.cu)
 const void* draft_kernel_ptr(int dtype, bool vector_path, bool stoch);
 // the cross-family vocabulary map (k_xvocab.cu): xvocab_gather<T, WITH_T>,
