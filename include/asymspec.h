@@ -336,13 +336,13 @@ int asymspec_fuse_verify_host(const void* h_logits_full, const void* h_logits_co
  *                                  positive mass.
  * Arguments (device pointers, caller-owned, not retained):
  *   logits      [rows, V] row-major, fp32 or bf16 (dtype), element-aligned;
- *               16-byte aligned with V * element size a multiple of 16 takes
- *               the vector path (same results)
+ *               rows off the 16-byte boundaries cost two partly filled vectors
+ *               (same results)
  *   uniforms    [rows] float32, stochastic mode only
  *   out_tokens  [rows] int32; out_probs [rows] float32
  *   cluster_size  CTAs that share a row (1, 2, 4 or 8; each reads one
  *               contiguous slice of it), or 0 for the library's choice: the
- *               smallest that gives at least 4 CTAs per SM, up to 8, while a
+ *               smallest that gives at least 3 CTAs per SM, up to 8, while a
  *               slice keeps at least 512 vectors.  Results do not depend on it
  *               beyond fp32 rounding of the sums.
  * One kernel launch on `stream` (rows x cluster_size CTAs), no workspace,

@@ -951,17 +951,23 @@ int asymspec_draft_sample(const void* logits, int rows, int V, int dtype, int mo
   if (!aligned(logits, elt) || !aligned(out_tokens, 4) || !aligned(out_probs, 4) ||
       (stoch && !aligned(uniforms, 4)))
     return ASYMSPEC_ERR_MISALIGNED;
-  const bool vec = (static_cast<long long>(V) * elt) % 16 == 0 && aligned(logits, 16);
-  const int VE = vec ? 16 / elt : 1;
-  const int nv = V / VE;
+  const bool edge = (static_cast<long long>(V) * elt) % 16 != 0 || !aligned(logits, 16);
+  const int VE = 16 / elt;
+  // (a row off the 16-byte boundaries may touch one vector more than it fills)
+  const int nv = edge ? (V + 2 * VE - 2) / VE : V / VE;
   int C = cluster_size;
   if (C == 0) {
     int device = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return cuda_fail(e);
+    // the smallest C that gives every SM three CTAs (of the four it holds): a
+    // CTA's start and its reductions cost about 5 us, so more, smaller ones
+    // lose.  Measured (us, bf16 V=128256, sampling; C = 1, 2, 4, 8): 512 rows
+    // 28.5 29.6 30.8 39.0, 256 rows 17.8 17.0 18.7 22.2, 64 rows 13.3 9.2 7.9
+    // 8.0; 128 rows of fp32 V=151936 25.4 19.2 18.8 19.6
     C = 1;
-    while (C < kDMaxCluster && static_cast<long long>(rows) * C < 4LL * sms &&
+    while (C < kDMaxCluster && static_cast<long long>(rows) * C < 3LL * sms &&
            (nv + 2 * C - 1) / (2 * C) >= 512)
       C *= 2;
   }
@@ -972,14 +978,15 @@ int asymspec_draft_sample(const void* logits, int rows, int V, int dtype, int mo
   P.probs = out_probs;
   P.rows = rows;
   P.V = V;
-  P.nv = nv;
+  P.head0 = static_cast<int>(reinterpret_cast<uintptr_t>(logits) % 16) / elt;
   P.W = (nv + C - 1) / C;
   // sampling: one float of group mass per warp and round of a slice
   const size_t smem =
-      stoch ? static_cast<size_t>((P.W + kDThreads - 1) / kDThreads) * kDWarps * sizeof(float) : 0;
-  const void* fn = draft_kernel_ptr(dtype, vec, stoch);
+      kDRingBytes +
+      (stoch ? static_cast<size_t>((P.W + kDThreads - 1) / kDThreads) * kDWarps * sizeof(float) : 0);
+  const void* fn = draft_kernel_ptr(dtype, edge, stoch);
   cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024)
+  if (smem > 47 * 1024)  // (beside the static shared memory: 48 KB without it)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return cuda_fail(e);
   cudaLaunchConfig_t cfg = {};

@@ -4,16 +4,18 @@
 
 namespace asymspec_impl {
 
-template <typename T, int VE>
-const void* draft_pick(bool stoch) {
-  return stoch ? reinterpret_cast<const void*>(&draft_kernel<T, VE, true>)
-               : reinterpret_cast<const void*>(&draft_kernel<T, VE, false>);
+template <typename T>
+const void* draft_pick(bool edge, bool stoch) {
+  if (edge)
+    return stoch ? reinterpret_cast<const void*>(&draft_kernel<T, true, true>)
+                 : reinterpret_cast<const void*>(&draft_kernel<T, true, false>);
+  return stoch ? reinterpret_cast<const void*>(&draft_kernel<T, false, true>)
+               : reinterpret_cast<const void*>(&draft_kernel<T, false, false>);
 }
 
-const void* draft_kernel_ptr(int dtype, bool vector_path, bool stoch) {
-  if (dtype == ASYMSPEC_FP32)
-    return vector_path ? draft_pick<float, 4>(stoch) : draft_pick<float, 1>(stoch);
-  return vector_path ? draft_pick<__nv_bfloat16, 8>(stoch) : draft_pick<__nv_bfloat16, 1>(stoch);
+const void* draft_kernel_ptr(int dtype, bool edge, bool stoch) {
+  return dtype == ASYMSPEC_FP32 ? draft_pick<float>(edge, stoch)
+                                : draft_pick<__nv_bfloat16>(edge, stoch);
 }
 
 }  // namespace asymspec_impl

@@ -6,8 +6,16 @@
 // One cluster of C CTAs (1 <= C <= 8) per row: CTA c owns the vectors
 // [c W, (c + 1) W) of the row (VE elements each; the last slice may be
 // shorter or empty).  In a slice, vector v0 + r kDThreads + t is handled by
-// thread t in round r, kDUnroll rounds' loads issued before any is used (in
-// sampling, the next kDUnroll rounds' too).
+// thread t in round r, read through the thread's own slots of a ring in shared
+// memory (cp.async, kDRing rounds in flight without holding registers).
+// What bounds it: HBM in the middle, and about 7 us of starting a CTA, its
+// reductions and the walk (512 rows of bf16 V=128256: 28.5 us, 19.7 at the
+// copy rate; 29.7 with the next batch of rounds in registers instead of the
+// ring, and one element at a time 80.6 us for V=100003, 28.9 now).
+// EDGE: a row off the 16-byte boundaries is cut at them: vector 0 starts
+// `head` elements before the row and the last may end after it; their
+// elements inside the row are loaded one by one, the others stand as the
+// type's lowest value, which adds no mass and is never drawn.
 // Each CTA reads its slice once from HBM and pushes a summary (reference,
 // mass relative to it, finiteness sum, argmax index) into every CTA of the
 // cluster; after one cluster barrier every CTA combines the C summaries
@@ -39,7 +47,10 @@ namespace asymspec_impl {
 
 constexpr int kDThreads = 256;
 constexpr int kDWarps = kDThreads / 32;
-constexpr int kDUnroll = 4;
+constexpr int kDUnroll = 4;       // rounds used at a time
+constexpr int kDRing = 8;         // rounds in flight
+constexpr int kDRingBytes = kDRing * kDThreads * 16;
+static_assert(kDRing == 2 * kDUnroll, "one batch in use, one behind it in flight");
 constexpr int kDMaxCluster = 8;
 constexpr float kDFinScale = 9.094947017729282e-13f;  // 2^-40
 constexpr float kDGuard = 1.2676506002282294e30f;     // 2^100
@@ -49,8 +60,9 @@ struct DParams {
   const float* unif;   // [rows] (sampling)
   int32_t* tokens;     // [rows]
   float* probs;        // [rows]
-  int rows, V, nv;     // nv = V / VE vectors per row
+  int rows, V;
   int W;               // vectors per CTA slice
+  int head0;           // EDGE: elements from a 16-byte boundary to the logits
 };
 
 // A CTA's summary of its slice.
@@ -90,37 +102,78 @@ __device__ __forceinline__ float dwarp_incl_scan(float v, int lane) {
   return v;
 }
 
-// A vector of VE consecutive logits as loaded: 8 packed bf16, 4 fp32, or one
-// element of either type (widened on load).
-template <typename T, int VE>
+// A vector of consecutive logits as loaded: 8 packed bf16 or 4 fp32.
+template <typename T>
 struct DRaw;
 template <>
-struct DRaw<__nv_bfloat16, 8> {
+struct DRaw<__nv_bfloat16> {
+  static constexpr int VE = 8;
   uint4 q;
 };
 template <>
-struct DRaw<float, 4> {
+struct DRaw<float> {
+  static constexpr int VE = 4;
   float4 q;
 };
-template <typename T>
-struct DRaw<T, 1> {
-  float x;
+
+// One row, cut into vectors: vector v holds elements [v VE - head, (v + 1) VE
+// - head); vectors [in0, in1) lie inside the row whole.
+template <typename T, bool EDGE>
+struct DRow {
+  static constexpr int VE = DRaw<T>::VE;
+  const T* base;  // vector 0 (may precede the row)
+  int V, head, nvec, in0, in1;
+  __device__ __forceinline__ DRow(const DParams& P, int row) {
+    const long long off = static_cast<long long>(row) * P.V;
+    V = P.V;
+    head = EDGE ? static_cast<int>((off + P.head0) & (VE - 1)) : 0;
+    base = static_cast<const T*>(P.logits) + off - head;
+    nvec = (head + V + VE - 1) / VE;
+    in0 = EDGE ? (head != 0) : 0;
+    in1 = EDGE ? (head + V) / VE : nvec;
+  }
+  __device__ __forceinline__ bool whole(int v) const { return !EDGE || (v >= in0 && v < in1); }
+  __device__ __forceinline__ int element(int v, int e) const { return v * VE + e - head; }
+  __device__ __forceinline__ bool inside(int v, int e) const {
+    const int i = element(v, e);
+    return !EDGE || (i >= 0 && i < V);
+  }
 };
 
-__device__ __forceinline__ void dld(const __nv_bfloat16* row, int v, DRaw<__nv_bfloat16, 8>& r) {
-  r.q = __ldg(reinterpret_cast<const uint4*>(row) + v);
+// A partial vector: its elements inside the row, the others the type's lowest.
+template <bool EDGE>
+__device__ __noinline__ DRaw<__nv_bfloat16> dld_edge(const DRow<__nv_bfloat16, EDGE>& r, int v) {
+  const unsigned short* p = reinterpret_cast<const unsigned short*>(r.base) + static_cast<long long>(v) * 8;
+  unsigned w[4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const unsigned lo = r.inside(v, 2 * h) ? __ldg(p + 2 * h) : 0xFF7Fu;
+    const unsigned hi = r.inside(v, 2 * h + 1) ? __ldg(p + 2 * h + 1) : 0xFF7Fu;
+    w[h] = hi << 16 | lo;
+  }
+  return {make_uint4(w[0], w[1], w[2], w[3])};
 }
-__device__ __forceinline__ void dld(const float* row, int v, DRaw<float, 4>& r) {
-  r.q = __ldg(reinterpret_cast<const float4*>(row) + v);
+template <bool EDGE>
+__device__ __noinline__ DRaw<float> dld_edge(const DRow<float, EDGE>& r, int v) {
+  const float* p = r.base + static_cast<long long>(v) * 4;
+  float x[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) x[e] = r.inside(v, e) ? __ldg(p + e) : -3.402823466e38f;
+  return {make_float4(x[0], x[1], x[2], x[3])};
 }
-__device__ __forceinline__ void dld(const float* row, int v, DRaw<float, 1>& r) { r.x = __ldg(row + v); }
-__device__ __forceinline__ void dld(const __nv_bfloat16* row, int v, DRaw<__nv_bfloat16, 1>& r) {
-  r.x = __uint_as_float(static_cast<unsigned>(__ldg(reinterpret_cast<const unsigned short*>(row) + v))
-                        << 16);
+// Vector v of the row.
+template <typename T, bool EDGE>
+__device__ __forceinline__ DRaw<T> dld(const DRow<T, EDGE>& r, int v) {
+  if constexpr (EDGE) {
+    if (!r.whole(v)) return dld_edge(r, v);
+  }
+  DRaw<T> x;
+  x.q = __ldg(reinterpret_cast<const decltype(x.q)*>(r.base) + v);
+  return x;
 }
 
 // The vector widened to fp32.
-__device__ __forceinline__ void dwiden(const DRaw<__nv_bfloat16, 8>& r, float (&x)[8]) {
+__device__ __forceinline__ void dwiden(const DRaw<__nv_bfloat16>& r, float (&x)[8]) {
   const unsigned w[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
 #pragma unroll
   for (int h = 0; h < 4; ++h) {
@@ -128,26 +181,69 @@ __device__ __forceinline__ void dwiden(const DRaw<__nv_bfloat16, 8>& r, float (&
     x[2 * h + 1] = __uint_as_float(w[h] & 0xFFFF0000u);
   }
 }
-__device__ __forceinline__ void dwiden(const DRaw<float, 4>& r, float (&x)[4]) {
+__device__ __forceinline__ void dwiden(const DRaw<float>& r, float (&x)[4]) {
   x[0] = r.q.x;
   x[1] = r.q.y;
   x[2] = r.q.z;
   x[3] = r.q.w;
 }
-template <typename T>
-__device__ __forceinline__ void dwiden(const DRaw<T, 1>& r, float (&x)[1]) {
-  x[0] = r.x;
+
+// The thread's slots of the ring: slot q of round r = q (mod kDRing).  A
+// thread reads back only what it copied itself, so no barrier is needed.
+template <typename T, bool EDGE>
+__device__ __forceinline__ void dring_issue(uint4* ring, const DRow<T, EDGE>& r, int v0, int v1,
+                                            int round) {
+#pragma unroll
+  for (int u = 0; u < kDUnroll; ++u) {
+    const int v = v0 + (round + u) * kDThreads + static_cast<int>(threadIdx.x);
+    uint4* d = ring + ((round + u) % kDRing) * kDThreads + threadIdx.x;
+    if (v < v1) {
+      if (r.whole(v)) {
+        cp_async16(d, r.base + static_cast<long long>(v) * DRaw<T>::VE);
+      } else if constexpr (EDGE) {
+        DRaw<T> x = dld_edge(r, v);
+        *reinterpret_cast<decltype(x.q)*>(d) = x.q;
+      }
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// use(round, raw) for every batch of kDUnroll rounds of the slice, in order
+// (raw[u] of a vector at or past v1 is undefined).
+template <typename T, bool EDGE, typename Use>
+__device__ __forceinline__ void dring_rounds(uint4* ring, const DRow<T, EDGE>& r, int v0, int v1,
+                                             Use&& use) {
+  const int rounds = (v1 - v0 + kDThreads - 1) / kDThreads;
+  for (int q = 0; q < rounds; q += kDUnroll) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    DRaw<T> raw[kDUnroll];
+#pragma unroll
+    for (int u = 0; u < kDUnroll; ++u)
+      raw[u].q = *reinterpret_cast<const decltype(raw[u].q)*>(
+          ring + ((q + u) % kDRing) * kDThreads + threadIdx.x);
+    use(q, raw);
+    // the slots just used take the batch after the next (their values were
+    // consumed by instructions this thread has already issued)
+    dring_issue<T, EDGE>(ring, r, v0, v1, q + kDRing);
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+// The first kDRing rounds (two commit groups).
+template <typename T, bool EDGE>
+__device__ __forceinline__ void dring_start(uint4* ring, const DRow<T, EDGE>& r, int v0, int v1) {
+  dring_issue<T, EDGE>(ring, r, v0, v1, 0);
+  dring_issue<T, EDGE>(ring, r, v0, v1, kDUnroll);
 }
 
 // The finiteness sum f = sum x 2^-40: packed bf16 pairs for bf16 vectors
 // (non-finite values propagate through bf16 arithmetic as through fp32), fp32
 // pairs for fp32 vectors.
-template <typename T, int VE>
+template <typename T>
 struct DFin;
 template <>
-struct DFin<__nv_bfloat16, 8> {
+struct DFin<__nv_bfloat16> {
   unsigned acc = 0u;  // two bf16 partial sums
-  __device__ __forceinline__ void add(const DRaw<__nv_bfloat16, 8>& r) {
+  __device__ __forceinline__ void add(const DRaw<__nv_bfloat16>& r) {
     const unsigned scale = 0x2B802B80u;  // 2^-40 in both halves
     const unsigned w[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
 #pragma unroll
@@ -158,22 +254,15 @@ struct DFin<__nv_bfloat16, 8> {
   }
 };
 template <>
-struct DFin<float, 4> {
+struct DFin<float> {
   f2 acc = 0ull;
-  __device__ __forceinline__ void add(const DRaw<float, 4>& r) {
+  __device__ __forceinline__ void add(const DRaw<float>& r) {
     const f2 scale = pk(kDFinScale, kDFinScale);
     acc = fma2(pk(r.q.x, r.q.y), scale, acc);
     acc = fma2(pk(r.q.z, r.q.w), scale, acc);
   }
   __device__ __forceinline__ float value() const { return hsum2(acc); }
 };
-template <typename T>
-struct DFin<T, 1> {
-  float acc = 0.f;
-  __device__ __forceinline__ void add(const DRaw<T, 1>& r) { acc = fmaf(r.x, kDFinScale, acc); }
-  __device__ __forceinline__ float value() const { return acc; }
-};
-
 template <int VE>
 __device__ __forceinline__ float dvmax(const float (&x)[VE]) {
   float m = x[0];
@@ -185,15 +274,11 @@ __device__ __forceinline__ float dvmax(const float (&x)[VE]) {
 // Sum of 2^(x log2 e + nm2) over a vector (nm2 = -ref log2 e), in fp32 pairs.
 template <int VE>
 __device__ __forceinline__ float dmass(const float (&x)[VE], float nm2) {
-  if constexpr (VE == 1) {
-    return ex2(fmaf(x[0], kLog2e, nm2));
-  } else {
-    const f2 l2 = pk(kLog2e, kLog2e), n2 = pk(nm2, nm2);
-    f2 acc = ex2_2(fma2(pk(x[0], x[1]), l2, n2));
+  const f2 l2 = pk(kLog2e, kLog2e), n2 = pk(nm2, nm2);
+  f2 acc = ex2_2(fma2(pk(x[0], x[1]), l2, n2));
 #pragma unroll
-    for (int h = 1; h < VE / 2; ++h) acc = add2(acc, ex2_2(fma2(pk(x[2 * h], x[2 * h + 1]), l2, n2)));
-    return hsum2(acc);
-  }
+  for (int h = 1; h < VE / 2; ++h) acc = add2(acc, ex2_2(fma2(pk(x[2 * h], x[2 * h + 1]), l2, n2)));
+  return hsum2(acc);
 }
 
 // Warp sums of four per-lane values at once: lane l returns the sum over the
@@ -221,41 +306,38 @@ __device__ __forceinline__ float drescale(float mass, float ref, float R) {
 
 // ---------------------------------------------------------------- greedy slice
 
-template <typename T, int VE>
-__device__ __forceinline__ DSlice slice_greedy(const T* a, int v0, int v1, DShared& sh) {
+template <typename T, bool EDGE>
+__device__ __forceinline__ DSlice slice_greedy(const DRow<T, EDGE>& a, int v0, int v1, uint4* ring,
+                                               DShared& sh) {
+  constexpr int VE = DRaw<T>::VE;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = v1 - v0, full = n / kDThreads, rounds = (n + kDThreads - 1) / kDThreads;
-  float m = -INFINITY, s = 0.f;
-  DFin<T, VE> fin;
+  float m = -INFINITY;
+  float su[kDUnroll] = {};  // one sum per round of a batch: shorter chains of roundings
+  DFin<T> fin;
   int bvec = INT_MAX;
-  auto take = [&](const DRaw<T, VE>& raw, int v) {
+  auto take = [&](const DRaw<T>& raw, int v, float& s) {
     float x[VE];
     dwiden(raw, x);
     const float vm = dvmax(x);
     if (vm > m) {  // strict: the lowest vector of this thread keeps the maximum
-      s *= ex2((m - vm) * kLog2e);
+      const float f = ex2((m - vm) * kLog2e);
+#pragma unroll
+      for (int u = 0; u < kDUnroll; ++u) su[u] *= f;
       m = vm;
       bvec = v;
     }
     s += dmass(x, -m * kLog2e);
     fin.add(raw);
   };
-  int r = 0;
-  for (; r + kDUnroll <= full; r += kDUnroll) {
-    DRaw<T, VE> raw[kDUnroll];
+  dring_start<T, EDGE>(ring, a, v0, v1);
+  dring_rounds<T, EDGE>(ring, a, v0, v1, [&](int r, const DRaw<T> (&raw)[kDUnroll]) {
 #pragma unroll
-    for (int u = 0; u < kDUnroll; ++u) dld(a, v0 + (r + u) * kDThreads + tid, raw[u]);
-#pragma unroll
-    for (int u = 0; u < kDUnroll; ++u) take(raw[u], v0 + (r + u) * kDThreads + tid);
-  }
-  for (; r < rounds; ++r) {
-    const int v = v0 + r * kDThreads + tid;
-    if (v < v1) {
-      DRaw<T, VE> raw;
-      dld(a, v, raw);
-      take(raw, v);
+    for (int u = 0; u < kDUnroll; ++u) {
+      const int v = v0 + (r + u) * kDThreads + tid;
+      if (v < v1) take(raw[u], v, su[u]);
     }
-  }
+  });
+  const float s = (su[0] + su[1]) + (su[2] + su[3]);
   // the CTA maximum, the lowest vector holding it, the sum rescaled to it
   const float w = dwarp_max(m);
   if (lane == 0) sh.red[warp] = w;
@@ -278,13 +360,11 @@ __device__ __forceinline__ DSlice slice_greedy(const T* a, int v0, int v1, DShar
   const int vi = __reduce_min_sync(0xffffffffu, lane < kDWarps ? sh.redi[lane] : INT_MAX);
   int idx = INT_MAX;
   if (warp == 0 && lane == 0 && vi < v1) {
-    DRaw<T, VE> raw;
-    dld(a, vi, raw);
     float x[VE];
-    dwiden(raw, x);
+    dwiden(dld<T, EDGE>(a, vi), x);
 #pragma unroll
     for (int e = VE - 1; e >= 0; --e)
-      if (x[e] == M) idx = vi * VE + e;
+      if (x[e] == M && a.inside(vi, e)) idx = a.element(vi, e);
   }
   out.idx = __shfl_sync(0xffffffffu, idx, 0);
   return out;  // valid in warp 0
@@ -292,78 +372,65 @@ __device__ __forceinline__ DSlice slice_greedy(const T* a, int v0, int v1, DShar
 
 // -------------------------------------------------------------- sampling slice
 
-// Loads of rounds [r, r + kDUnroll) of the slice (vectors past v1 skipped).
-template <typename T, int VE>
-__device__ __forceinline__ void dld_batch(const T* a, int v0, int v1, int r,
-                                          DRaw<T, VE> (&raw)[kDUnroll]) {
-#pragma unroll
-  for (int u = 0; u < kDUnroll; ++u) {
-    const int v = v0 + (r + u) * kDThreads + threadIdx.x;
-    if (v < v1) dld(a, v, raw[u]);
-  }
-}
-
 // Group masses of the slice against the warp reference `ref`: gm[r kDWarps +
 // warp] = the mass of vectors v0 + r kDThreads + warp 32 + [0, 32), summed
-// kDUnroll rounds at a time.  `cur` holds the first batch's loads (rounds
-// 0 .. kDUnroll - 1); each next batch is loaded before the current one is
-// used, so a slice of two batches costs one memory round trip.  Adds the
-// thread's share to tot (and, when FIN, its finiteness sum to fin); returns
-// true if a group's mass reached kDGuard (or is not a number).
-template <typename T, int VE, bool FIN>
-__device__ __forceinline__ bool slice_masses(const T* a, int v0, int v1, float ref, float* gm,
-                                             float& tot, DFin<T, VE>& fin,
-                                             DRaw<T, VE> (&cur)[kDUnroll]) {
+// kDUnroll rounds at a time, read through the ring (the caller started it).
+// Adds the thread's share to tot (and, when FIN, its finiteness sum to fin);
+// returns true if a group's mass reached kDGuard (or is not a number).
+template <typename T, bool EDGE, bool FIN>
+__device__ __forceinline__ bool slice_masses(const DRow<T, EDGE>& a, int v0, int v1, float ref,
+                                             uint4* ring, float* gm, float& tot, DFin<T>& fin) {
   static_assert(kDUnroll == 4, "dwarp_sum4 sums four rounds");
+  constexpr int VE = DRaw<T>::VE;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rounds = (v1 - v0 + kDThreads - 1) / kDThreads;
   const float nm2 = -ref * kLog2e;
   bool over = false;
-  for (int r = 0; r < rounds; r += kDUnroll) {
-    DRaw<T, VE> nxt[kDUnroll];
-    if (r + kDUnroll < rounds) dld_batch<T, VE>(a, v0, v1, r + kDUnroll, nxt);
+  dring_rounds<T, EDGE>(ring, a, v0, v1, [&](int r, const DRaw<T> (&raw)[kDUnroll]) {
     float mv[kDUnroll];
 #pragma unroll
     for (int u = 0; u < kDUnroll; ++u) {
       mv[u] = 0.f;
       if (v0 + (r + u) * kDThreads + tid < v1) {  // implies r + u < rounds
         float x[VE];
-        dwiden(cur[u], x);
+        dwiden(raw[u], x);
         mv[u] = dmass(x, nm2);
-        if (FIN) fin.add(cur[u]);
+        if (FIN) fin.add(raw[u]);
       }
-      tot += mv[u];
     }
+    tot += (mv[0] + mv[1]) + (mv[2] + mv[3]);  // (a shorter chain of roundings)
     const float g = dwarp_sum4(mv[0], mv[1], mv[2], mv[3], lane);
     over |= !(g < kDGuard);
     const int q = lane >> 3;  // lanes 0, 8, 16, 24 hold rounds r .. r + 3
     if ((lane & 7) == 0 && r + q < rounds) gm[(r + q) * kDWarps + warp] = g;
-#pragma unroll
-    for (int u = 0; u < kDUnroll; ++u) cur[u] = nxt[u];
-  }
+  });
   return over;
 }
 
-template <typename T, int VE>
-__device__ __forceinline__ DSlice slice_sample(const T* a, int v0, int v1, float* gm, DShared& sh) {
+template <typename T, bool EDGE>
+__device__ __forceinline__ DSlice slice_sample(const DRow<T, EDGE>& a, int v0, int v1, uint4* ring,
+                                               float* gm, DShared& sh) {
+  constexpr int VE = DRaw<T>::VE;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // the first batch of rounds; the warp reference: the maximum of the
-  // warp's first-round vectors (-inf if none)
-  DRaw<T, VE> first[kDUnroll];
-  dld_batch<T, VE>(a, v0, v1, 0, first);
+  // the warp reference: the maximum of the warp's first-round vectors (-inf
+  // if none)
+  dring_start<T, EDGE>(ring, a, v0, v1);
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
   float ref;
   {
     float r0 = -INFINITY;
     if (v0 + tid < v1) {
+      DRaw<T> raw;
+      raw.q = *reinterpret_cast<const decltype(raw.q)*>(ring + tid);
       float x[VE];
-      dwiden(first[0], x);
+      dwiden(raw, x);
       r0 = dvmax(x);
     }
     ref = dwarp_max(r0);
   }
   float tot = 0.f;
-  DFin<T, VE> fin;
-  const bool over = slice_masses<T, VE, true>(a, v0, v1, ref, gm, tot, fin, first);
+  DFin<T> fin;
+  const bool over = slice_masses<T, EDGE, true>(a, v0, v1, ref, ring, gm, tot, fin);
   if (__syncthreads_or(over)) {
     // an entry far above its warp's reference: the exact slice maximum, then
     // every group again against it
@@ -372,10 +439,8 @@ __device__ __forceinline__ DSlice slice_sample(const T* a, int v0, int v1, float
     for (int r = 0; r < rounds; ++r) {
       const int v = v0 + r * kDThreads + tid;
       if (v < v1) {
-        DRaw<T, VE> raw;
-        dld(a, v, raw);
         float x[VE];
-        dwiden(raw, x);
+        dwiden(dld<T, EDGE>(a, v), x);
         m = fmaxf(m, dvmax(x));
       }
     }
@@ -384,9 +449,9 @@ __device__ __forceinline__ DSlice slice_sample(const T* a, int v0, int v1, float
     __syncthreads();
     ref = dwarp_max(lane < kDWarps ? sh.red[lane] : -INFINITY);
     tot = 0.f;
-    DFin<T, VE> unused;
-    dld_batch<T, VE>(a, v0, v1, 0, first);
-    slice_masses<T, VE, false>(a, v0, v1, ref, gm, tot, unused, first);
+    DFin<T> unused;
+    dring_start<T, EDGE>(ring, a, v0, v1);
+    slice_masses<T, EDGE, false>(a, v0, v1, ref, ring, gm, tot, unused);
     __syncthreads();  // every warp has read sh.red
   }
   const float wt = dwarp_sum(tot), wf = dwarp_sum(fin.value());
@@ -408,10 +473,11 @@ __device__ __forceinline__ DSlice slice_sample(const T* a, int v0, int v1, float
 // The owner CTA's walk: the group, the vector and the element holding the
 // target tau (in units of 2^R) inside the slice; `last` takes the last entry
 // of positive mass instead.  Warp 0 only; lane `vc` writes the row's outputs.
-template <typename T, int VE>
-__device__ __forceinline__ void slice_walk(const DParams& P, const T* a, int v0, int v1,
+template <typename T, bool EDGE>
+__device__ __forceinline__ void slice_walk(const DParams& P, const DRow<T, EDGE>& a, int v0, int v1,
                                            const float* gm, const DShared& sh, float R, float S,
                                            float tau, bool last, int row) {
+  constexpr int VE = DRaw<T>::VE;
   const int lane = threadIdx.x & 31;
   const int ng = (v1 - v0 + kDThreads - 1) / kDThreads * kDWarps, gpl = (ng + 31) / 32;
   // lane l owns groups [l gpl, (l + 1) gpl)
@@ -458,9 +524,7 @@ __device__ __forceinline__ void slice_walk(const DParams& P, const T* a, int v0,
   float x[VE];
   float mv = 0.f;
   if (gsel >= 0 && v < v1) {
-    DRaw<T, VE> raw;
-    dld(a, v, raw);
-    dwiden(raw, x);
+    dwiden(dld<T, EDGE>(a, v), x);
     mv = dmass(x, nm2);
   }
   const float vin = dwarp_incl_scan(mv, lane), vex = vin - mv;
@@ -494,7 +558,7 @@ __device__ __forceinline__ void slice_walk(const DParams& P, const T* a, int v0,
       qpick = qlast;
     }
     if (pick >= 0) {
-      tok = v * VE + pick;
+      tok = a.element(v, pick);
       pr = qpick / S;
     }
   }
@@ -504,21 +568,24 @@ __device__ __forceinline__ void slice_walk(const DParams& P, const T* a, int v0,
 
 // ------------------------------------------------------------------- the kernel
 
-// Grid: rows x C CTAs in clusters of C.  Shared memory (sampling): one float
-// of group mass per warp and round of a slice.
-template <typename T, int VE, bool STOCH>
+// Grid: rows x C CTAs in clusters of C.  Shared memory: the ring, then
+// (sampling) one float of group mass per warp and round of a slice.
+template <typename T, bool EDGE, bool STOCH>
 __global__ void __launch_bounds__(kDThreads) draft_kernel(const __grid_constant__ DParams P) {
-  extern __shared__ float gm[];
+  extern __shared__ __align__(16) unsigned char dsmem[];
+  uint4* ring = reinterpret_cast<uint4*>(dsmem);
+  float* gm = reinterpret_cast<float*>(dsmem + kDRingBytes);
   __shared__ DShared sh;
   cg::cluster_group cluster = cg::this_cluster();
   const int C = static_cast<int>(cluster.num_blocks());
   const int rank = static_cast<int>(cluster.block_rank());
   const int row = static_cast<int>(blockIdx.x) / C;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const T* a = static_cast<const T*>(P.logits) + static_cast<size_t>(row) * P.V;
-  const int v0 = min(rank * P.W, P.nv), v1 = min(v0 + P.W, P.nv);
+  const DRow<T, EDGE> a(P, row);
+  const int v0 = min(rank * P.W, a.nvec), v1 = min(v0 + P.W, a.nvec);
 
-  const DSlice mine = STOCH ? slice_sample<T, VE>(a, v0, v1, gm, sh) : slice_greedy<T, VE>(a, v0, v1, sh);
+  const DSlice mine = STOCH ? slice_sample<T, EDGE>(a, v0, v1, ring, gm, sh)
+                            : slice_greedy<T, EDGE>(a, v0, v1, ring, sh);
   if (warp == 0 && lane < C) *cluster.map_shared_rank(&sh.slot[rank], lane) = mine;
   cluster.sync();  // every CTA's summary is in every CTA; nothing remote after this
   if (warp != 0) return;
@@ -554,7 +621,7 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const __grid_constant_
     const float tloc = fmaxf(tau - __shfl_sync(0xffffffffu, excl, owner), 0.f);
     if (lane < kDWarps) sh.wscale[lane] = drescale(1.f, sh.wref[lane], R);
     __syncwarp();
-    slice_walk<T, VE>(P, a, v0, v1, gm, sh, R, S, tloc, hit == 0u, row);
+    slice_walk<T, EDGE>(P, a, v0, v1, gm, sh, R, S, tloc, hit == 0u, row);
   }
 }
 

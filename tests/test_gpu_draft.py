@@ -244,3 +244,32 @@ def test_draft_no_rows_is_a_no_op(torch):
     a = torch.zeros((0, 64), dtype=torch.float32, device="cuda")
     tok, pr = A.draft_tokens(a)
     assert tok.numel() == 0 and pr.numel() == 0
+
+
+@pytest.mark.parametrize("mode", [GREEDY, STOCH], ids=["greedy", "stochastic"])
+@pytest.mark.parametrize("dtype", [synth.FP32, synth.BF16], ids=["fp32", "bf16"])
+@pytest.mark.parametrize("V", [2, 3, 7, 8, 9, 17, 2047, 33331])
+def test_draft_rows_off_the_vector_boundaries(torch, V, dtype, mode):
+    # every offset of a row inside its first vector, the draw among the first
+    # or last elements (which no whole vector holds), logits down to the type's
+    # lowest value (what stands in for the elements outside the row)
+    rows = 6
+    rng = np.random.default_rng(V)
+    base = rng.normal(0, 2, (rows, V)).astype(np.float32)
+    base[0, 0] += 20.0
+    base[1, V - 1] += 20.0
+    base[2] = -3.0e38
+    if dtype == synth.BF16:
+        logits = (base.view(np.uint32) >> 16).astype(np.uint16)
+    else:
+        logits = base
+    u = rng.uniform(0, 1, rows).astype(np.float32)
+    o = O.draft_sample(logits, u, dtype=dtype, mode=mode)
+    ok = np.arange(rows) != 2  # (its exponents overflow fp32 in sampling)
+    for offset in (0, 1, 3, 5):
+        tok, pr = run(torch, logits, dtype, mode, u if mode == STOCH else None, offset)
+        if mode == GREEDY:
+            assert tok[2] == 0
+        good = ok & ~o.flagged
+        assert np.array_equal(tok[good], o.tokens[good])
+        np.testing.assert_allclose(pr[good], o.probs[good], rtol=PROB_RTOL)
