@@ -80,17 +80,19 @@ __device__ __forceinline__ bool full_pass1(uint4* ring, const Streams<T>& g, int
   int rs = -1, rt = -1;
   ring_steps<T, true, true>(ring, g, v0, v1, [&](int r, const RawVec<T>& va, const RawVec<T>& vb,
                                                  const RawVec<T>& vt, auto) {
-    f2 sc[NP], tc[NP];
+    f2 sc[NP], tc[NP], e[4][NP];
 #pragma unroll
     for (int h = 0; h < NP; ++h) {
       const f2 a2 = va.pair(h), b2 = vb.pair(h);
       tc[h] = vt.pair(h);
       sc[h] = fma2(beta2, sub2(a2, b2), tc[h]);
-      acc[0] = add2(acc[0], ex2_2(fma2(a2, L2, n2[0])));
-      acc[1] = add2(acc[1], ex2_2(fma2(b2, L2, n2[1])));
-      acc[2] = add2(acc[2], ex2_2(fma2(tc[h], L2, n2[2])));
-      acc[3] = add2(acc[3], ex2_2(fma2(sc[h], L2, n2[3])));
+      e[0][h] = ex2_2(fma2(a2, L2, n2[0]));
+      e[1][h] = ex2_2(fma2(b2, L2, n2[1]));
+      e[2][h] = ex2_2(fma2(tc[h], L2, n2[2]));
+      e[3][h] = ex2_2(fma2(sc[h], L2, n2[3]));
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = add2(acc[q], vsum2(e[q]));
     // strictly larger wins, so the lane's earliest vector keeps a tie
     const float cs = vmax_nan(sc), ct = vmax_nan(tc);
     rs = cs > bs ? r : rs;

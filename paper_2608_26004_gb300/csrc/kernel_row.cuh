@@ -366,6 +366,13 @@ __device__ __forceinline__ EdgeVals load_edges(const KParams& P, const RowCut<T,
   return ed;
 }
 
+// The sum of a vector's pairs.
+template <int NP>
+__device__ __forceinline__ f2 vsum2(const f2 (&x)[NP]) {
+  if constexpr (NP == 4) return add2(add2(x[0], x[1]), add2(x[2], x[3]));
+  else return add2(x[0], x[1]);
+}
+
 // Larger of three with NaN winning (non-finite scores are flagged at the end).
 __device__ __forceinline__ float max3_nan(float a, float b, float c) {
   float r;
@@ -442,6 +449,7 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
   ring_steps<T, AB, true>(ring, g, v0, v1, [&](int r, const RawVec<T>& va, const RawVec<T>& vb,
                                                const RawVec<T>& vt, auto) {
     f2 sc[NP];  // the argmax's scores
+    f2 ea[NP], eb[NP], e3[NP];
 #pragma unroll
     for (int h = 0; h < NP; ++h) {
       const f2 t2 = vt.pair(h);
@@ -449,17 +457,24 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
         const f2 a2 = va.pair(h), b2 = vb.pair(h);
         const f2 amb = sub2(a2, b2);
         if (DRAFT) {
-          acc_a = add2(acc_a, ex2_2(fma2(a2, L2, nA2)));
-          acc_b = add2(acc_b, ex2_2(fma2(b2, L2, nB2)));
+          ea[h] = ex2_2(fma2(a2, L2, nA2));
+          eb[h] = ex2_2(fma2(b2, L2, nB2));
           fin = fma2(amb, 0ull, fin);  // 0 x (non-finite) is NaN
         }
-        if (STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, fma2(bL2, amb, n32))));
+        if (STOCH) e3[h] = ex2_2(fma2(t2, L2, fma2(bL2, amb, n32)));
         if (ARG) sc[h] = fma2(beta2, amb, t2);
       } else {
         sc[h] = t2;
       }
-      if (SUM3 && !STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, n32)));
+      if (SUM3 && !STOCH) e3[h] = ex2_2(fma2(t2, L2, n32));
     }
+    // a vector's terms are added among themselves first: one addition a step
+    // in the running sums' chains of roundings
+    if (DRAFT) {
+      acc_a = add2(acc_a, vsum2(ea));
+      acc_b = add2(acc_b, vsum2(eb));
+    }
+    if (SUM3) acc_3 = add2(acc_3, vsum2(e3));
     if (ARG) {
       // strictly larger wins, so the lane's earliest vector keeps a tie
       const float c = vmax_nan(sc);
