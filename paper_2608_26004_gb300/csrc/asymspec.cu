@@ -56,7 +56,6 @@ struct Plan {
   bool stoch, edge;  // its mode; its form for rows off the 16-byte boundaries
   bool full;         // the recording row kernel (fuse_verify_full) instead
   int nt;            // threads per CTA (kRowThreads or kTThreads)
-  int grid_y;        // the row kernel's grid is (C (K+1), B): grid_y = B (1 otherwise)
 };
 
 const void* row_kernel(int dtype, bool stoch, bool edge, bool full) {
@@ -189,7 +188,6 @@ bool plan_row(int V, int dtype, bool stoch, bool edge, bool full, int forced_C, 
         q.smem = smem(c);
         q.nt = kRowThreads;
         q.kernel = ASYMSPEC_KERNEL_TMA;
-        q.grid_y = 1;
         int n = 0;
         if (query && active_clusters(fn, q, dev.device, &n) == cudaSuccess && n > 0) resident = n;
         cudaGetLastError();
@@ -258,6 +256,19 @@ struct RowProgram {
   bool ok, stoch, full;
 };
 
+// KParams::tail: none in a grid of one wave (per_sm CTAs an SM), else as many
+// elements as the chip holds clusters.
+int tail_elements(const Plan& pl, int B, int per_sm) {
+  const int slots = device_shape().sms * per_sm;
+  return pl.ctas > slots ? std::min(B, slots / pl.C) : 0;
+}
+
+// The grid of the streaming kernels (cluster_row).
+dim3 row_grid(const Plan& pl, int B, int K, int tail) {
+  return tail ? dim3(static_cast<unsigned>(pl.ctas))
+              : dim3(static_cast<unsigned>(pl.C * (K + 1)), static_cast<unsigned>(B));
+}
+
 RowProgram row_program(const asymspec_gate_params& gp, bool full, bool tokens) {
   return {(gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB && (full || !tokens),
           gp.mode == ASYMSPEC_MODE_STOCHASTIC, full};
@@ -287,10 +298,9 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
   pl->vector_path = vec_ok;
   pl->row = false;
   pl->nt = kTThreads;
-  pl->grid_y = 1;
   if (ws_bytes < cluster_ws_bytes(B, K)) return ASYMSPEC_ERR_WORKSPACE;
   bool ok = false;
-  // (its grid is (C (K+1), B): B up to 65535)
+  // (decide_full's grid is (K+1, B): B up to 65535)
   // Greedy and recorded steps stream too (B=64, K=7, V=128256 bf16 greedy:
   // 114 us of staged kernel against 65 us; B=8, K=5, V=151936 bf16 greedy with
   // every row recorded: 48 us a step against 28).  The staged kernel's copy waits are
@@ -305,7 +315,6 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
       pl->kernel = ASYMSPEC_KERNEL_TMA;
       pl->VE = 16 / elt;
       pl->row = true;
-      pl->grid_y = B;
       ok = true;
     } else if (forced_kernel == ASYMSPEC_KERNEL_TMA) {
       return ASYMSPEC_ERR_WORKSPACE;
@@ -406,9 +415,7 @@ cudaLaunchConfig_t launch_config(const Plan& pl, long long ctas, cudaStream_t st
   attr[0].val.clusterDim.x = pl.C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = pl.grid_y > 1 ? dim3(static_cast<unsigned>(ctas / pl.grid_y),
-                                     static_cast<unsigned>(pl.grid_y))
-                              : dim3(static_cast<unsigned>(ctas));
+  cfg.gridDim = dim3(static_cast<unsigned>(ctas));
   cfg.blockDim = dim3(pl.kernel == ASYMSPEC_KERNEL_GENERIC ? kThreads : pl.nt);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = stream;
@@ -430,9 +437,7 @@ cudaError_t active_clusters(KernelFn fn, const Plan& pl, int device, int* out) {
       }
   }
   cudaLaunchAttribute attr[1];
-  Plan one = pl;  // a grid of one cluster
-  one.grid_y = 1;
-  cudaLaunchConfig_t cfg = launch_config(one, pl.C, nullptr, attr);
+  cudaLaunchConfig_t cfg = launch_config(pl, pl.C, nullptr, attr);  // a grid of one cluster
   int n = 0;
   const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
   if (e != cudaSuccess) return e;
@@ -730,6 +735,7 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   P.recs = static_cast<int4*>(workspace);
   P.tma_threads = pl.nt;
   P.head0 = static_cast<int>(offset(logits_full) / elt);
+  P.tail = pl.row ? tail_elements(pl, B, pl.full ? kFullMinBlocks : kRowMinBlocks) : 0;
   P.lp_vec = P.head0 == 0 && aligned(out_fused_logprobs, 16) ? 1 : 0;
   // the chunk waits of the TMA kernel: bounded, or (test hook) giving up at once
   P.copy_wait_ns =
@@ -749,6 +755,7 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   const long long ctas = pl.ctas;  // one cluster of C CTAs per row
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = launch_config(pl, ctas, static_cast<cudaStream_t>(stream), attr);
+  if (pl.row) cfg.gridDim = row_grid(pl, B, K, P.tail);
   void* args[] = {&P};
   P.group_stride = pl.group_stride;
   if (pl.kernel == ASYMSPEC_KERNEL_TMA) {
@@ -1095,6 +1102,7 @@ bool plan_xrow(int S, int elt, long long rows, int sms, Plan* pl) {
     pl->smem = static_cast<int>(smem);
     pl->nt = kXRowThreads;
   }
+  pl->ctas = rows * pl->C;
   return best > 0.0;
 }
 
@@ -1122,7 +1130,9 @@ int run_xrow(const Plan& pl, const void* a, const void* b, int V_d, const void* 
   P.C = pl.C;
   P.W = pl.W;
   P.sh_off = pl.sh_off;
-  P.rows = static_cast<long long>(B) * (K + 1);
+  const long long rows = static_cast<long long>(B) * (K + 1);
+  P.rows = rows;
+  P.tail = tail_elements(pl, B, 1);
   P.out_len = out_len;
   P.out_next = out_next;
   P.err_word = err_word;
@@ -1149,7 +1159,7 @@ int run_xrow(const Plan& pl, const void* a, const void* b, int V_d, const void* 
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(pl.C * (K + 1)), static_cast<unsigned>(B));
+  cfg.gridDim = row_grid(pl, B, K, P.tail);
   cfg.blockDim = dim3(pl.nt);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = st;
@@ -1298,7 +1308,7 @@ int asymspec_fuse_verify_xvocab(const void* logits_full, const void* logits_comp
   const long long rows = static_cast<long long>(B) * (K + 1);
   const int elt = elt_size(dtype);
   Plan pl = {};
-  if ((gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB && B <= 65535 && rows <= 8LL * 65535 &&
+  if ((gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB && rows <= 8LL * 65535 &&
       plan_xrow(S, elt, rows, device_shape().sms, &pl)) {
     if (!logits_full || !logits_comp || !logits_ver || !map_d || !map_v) return ASYMSPEC_ERR_INVALID_ARG;
     if (!aligned(logits_full, elt) || !aligned(logits_comp, elt) || !aligned(logits_ver, elt) ||

@@ -301,8 +301,9 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
   const int tid = static_cast<int>(threadIdx.x);
   const int lane = tid & 31, warp = tid >> 5;
   const int C = P.C;
-  const int k = static_cast<int>(cluster_id_x());
-  const unsigned row32 = cluster_id_y() * static_cast<unsigned>(P.K + 1) + static_cast<unsigned>(k);
+  unsigned bi, k;
+  cluster_row(P, bi, k);
+  const unsigned row32 = bi * static_cast<unsigned>(P.K + 1) + k;
   const RowCut<T, EDGE> cut(P, row32);
   const int Wv = P.W / VE, s0 = rank * Wv;  // the slice: vectors [s0, s0 + nv) of the row
   const int nv = max(0, min(Wv, cut.nvec - s0));

@@ -352,8 +352,7 @@ __host__ __device__ constexpr int xrow_shared_bytes(int C) {
   return static_cast<int>(sizeof(RowShared) + C * kXRowWarps * sizeof(W1));
 }
 
-// Grid: (C (K+1), B) CTAs of kXRowThreads threads in clusters of (C, 1, 1),
-// one CTA an SM.  P.V = S; P.tokens holds pair indices.  Leaves what
+// Grid: C B (K+1) CTAs of kXRowThreads threads in clusters of C, one CTA an SM.  P.V = S; P.tokens holds pair indices.  Leaves what
 // fuse_verify_row leaves, C kXRowWarps records a row.
 template <typename T, bool STOCH>
 __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParams P,
@@ -366,10 +365,10 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
   const int tid = static_cast<int>(threadIdx.x);
   const int lane = tid & 31, warp = tid >> 5;
   const int C = P.C;
-  const int k = static_cast<int>(cluster_id_x());
-  const int bi = static_cast<int>(cluster_id_y());
-  const unsigned row32 = static_cast<unsigned>(bi) * static_cast<unsigned>(P.K + 1) +
-                         static_cast<unsigned>(k);
+  unsigned ubi, uk;
+  cluster_row(P, ubi, uk);
+  const int k = static_cast<int>(uk), bi = static_cast<int>(ubi);
+  const unsigned row32 = ubi * static_cast<unsigned>(P.K + 1) + uk;
   const bool draft = k < P.K;
   const bool only_t = !STOCH && !draft && !P.fuse_bonus;  // Algorithm 1 emits argmax t
   const int j0 = rank * P.W, n = max(0, min(P.W, P.V - j0));

@@ -230,3 +230,18 @@ def test_recorded_rows(torch, B, K, V, dtype, offset, cluster, mode):
         compare(batch, g, o, mode=mode, check_stats=div != A.DIV_KL)
         err = np.abs(g["row_stats"][..., 4] - o.D)
         assert np.all(err <= D_TOL * np.maximum(1.0, np.abs(o.D)))
+
+
+# ---------------------------------------------------------------- the order of the rows
+
+@pytest.mark.parametrize("B,K", [(40, 3), (300, 1), (61, 5), (127, 4)])
+@pytest.mark.parametrize("mode", [GREEDY, STOCH])
+def test_every_row_is_taken_in_batches_of_several_waves(torch, B, K, mode):
+    # more clusters than the chip holds: the bonus rows of the last elements
+    # come last (all of them, or some), recorded rows likewise
+    batch, _ = batch_over_the_threshold(B, K, 2048, synth.BF16, 2000 + B, torch, mode)
+    o = run_oracle(batch, mode=mode)
+    for cluster in (0, 4, 16):
+        g = run_gpu(batch, torch, mode=mode, full="row", cluster_size=cluster)
+        check_decisions(batch, np.arange(B), g["accept_len"], g["next_token"], o, mode)
+    compare(batch, run_gpu(batch, torch, mode=mode, cluster_size=16), o, mode=mode)
