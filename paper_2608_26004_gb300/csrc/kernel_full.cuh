@@ -23,8 +23,8 @@ namespace asymspec_impl {
 
 constexpr int kFullMinBlocks = 3;  // CTAs per SM (85 registers a thread)
 
-// A warp's pass-1 record: the references (nats) and sums of
-// 2^((x - ref) log2 e) of a, b, t and s; the largest s and t and the lowest
+// A warp's pass-1 record: the references (whole numbers, in log2 units) and
+// sums of 2^(x log2 e - ref) of a, b, t and s; the largest s and t and the lowest
 // vectors that hold them (INT_MAX: none; NaN: non-finite values were seen).
 struct __align__(16) WF {
   float ref[4], s[4];
@@ -72,8 +72,8 @@ __device__ __forceinline__ bool full_pass1(uint4* ring, const Streams<T>& g, int
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (EDGE && ed.own) ref[q] = fmaxf(ref[q], ev[q]);
-    ref[q] = warp_max(ref[q]);
-    n2[q] = pk(-ref[q] * kLog2e, -ref[q] * kLog2e);
+    ref[q] = ref_of(warp_max(ref[q]));
+    n2[q] = pk(-ref[q], -ref[q]);
     acc[q] = 0ull;
   }
   float bs = -INFINITY, bt = -INFINITY;
@@ -169,8 +169,9 @@ __device__ __noinline__ void full_pass1_online(const Streams<T>& g, int v0, int 
   for (int q = 0; q < 4; ++q) {
     const float M = warp_max(m[q]);
     const float sc = (s[q] == 0.f || m[q] == M) ? s[q] : s[q] * ex2((m[q] - M) * kLog2e);
-    e.ref[q] = M;
+    e.ref[q] = ref_of(M);
     e.s[q] = warp_sum(sc);
+    e.s[q] *= ref_residual(M, e.ref[q]);
   }
 }
 
@@ -199,14 +200,14 @@ __device__ __forceinline__ void combine_full(const WF* rec, int n, float (&lse)[
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float s = rec[i].s[q], r = rec[i].ref[q];
-      sum[q] += (s == 0.f || r == ref[q]) ? s : s * ex2((r - ref[q]) * kLog2e);
+      sum[q] += (s == 0.f || r == ref[q]) ? s : s * ex2(r - ref[q]);
     }
     if (rec[i].vs == vs) is = min(is, rec[i].is);
     if (rec[i].vt == vt) it = min(it, rec[i].it);
   }
   warp_sum4(sum[0], sum[1], sum[2], sum[3]);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) lse[q] = ref[q] + logf(sum[q]);
+  for (int q = 0; q < 4; ++q) lse[q] = lse_of(ref[q], sum[q]);
   is = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(is)));
   it = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(it)));
   if (__any_sync(0xffffffffu, bad_s)) vs = NAN;
@@ -404,7 +405,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
       jsum = row_jsd_wide<T, EDGE>(g, v0, v1, A2, B2, ed);
   }
   if (lane == 0) {
-    const float qf = STOCH && e.s[3] > 0.f ? e.s[3] * ex2(e.ref[3] * kLog2e - S2) : 0.f;
+    const float qf = STOCH && e.s[3] > 0.f ? e.s[3] * ex2(e.ref[3] - S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

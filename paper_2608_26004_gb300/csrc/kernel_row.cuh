@@ -155,8 +155,8 @@ constexpr int kRowThreads = 256;  // threads per CTA of the row kernel
 constexpr int kRowMinBlocks = 4;  // CTAs per SM (64 registers a thread)
 static_assert(kRowThreads / 32 <= kRowMaxWarps, "one record slot per warp");
 
-// A warp's pass-1 record: the references (nats) and sums of
-// 2^((x - ref) log2 e) of a, b and the fused score (stochastic) or t
+// A warp's pass-1 record: the references (whole numbers, in log2 units) and
+// sums of 2^(x log2 e - ref) of a, b and the fused score (stochastic) or t
 // (greedy); greedy: the largest fused score (t on an unfused bonus row) and
 // the lowest vector of the row that holds it (INT_MAX: none; NaN: non-finite
 // scores were seen).
@@ -165,6 +165,32 @@ struct __align__(16) W1 {
   float v;
   int vec;
 };
+
+// A stream's reference from one of its values: a whole number of log2 units,
+// so that neither the exponents' reference nor a rescale between two
+// references (a power of two) adds a rounding.
+__device__ __forceinline__ float ref_of(float x) { return rintf(x * kLog2e); }
+
+// 2^(x log2 e - ref_of(x)), the factor that takes a sum against x (nats) to
+// one against its reference; 1 where fp32 does not resolve it (no finite sum
+// has |x| that large but for logits of 10^6 and more).
+__device__ __forceinline__ float ref_residual(float x, float ref) {
+  return fabsf(ref) < 4194304.f ? ex2(fmaf(x, kLog2e, -ref)) : 1.f;
+}
+
+// ln(2^ref sum) with the exponents kept apart from the logarithm of the
+// significand (ln 2 in two parts, the first of 12 bits, so that its product
+// with the exponent is exact): ref + log2 sum is usually a small difference of
+// larger numbers.
+__device__ __forceinline__ float lse_of(float ref, float sum) {
+  if (!(sum >= kMinNormal && sum <= 3.402823466e38f)) return ref * kLn2 + logf(sum);
+  const int bits = __float_as_int(sum);
+  const float n = ref + static_cast<float>((bits >> 23) - 127);
+  const float m = __int_as_float((bits & 0x007FFFFF) | 0x3F800000);
+  constexpr double kLn2d = 0.69314718055994530942;
+  constexpr double hi = 2839.0 / 4096.0;
+  return fmaf(n, static_cast<float>(hi), fmaf(n, static_cast<float>(kLn2d - hi), logf(m)));
+}
 
 // What pass 2 does for a row (row_path): nothing, the residual masses alone,
 // or the divergence (and, in stochastic mode, the masses).
@@ -441,7 +467,10 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
     rb0 = warp_max(rb0);
   }
   if (SUM3) r30 = warp_max(r30);
-  const float nA = -ra0 * kLog2e, nB = -rb0 * kLog2e, n3 = -r30 * kLog2e;
+  ra0 = ref_of(ra0);
+  rb0 = ref_of(rb0);
+  r30 = ref_of(r30);
+  const float nA = -ra0, nB = -rb0, n3 = -r30;
   const f2 nA2 = pk(nA, nA), nB2 = pk(nB, nB), n32 = pk(n3, n3);
   f2 acc_a = 0ull, acc_b = 0ull, acc_3 = 0ull, fin = 0ull;
   float best = -INFINITY;
@@ -576,8 +605,9 @@ __device__ __noinline__ void row_pass1_online(const Streams<T>& g, int v0, int v
     const float M = warp_max(m[q]);
     float sc = (s[q] == 0.f || m[q] == M) ? s[q] : s[q] * ex2((m[q] - M) * kLog2e);
     if (q == 0 && DRAFT && chk) sc += fin;  // 0, or NaN
-    e.ref[q] = M;
+    e.ref[q] = ref_of(M);
     e.s[q] = warp_sum(sc);
+    e.s[q] *= ref_residual(M, e.ref[q]);
   }
   if (!DRAFT) {
     e.ref[0] = e.ref[1] = -INFINITY;
@@ -708,8 +738,7 @@ __device__ __forceinline__ void combine_records(const W1* rec, int n, float (&re
     const W1 r = rec[i];
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-      sum[q] += (r.s[q] == 0.f || r.ref[q] == ref[q]) ? r.s[q]
-                                                      : r.s[q] * ex2((r.ref[q] - ref[q]) * kLog2e);
+      sum[q] += (r.s[q] == 0.f || r.ref[q] == ref[q]) ? r.s[q] : r.s[q] * ex2(r.ref[q] - ref[q]);
     if (r.v == v) lo = min(lo, r.vec);
   }
   float z = 0.f;
@@ -892,10 +921,10 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
     int vec;
     combine_records(sh->recv(), nrec, ref, sum, v, vec);
     float lse[4];
-    lse[0] = draft ? ref[0] + logf(sum[0]) : NAN;
-    lse[1] = draft ? ref[1] + logf(sum[1]) : NAN;
-    lse[2] = !STOCH && draft ? ref[2] + logf(sum[2]) : NAN;
-    lse[3] = STOCH ? ref[2] + logf(sum[2]) : NAN;
+    lse[0] = draft ? lse_of(ref[0], sum[0]) : NAN;
+    lse[1] = draft ? lse_of(ref[1], sum[1]) : NAN;
+    lse[2] = !STOCH && draft ? lse_of(ref[2], sum[2]) : NAN;
+    lse[3] = STOCH ? lse_of(ref[2], sum[2]) : NAN;
     // (a token outside the vocabulary voids the element whatever the row does)
     const int path = draft && tok_ok ? row_path<STOCH>(P, lse, da, db, dt, u, pd) : kPathAccept;
     if (lane == 0) {
@@ -954,7 +983,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
     // this warp's record: its block is one inverse-CDF group of the row.  The
     // fused mass (the bonus row's draw, and a draft row's where the row's
     // whole residual is zero) comes from the warp's pass-1 sum.
-    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(e.ref[2] * kLog2e - S2) : 0.f;
+    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(e.ref[2] - S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

@@ -154,7 +154,10 @@ __device__ __forceinline__ bool x_pass1(const XSlice<T>& x, int p0, int p1, floa
     rb0 = warp_max(rb0);
   }
   if (SUM3) r30 = warp_max(r30);
-  const float nA = -ra0 * kLog2e, nB = -rb0 * kLog2e, n3 = -r30 * kLog2e;
+  ra0 = ref_of(ra0);
+  rb0 = ref_of(rb0);
+  r30 = ref_of(r30);
+  const float nA = -ra0, nB = -rb0, n3 = -r30;
   const f2 nA2 = pk(nA, nA), nB2 = pk(nB, nB), n32 = pk(n3, n3);
   f2 acc_a = 0ull, acc_b = 0ull, acc_3 = 0ull, fin = 0ull;
   float best = -INFINITY;
@@ -236,8 +239,9 @@ __device__ __noinline__ void x_pass1_online(const XSlice<T>& x, int p0, int p1, 
     const float M = warp_max(m[q]);
     float sc = (s[q] == 0.f || m[q] == M) ? s[q] : s[q] * ex2((m[q] - M) * kLog2e);
     if (q == 0 && DRAFT && chk) sc += fin;  // 0, or NaN
-    e.ref[q] = M;
+    e.ref[q] = ref_of(M);
     e.s[q] = warp_sum(sc);
+    e.s[q] *= ref_residual(M, e.ref[q]);
   }
   if (!DRAFT) {
     e.ref[0] = e.ref[1] = -INFINITY;
@@ -449,10 +453,10 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
     int vec;
     combine_records(sh->recv(), nrec, ref, sum, v, vec);
     float lse[4];
-    lse[0] = draft ? ref[0] + logf(sum[0]) : NAN;
-    lse[1] = draft ? ref[1] + logf(sum[1]) : NAN;
-    lse[2] = !STOCH && draft ? ref[2] + logf(sum[2]) : NAN;
-    lse[3] = STOCH ? ref[2] + logf(sum[2]) : NAN;
+    lse[0] = draft ? lse_of(ref[0], sum[0]) : NAN;
+    lse[1] = draft ? lse_of(ref[1], sum[1]) : NAN;
+    lse[2] = !STOCH && draft ? lse_of(ref[2], sum[2]) : NAN;
+    lse[3] = STOCH ? lse_of(ref[2], sum[2]) : NAN;
     const int path = draft && tok_ok ? row_path<STOCH>(P, lse, da, db, dt, u, pd) : kPathAccept;
     if (lane == 0) {
 #pragma unroll
@@ -485,7 +489,7 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
       jsum = x_jsd_wide<T>(x, p0, p1, A2, B2);
   }
   if (lane == 0 && (second || (STOCH && !draft))) {
-    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(e.ref[2] * kLog2e - S2) : 0.f;
+    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(e.ref[2] - S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + (static_cast<size_t>(row32) * nrec + rank * NW + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);
