@@ -256,17 +256,16 @@ struct RowProgram {
   bool ok, stoch, full;
 };
 
-// KParams::tail: none in a grid of one wave (per_sm CTAs an SM), else as many
-// elements as the chip holds clusters.
-int tail_elements(const Plan& pl, int B, int per_sm) {
+// KParams::tail_first: no element's in a grid of one wave (per_sm CTAs an SM),
+// else the last ones', as many as the chip holds clusters.
+int tail_first(const Plan& pl, int B, int per_sm) {
   const int slots = device_shape().sms * per_sm;
-  return pl.ctas > slots ? std::min(B, slots / pl.C) : 0;
+  return pl.ctas > slots ? std::max(0, B - slots / pl.C) : B;
 }
 
-// The grid of the streaming kernels (cluster_row).
-dim3 row_grid(const Plan& pl, int B, int K, int tail) {
-  return tail ? dim3(static_cast<unsigned>(pl.ctas))
-              : dim3(static_cast<unsigned>(pl.C * (K + 1)), static_cast<unsigned>(B));
+// The streaming kernels' grid: a cluster per row (cluster_row); B up to 65535.
+dim3 row_grid(const Plan& pl, int B, int K) {
+  return dim3(static_cast<unsigned>(pl.C * (K + 1)), static_cast<unsigned>(B));
 }
 
 RowProgram row_program(const asymspec_gate_params& gp, bool full, bool tokens) {
@@ -735,7 +734,7 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   P.recs = static_cast<int4*>(workspace);
   P.tma_threads = pl.nt;
   P.head0 = static_cast<int>(offset(logits_full) / elt);
-  P.tail = pl.row ? tail_elements(pl, B, pl.full ? kFullMinBlocks : kRowMinBlocks) : 0;
+  P.tail_first = pl.row ? tail_first(pl, B, pl.full ? kFullMinBlocks : kRowMinBlocks) : B;
   P.lp_vec = P.head0 == 0 && aligned(out_fused_logprobs, 16) ? 1 : 0;
   // the chunk waits of the TMA kernel: bounded, or (test hook) giving up at once
   P.copy_wait_ns =
@@ -755,7 +754,7 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   const long long ctas = pl.ctas;  // one cluster of C CTAs per row
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = launch_config(pl, ctas, static_cast<cudaStream_t>(stream), attr);
-  if (pl.row) cfg.gridDim = row_grid(pl, B, K, P.tail);
+  if (pl.row) cfg.gridDim = row_grid(pl, B, K);
   void* args[] = {&P};
   P.group_stride = pl.group_stride;
   if (pl.kernel == ASYMSPEC_KERNEL_TMA) {
@@ -1132,7 +1131,7 @@ int run_xrow(const Plan& pl, const void* a, const void* b, int V_d, const void* 
   P.sh_off = pl.sh_off;
   const long long rows = static_cast<long long>(B) * (K + 1);
   P.rows = rows;
-  P.tail = tail_elements(pl, B, 1);
+  P.tail_first = tail_first(pl, B, 1);
   P.out_len = out_len;
   P.out_next = out_next;
   P.err_word = err_word;
@@ -1159,7 +1158,7 @@ int run_xrow(const Plan& pl, const void* a, const void* b, int V_d, const void* 
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = row_grid(pl, B, K, P.tail);
+  cfg.gridDim = row_grid(pl, B, K);
   cfg.blockDim = dim3(pl.nt);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = st;
@@ -1308,7 +1307,8 @@ int asymspec_fuse_verify_xvocab(const void* logits_full, const void* logits_comp
   const long long rows = static_cast<long long>(B) * (K + 1);
   const int elt = elt_size(dtype);
   Plan pl = {};
-  if ((gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB && rows <= 8LL * 65535 &&
+  if ((gp.flags & ASYMSPEC_FLAG_DELTA_MASK) == ASYMSPEC_DELTA_AB &&
+      B <= 65535 && rows <= 8LL * 65535 &&
       plan_xrow(S, elt, rows, device_shape().sms, &pl)) {
     if (!logits_full || !logits_comp || !logits_ver || !map_d || !map_v) return ASYMSPEC_ERR_INVALID_ARG;
     if (!aligned(logits_full, elt) || !aligned(logits_comp, elt) || !aligned(logits_ver, elt) ||

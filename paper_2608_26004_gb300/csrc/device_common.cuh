@@ -437,7 +437,7 @@ struct KParams {
   int tma_threads;      // threads per CTA of the row kernel (its group layout)
   unsigned long long copy_wait_ns;  // limit of each bulk-copy wait (0: give up at once)
   int lp_vec;           // fuse_verify_full: logprobs takes 16-byte stores
-  int tail;             // cluster_row: elements whose bonus rows come last
+  int tail_first;       // cluster_row: from this element on bonus rows come last
   int head0;            // fuse_verify_row, EDGE: elements from a 16-byte boundary to the logits
 };
 

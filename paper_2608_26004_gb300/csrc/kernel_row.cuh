@@ -183,10 +183,10 @@ __device__ __forceinline__ float ref_residual(float x, float ref) {
 // with the exponent is exact): ref + log2 sum is usually a small difference of
 // larger numbers.
 __device__ __forceinline__ float lse_of(float ref, float sum) {
-  if (!(sum >= kMinNormal && sum <= 3.402823466e38f)) return ref * kLn2 + logf(sum);
+  const bool normal = sum >= kMinNormal && sum <= 3.402823466e38f;  // else logf as it is
   const int bits = __float_as_int(sum);
-  const float n = ref + static_cast<float>((bits >> 23) - 127);
-  const float m = __int_as_float((bits & 0x007FFFFF) | 0x3F800000);
+  const float n = normal ? ref + static_cast<float>((bits >> 23) - 127) : ref;
+  const float m = normal ? __int_as_float((bits & 0x007FFFFF) | 0x3F800000) : sum;
   constexpr double kLn2d = 0.69314718055994530942;
   constexpr double hi = 2839.0 / 4096.0;
   return fmaf(n, static_cast<float>(hi), fmaf(n, static_cast<float>(kLn2d - hi), logf(m)));
@@ -748,35 +748,27 @@ __device__ __forceinline__ void combine_records(const W1* rec, int n, float (&re
 }
 
 // The row of this cluster: in memory order, but the bonus rows of the last
-// KParams::tail elements (about as many as the chip holds clusters; a grid of
-// one wave has none and is (C (K+1), B)) come last: they have no second pass, so the grid does not
-// end on rows that have.  B=64, K=7, V=128256 bf16: stochastic 73.4 -> 71.8 us
-// a step, greedy 66.1 -> 64.6.  (All bonus rows last cost fp32 rows of B=256
-// 0.6 %, all rows k-major 1.4 %: the rows in flight lie on more pages.)
+// elements (from KParams::tail_first on, about as many as the chip holds
+// clusters; a grid of one wave has none) come last: they have no second pass,
+// so the grid does not end on rows that have.  B=64, K=7, V=128256 bf16:
+// stochastic 72.8 -> 71.4 us a step, greedy 65.5 -> 64.3.  (All bonus rows last
+// cost fp32 rows of B=256 0.6 %, all rows k-major 1.4 %: the rows in flight lie
+// on more pages.)
 __device__ __forceinline__ void cluster_row(const KParams& P, unsigned& bi, unsigned& k) {
-  unsigned c;
-  asm("mov.u32 %0, %%clusterid.x;" : "=r"(c));
-  const unsigned K = static_cast<unsigned>(P.K), K1 = K + 1u, tail = static_cast<unsigned>(P.tail);
-  if (tail == 0u) {
-    k = c;
-    asm("mov.u32 %0, %%clusterid.y;" : "=r"(bi));
-    return;
-  }
-  const unsigned first = static_cast<unsigned>(P.B) - tail;  // elements in plain order
-  if (c < first * K1) {
-    bi = c / K1;
-    k = c - bi * K1;
-    return;
-  }
-  c -= first * K1;
-  if (c < tail * K) {
-    bi = c / K;
-    k = c - bi * K;
+  asm("mov.u32 %0, %%clusterid.x;" : "=r"(k));
+  asm("mov.u32 %0, %%clusterid.y;" : "=r"(bi));
+  const unsigned first = static_cast<unsigned>(P.tail_first);
+  if (bi < first) return;
+  const unsigned K = static_cast<unsigned>(P.K);
+  const unsigned l = (bi - first) * (K + 1u) + k;  // of the last elements' rows
+  const unsigned drafts = (static_cast<unsigned>(P.B) - first) * K;
+  if (l < drafts) {
+    bi = first + l / K;
+    k = l % K;
   } else {
-    bi = c - tail * K;
+    bi = first + l - drafts;
     k = K;
   }
-  bi += first;
 }
 
 // What a draft row's second pass has to find out, from its normalisers and
