@@ -249,6 +249,25 @@ TmaLayout tma_layout(int B, int K, int C, int group_stride = kGroupsMax) {
   return L;
 }
 
+// The streaming kernels' parts of a workspace that holds tma_layout(B, K, C):
+// at its end, where they take the room of the group masses too (those kernels
+// keep none).  A workspace may serve calls of other B, whose tickets must
+// still be zero then: they lie among its first bytes (after 16 (K + 1) a batch
+// element), which these parts leave alone.  fuse_verify_full clears its own.
+struct RowLayout {
+  size_t recs, tickets, stat, p2rec;
+};
+
+RowLayout row_layout(int B, int K, int C, size_t workspace_bytes) {
+  const size_t R = static_cast<size_t>(B) * (K + 1);
+  RowLayout L;
+  L.p2rec = (workspace_bytes - R * C * kRowMaxWarps * sizeof(X2)) / 256 * 256;
+  L.stat = L.p2rec - round_up(R * sizeof(RowStat), 256);
+  L.tickets = L.stat - round_up(static_cast<size_t>(B) * sizeof(unsigned), 256);
+  L.recs = L.tickets - ws_records_bytes(B, K);
+  return L;
+}
+
 // What the streaming row kernels could take of a call: delta = a - b, and no
 // per-row outputs (fuse_verify_row) or all of what they need (fuse_verify_full);
 // the row tokens alone stay with the staged kernel.
@@ -758,11 +777,19 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   void* args[] = {&P};
   P.group_stride = pl.group_stride;
   if (pl.kernel == ASYMSPEC_KERNEL_TMA) {
-    const TmaLayout L = tma_layout(B, K, pl.C, pl.group_stride);
     char* base = static_cast<char*>(workspace);
-    P.row_stat = base + L.stat;
-    P.pass2_rec = reinterpret_cast<float*>(base + L.p2rec);
-    P.group_mass = reinterpret_cast<float*>(base + L.groups);
+    if (pl.row) {
+      const RowLayout L = row_layout(B, K, pl.C, workspace_bytes);
+      P.recs = reinterpret_cast<int4*>(base + L.recs);
+      P.tickets = reinterpret_cast<unsigned int*>(base + L.tickets);
+      P.row_stat = base + L.stat;
+      P.pass2_rec = reinterpret_cast<float*>(base + L.p2rec);
+    } else {
+      const TmaLayout L = tma_layout(B, K, pl.C, pl.group_stride);
+      P.row_stat = base + L.stat;
+      P.pass2_rec = reinterpret_cast<float*>(base + L.p2rec);
+      P.group_mass = reinterpret_cast<float*>(base + L.groups);
+    }
   }
   e = record_timing(opts, true, cfg.stream);
   if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, fn, args);

@@ -304,6 +304,8 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
   const int C = P.C;
   unsigned bi, k;
   cluster_row(P, bi, k);
+  // the counter of the element's decided rows (decide_full waits for this grid)
+  if (k == 0 && rank == 0 && tid == 0) P.tickets[bi] = 0u;
   const unsigned row32 = bi * static_cast<unsigned>(P.K + 1) + k;
   const RowCut<T, EDGE> cut(P, row32);
   const int Wv = P.W / VE, s0 = rank * Wv;  // the slice: vectors [s0, s0 + nv) of the row

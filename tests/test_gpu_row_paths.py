@@ -245,3 +245,29 @@ def test_every_row_is_taken_in_batches_of_several_waves(torch, B, K, mode):
         g = run_gpu(batch, torch, mode=mode, full="row", cluster_size=cluster)
         check_decisions(batch, np.arange(B), g["accept_len"], g["next_token"], o, mode)
     compare(batch, run_gpu(batch, torch, mode=mode, cluster_size=16), o, mode=mode)
+
+
+@pytest.mark.parametrize("first,second", [
+    # (B, V, recorded) of two calls on one workspace: every element of the
+    # second is decided, whatever the first left where its counters lie
+    ((4, 16392, False), (64, 16392, True)),
+    ((4, 16391, False), (64, 1001, False)),   # then the generic kernel
+    ((64, 16392, True), (4, 1001, False)),
+    ((64, 16392, True), (4, 16392, True)),
+])
+@pytest.mark.parametrize("mode", [GREEDY, STOCH])
+def test_batches_of_several_sizes_share_a_workspace(torch, mode, first, second):
+    K = 7
+    fv = A.FuseVerify(64, K, V_max=16392)
+    for B, V, recorded in (first, second):
+        batch = synth.generate(synth.Recipe(), 7, B, K, V, synth.BF16)
+        x = device_inputs(batch, torch)
+        out = {"accept_len": torch.full((B,), -7, dtype=torch.int32, device="cuda"),
+               "next_token": torch.full((B,), -7, dtype=torch.int32, device="cuda"),
+               "error_word": torch.zeros(1, dtype=torch.int32, device="cuda")}
+        res = fv(x["a"], x["b"], x["t"], x["tokens"], x["probs"], x["unif"], mode=mode,
+                 row_stats=recorded, row_tokens=recorded, out=out)
+        torch.cuda.synchronize()
+        want = run_gpu(batch, torch, mode=mode, full=recorded, tokens=recorded, logprobs=False)
+        for name in ("accept_len", "next_token"):
+            np.testing.assert_array_equal(res[name].cpu().numpy(), want[name])
