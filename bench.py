@@ -85,8 +85,8 @@ def peaks():
 
 def kernel_name(A, info) -> str:
     """The row kernel a call launches (the roofline's kernel)."""
-    if info.kernel == A.KERNEL_TMA:
-        return "fuse_verify_row" if info.row_kernel else "fuse_verify_tma"
+    if info.kernel == A.KERNEL_TMA:  # both modes of the production program
+        return "fuse_verify_row"
     return "fuse_verify_generic" if info.kernel == A.KERNEL_GENERIC else str(info.kernel)
 
 
@@ -340,7 +340,7 @@ def draft_timing(torch, A, sets, B, K, V, mode, dev, steps):
 
 def xvocab_timing(torch, A, synth, mode, dev, steps, timed, stream):
     """The cross-family step (asymspec_fuse_verify_xvocab: map check, row kernel,
-    emission) on the bench workload's batch shape over a Qwen3-sized drafter
+    decision kernel) on the bench workload's batch shape over a Qwen3-sized drafter
     vocabulary, a Llama-3-sized verifier vocabulary and the paper's shared set,
     and its gather (asymspec_xvocab_gather) alone; CUDA events on the stream."""
     w = synth.CONFIGS[WORKLOAD_CFG]

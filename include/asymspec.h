@@ -182,7 +182,9 @@ void asymspec_default_gate_params(asymspec_gate_params* p);
  * record per row and 4 B of ticket per element (all the generic kernel
  * needs); then, for ASYMSPEC_KERNEL_TMA with clusters of C CTAs, 48 B of
  * pass-1 results per row and 352 B per row and CTA of pass-2 record and
- * inverse-CDF group masses, which its decision kernel reads.  With less than
+ * inverse-CDF group masses, which its decision kernel reads (its streaming
+ * row kernels keep all they leave at the end of the workspace, clear of any
+ * batch size's tickets).  With less than
  * the TMA part the automatic choice falls back to the generic kernel.  The tickets
  * must be zero before the first use (cudaMemset or
  * asymspec_workspace_reset); every call that completes leaves them zero

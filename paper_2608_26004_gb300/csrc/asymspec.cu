@@ -3,10 +3,10 @@
 //
 //   fuse_verify_tma      (kernel_tma.cuh) one cluster per row, each CTA's
 //                        slice brought in by chunked 1-D bulk copies, per-row
-//                        programs; 16-byte aligned rows with per-row outputs
-//                        or another delta source.  Its rows are decided, and
-//                        Algorithm 1's scan run, by decide_rows, a second
-//                        launch.
+//                        programs; 16-byte aligned rows where the streaming
+//                        kernels do not apply (the row tokens alone, another
+//                        delta source).  Its rows are decided, and Algorithm
+//                        1's scan run, by decide_rows, a second launch.
 //   fuse_verify_row      (kernel_row.cuh) the same decomposition with no
 //                        slice in shared memory (pass 1 from HBM, four CTAs
 //                        per SM; a second pass from the L2 only for rows whose
@@ -14,6 +14,10 @@
 //                        per-row outputs, delta = a - b), also for rows off
 //                        the 16-byte boundaries.  Its rows are decided by
 //                        decide_blocks.
+//   fuse_verify_full     (kernel_full.cuh) the same for the steps that record
+//                        row statistics or log-probabilities; decide_full.
+//   fuse_verify_xrow     (kernel_xrow.cuh) the cross-family step on the rows
+//                        as they are; decide_xrow.
 //   fuse_verify_generic  (kernel_generic.cuh) one cluster per row, any
 //                        element-aligned input; folds the scan into the same
 //                        launch through a per-element ticket in the workspace.
@@ -122,11 +126,10 @@ bool plan_tma(int V, int elt, int forced_C, Plan* pl) {
 // costs of a CTA (its launch, the first loads, the exchange of the pass-1
 // records) are spread.  With at least one wave of clusters of 8 (rows x 8 >=
 // 4 CTAs x SMs): the smallest C of kRowClusters whose resident clusters
-// hold at most kRowL2Budget of rows.  Measured on GB300 with a second pass on
-// every row (kernel time, rows in flight):
-//   B=64, K=7, V=128256 bf16:  C=5 103.4 us (90 MB), C=6 97.3 us (75 MB), C=8 102.4 us (57 MB)
-//   B=32, K=8, V=151936 bf16:  C=6 70.7 us (88 MB), C=7 71.7 us (74 MB), C=8 75.8 us (67 MB)
-//   B=128, K=4, V=151936 fp32: C=12 207.9 us (84 MB), C=16 247.8 us (60 MB)
+// hold at most kRowL2Budget of rows.  us a step, rows in flight:
+//   B=64, K=7, V=128256 bf16 stochastic: C=4 78.6, C=5 76.9 (90 MB), C=6 73.1 (75 MB), C=7 74.2,
+//     C=8 75.2 (57 MB), C=10 79.4; greedy: C=4 69.5, C=5 68.6, C=6 66.2, C=7 66.8, C=8 68.4
+//   B=256, K=4, V=151936 fp32 stochastic: C=10 386, C=12 363 (84 MB), C=16 381 (60 MB)
 // Smaller batches take C = 8.  A warp's block takes at most kWalkRounds
 // steps (the decision kernel's draw takes one vector of a block per thread).  Only the
 // pass-1 records live in shared memory.  forced_C: the caller's

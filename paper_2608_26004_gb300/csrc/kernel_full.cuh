@@ -13,8 +13,7 @@
 //
 // decide_full, one CTA per row: the row's divergence and record; in
 // stochastic mode every row's draw (the row tokens report it); the last row
-// of an element runs Algorithm 1's scan (its ticket, as in the generic
-// kernel).
+// of an element runs Algorithm 1's scan (a counter that the row kernel clears).
 #pragma once
 
 #include "kernel_row.cuh"

@@ -1,6 +1,7 @@
-// Staged fuse-and-verify kernel for 16-byte aligned rows (every program
-// but the production ones, which fuse_verify_row in kernel_row.cuh runs), and
-// its decision kernel.
+// Staged fuse-and-verify kernel for 16-byte aligned rows, and its decision
+// kernel: the programs that the streaming kernels (kernel_row.cuh,
+// kernel_full.cuh) do not take (the row tokens alone, delta from another
+// source, more than 65535 batch elements) and calls that ask for it.
 //
 // One cluster of C CTAs per row triple (one launch of the cluster per row;
 // the hardware hands out rows as clusters finish).  CTA r owns vocabulary
