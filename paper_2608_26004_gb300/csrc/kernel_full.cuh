@@ -22,7 +22,7 @@ namespace asymspec_impl {
 
 constexpr int kFullMinBlocks = 3;  // CTAs per SM (85 registers a thread)
 
-// A warp's pass-1 record: the references (whole numbers, in log2 units) and
+// A warp's pass-1 record: the references (whole numbers, in log2 units; EDGE: nats) and
 // sums of 2^(x log2 e - ref) of a, b, t and s; the largest s and t and the lowest
 // vectors that hold them (INT_MAX: none; NaN: non-finite values were seen).
 struct __align__(16) WF {
@@ -76,13 +76,16 @@ __device__ __forceinline__ bool full_pass1(uint4* ring, const Streams<T>& g, int
     acc[q] = 0ull;
   }
   float bs = -INFINITY, bt = -INFINITY;
+  float ma = -INFINITY, mb = -INFINITY;  // EDGE: the largest values
   int rs = -1, rt = -1;
   ring_steps<T, true, true>(ring, g, v0, v1, [&](int r, const RawVec<T>& va, const RawVec<T>& vb,
                                                  const RawVec<T>& vt, auto) {
-    f2 sc[NP], tc[NP], e[4][NP];
+    f2 sc[NP], tc[NP], e[4][NP], xa[NP], xb[NP];
 #pragma unroll
     for (int h = 0; h < NP; ++h) {
       const f2 a2 = va.pair(h), b2 = vb.pair(h);
+      xa[h] = a2;
+      xb[h] = b2;
       tc[h] = vt.pair(h);
       sc[h] = fma2(beta2, sub2(a2, b2), tc[h]);
       e[0][h] = ex2_2(fma2(a2, L2, n2[0]));
@@ -92,6 +95,10 @@ __device__ __forceinline__ bool full_pass1(uint4* ring, const Streams<T>& g, int
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[q] = add2(acc[q], vsum2(e[q]));
+    if (EDGE) {
+      ma = max_nan(ma, vmax_nan(xa));
+      mb = max_nan(mb, vmax_nan(xb));
+    }
     // strictly larger wins, so the lane's earliest vector keeps a tie
     const float cs = vmax_nan(sc), ct = vmax_nan(tc);
     rs = cs > bs ? r : rs;
@@ -108,6 +115,8 @@ __device__ __forceinline__ bool full_pass1(uint4* ring, const Streams<T>& g, int
     if (ed.tail && ev[3] > bs) vs = lastvec;
     if (ed.head && (ev[2] >= bt || bt != bt) && ev[2] > -INFINITY) vt = 0;
     if (ed.tail && ev[2] > bt) vt = lastvec;
+    ma = max_nan(ma, ev[0]);
+    mb = max_nan(mb, ev[1]);
     if (ed.head || ed.tail) {
       bs = max_nan(bs, ev[3]);
       bt = max_nan(bt, ev[2]);
@@ -125,6 +134,11 @@ __device__ __forceinline__ bool full_pass1(uint4* ring, const Streams<T>& g, int
   for (int q = 0; q < 4; ++q) {
     e.ref[q] = ref[q];
     e.s[q] = s[q];
+  }
+  if (EDGE) {
+    const float m[4] = {ma, mb, bt, bs};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) to_largest(e.s[q], e.ref[q], warp_max(m[q]));
   }
   warp_best(bs, vs);
   warp_best(bt, vt);
@@ -168,14 +182,15 @@ __device__ __noinline__ void full_pass1_online(const Streams<T>& g, int v0, int 
   for (int q = 0; q < 4; ++q) {
     const float M = warp_max(m[q]);
     const float sc = (s[q] == 0.f || m[q] == M) ? s[q] : s[q] * ex2((m[q] - M) * kLog2e);
-    e.ref[q] = ref_of(M);
+    e.ref[q] = EDGE ? M : ref_of(M);
     e.s[q] = warp_sum(sc);
-    e.s[q] *= ref_residual(M, e.ref[q]);
+    if (!EDGE) e.s[q] *= ref_residual(M, e.ref[q]);
   }
 }
 
 // The row's pass-1 result from the cluster's warp records (combine_records,
 // four streams and two argmaxes).
+template <bool EDGE>
 __device__ __forceinline__ void combine_full(const WF* rec, int n, float (&lse)[4], float& vs,
                                              int& is, float& vt, int& it) {
   const int lane = static_cast<int>(threadIdx.x & 31);
@@ -199,14 +214,14 @@ __device__ __forceinline__ void combine_full(const WF* rec, int n, float (&lse)[
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float s = rec[i].s[q], r = rec[i].ref[q];
-      sum[q] += (s == 0.f || r == ref[q]) ? s : s * ex2(r - ref[q]);
+      sum[q] += (s == 0.f || r == ref[q]) ? s : s * ref_factor<EDGE>(r - ref[q]);
     }
     if (rec[i].vs == vs) is = min(is, rec[i].is);
     if (rec[i].vt == vt) it = min(it, rec[i].it);
   }
   warp_sum4(sum[0], sum[1], sum[2], sum[3]);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) lse[q] = lse_of(ref[q], sum[q]);
+  for (int q = 0; q < 4; ++q) lse[q] = record_lse<EDGE>(ref[q], sum[q]);
   is = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(is)));
   it = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(it)));
   if (__any_sync(0xffffffffu, bad_s)) vs = NAN;
@@ -351,7 +366,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
     got = mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
     float lse[4], vs, vt;
     int is, it;
-    combine_full(recv, nrec, lse, vs, is, vt, it);
+    combine_full<EDGE>(recv, nrec, lse, vs, is, vt, it);
     if (lane == 0) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) sh->lse[q] = lse[q];
@@ -406,7 +421,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
       jsum = row_jsd_wide<T, EDGE>(g, v0, v1, A2, B2, ed);
   }
   if (lane == 0) {
-    const float qf = STOCH && e.s[3] > 0.f ? e.s[3] * ex2(e.ref[3] - S2) : 0.f;
+    const float qf = STOCH && e.s[3] > 0.f ? e.s[3] * ex2(EDGE ? fmaf(e.ref[3], kLog2e, -S2) : e.ref[3] - S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

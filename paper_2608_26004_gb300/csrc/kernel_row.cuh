@@ -155,8 +155,8 @@ constexpr int kRowThreads = 256;  // threads per CTA of the row kernel
 constexpr int kRowMinBlocks = 4;  // CTAs per SM (64 registers a thread)
 static_assert(kRowThreads / 32 <= kRowMaxWarps, "one record slot per warp");
 
-// A warp's pass-1 record: the references (whole numbers, in log2 units) and
-// sums of 2^(x log2 e - ref) of a, b and the fused score (stochastic) or t
+// A warp's pass-1 record: the references (whole numbers, in log2 units; EDGE:
+// nats) and sums of 2^(x log2 e - ref) of a, b and the fused score (stochastic) or t
 // (greedy); greedy: the largest fused score (t on an unfused bonus row) and
 // the lowest vector of the row that holds it (INT_MAX: none; NaN: non-finite
 // scores were seen).
@@ -190,6 +190,33 @@ __device__ __forceinline__ float lse_of(float ref, float sum) {
   constexpr double kLn2d = 0.69314718055994530942;
   constexpr double hi = 2839.0 / 4096.0;
   return fmaf(n, static_cast<float>(hi), fmaf(n, static_cast<float>(kLn2d - hi), logf(m)));
+}
+
+// EDGE rows and the cross-family step, which the generic kernel also took: a
+// warp's sum s, against ref, restated against the warp's largest
+// value M (nats), whose term is taken out as it went in and put back as exactly
+// 1.  The first step's reference may lie far below an entry that holds most of
+// a row, whose exponent then carries a rounding of up to 5e-7 and whose ex2 its
+// own error.  RMS error of the LSEs against 64 bits, V = 16385 to 149173: 2.0e-7
+// without, 7.1e-8 with it and 8.3e-8 in the generic kernel, which references each
+// thread's maximum; B=32, K=4, V=100003 bf16 greedy 24.6 -> 25.4 us a step.
+__device__ __forceinline__ void to_largest(float& s, float& ref, float M) {
+  if (M > -INFINITY) {
+    const float y = fmaf(M, kLog2e, -ref), rest = s - ex2(y);
+    s = rest > 0.f ? fmaf(rest, ex2(-y), 1.f) : rest <= 0.f ? 1.f : NAN;
+  }
+  ref = M;
+}
+
+// Their records hold the references in nats, the others' in whole log2 units:
+// the factor between two references, and the LSE.
+template <bool NATS>
+__device__ __forceinline__ float ref_factor(float d) {
+  return ex2(NATS ? d * kLog2e : d);
+}
+template <bool NATS>
+__device__ __forceinline__ float record_lse(float ref, float sum) {
+  return NATS ? ref + logf(sum) : lse_of(ref, sum);
 }
 
 // What pass 2 does for a row (row_path): nothing, the residual masses alone,
@@ -474,24 +501,29 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
   const f2 nA2 = pk(nA, nA), nB2 = pk(nB, nB), n32 = pk(n3, n3);
   f2 acc_a = 0ull, acc_b = 0ull, acc_3 = 0ull, fin = 0ull;
   float best = -INFINITY;
+  float ma = -INFINITY, mb = -INFINITY, m3 = -INFINITY;  // EDGE: the largest values
   int rbest = -1;
   ring_steps<T, AB, true>(ring, g, v0, v1, [&](int r, const RawVec<T>& va, const RawVec<T>& vb,
                                                const RawVec<T>& vt, auto) {
-    f2 sc[NP];  // the argmax's scores
-    f2 ea[NP], eb[NP], e3[NP];
+    f2 sc[NP];  // the argmax's scores (EDGE, stochastic: the summed scores)
+    f2 ea[NP], eb[NP], e3[NP], xa[NP], xb[NP], xt[NP];
 #pragma unroll
     for (int h = 0; h < NP; ++h) {
       const f2 t2 = vt.pair(h);
+      xt[h] = t2;
       if (AB) {
         const f2 a2 = va.pair(h), b2 = vb.pair(h);
         const f2 amb = sub2(a2, b2);
+        xa[h] = a2;
+        xb[h] = b2;
         if (DRAFT) {
           ea[h] = ex2_2(fma2(a2, L2, nA2));
           eb[h] = ex2_2(fma2(b2, L2, nB2));
           fin = fma2(amb, 0ull, fin);  // 0 x (non-finite) is NaN
         }
-        if (STOCH) e3[h] = ex2_2(fma2(t2, L2, fma2(bL2, amb, n32)));
-        if (ARG) sc[h] = fma2(beta2, amb, t2);
+        if (STOCH && !EDGE) e3[h] = ex2_2(fma2(t2, L2, fma2(bL2, amb, n32)));
+        if (ARG || EDGE) sc[h] = fma2(beta2, amb, t2);
+        if (STOCH && EDGE) e3[h] = ex2_2(fma2(sc[h], L2, n32));
       } else {
         sc[h] = t2;
       }
@@ -504,6 +536,13 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
       acc_b = add2(acc_b, vsum2(eb));
     }
     if (SUM3) acc_3 = add2(acc_3, vsum2(e3));
+    if (EDGE) {
+      if (DRAFT) {
+        ma = max_nan(ma, vmax_nan(xa));
+        mb = max_nan(mb, vmax_nan(xb));
+      }
+      if (SUM3) m3 = max_nan(m3, STOCH ? vmax_nan(sc) : vmax_nan(xt));
+    }
     if (ARG) {
       // strictly larger wins, so the lane's earliest vector keeps a tie
       const float c = vmax_nan(sc);
@@ -518,8 +557,11 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
       acc_b = add2(acc_b, pk(ex2(fmaf(ed.b, kLog2e, nB)), 0.f));
       fin = fma2(pk(amb, 0.f), 0ull, fin);
     }
-    if (STOCH) acc_3 = add2(acc_3, pk(ex2(fmaf(ed.t, kLog2e, fmaf(bl, amb, n3))), 0.f));
-    else if (SUM3) acc_3 = add2(acc_3, pk(ex2(fmaf(ed.t, kLog2e, n3)), 0.f));
+    const float x3 = STOCH ? se : ed.t;
+    if (SUM3) acc_3 = add2(acc_3, pk(ex2(fmaf(x3, kLog2e, n3)), 0.f));
+    ma = max_nan(ma, ed.a);
+    mb = max_nan(mb, ed.b);
+    m3 = max_nan(m3, x3);
   }
   bool ovf = false;
   e.ref[0] = ra0;
@@ -534,6 +576,13 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
     e.s[0] = sa;
     e.s[1] = sb;
     e.s[2] = s3;
+    if (EDGE) {
+      if (DRAFT) {
+        to_largest(e.s[0], e.ref[0], warp_max(ma));
+        to_largest(e.s[1], e.ref[1], warp_max(mb));
+      }
+      to_largest(e.s[2], e.ref[2], warp_max(m3));
+    }
   } else {
     e.s[0] = e.s[1] = e.s[2] = 0.f;
   }
@@ -605,9 +654,9 @@ __device__ __noinline__ void row_pass1_online(const Streams<T>& g, int v0, int v
     const float M = warp_max(m[q]);
     float sc = (s[q] == 0.f || m[q] == M) ? s[q] : s[q] * ex2((m[q] - M) * kLog2e);
     if (q == 0 && DRAFT && chk) sc += fin;  // 0, or NaN
-    e.ref[q] = ref_of(M);
+    e.ref[q] = EDGE ? M : ref_of(M);
     e.s[q] = warp_sum(sc);
-    e.s[q] *= ref_residual(M, e.ref[q]);
+    if (!EDGE) e.s[q] *= ref_residual(M, e.ref[q]);
   }
   if (!DRAFT) {
     e.ref[0] = e.ref[1] = -INFINITY;
@@ -713,6 +762,7 @@ __device__ __forceinline__ void cluster_wait() {
 // against it, the sums added; the largest score and its lowest vector.
 // Every lane ends with the same (bit-identical) result, and so does every
 // CTA, whose records are the same.
+template <bool NATS>
 __device__ __forceinline__ void combine_records(const W1* rec, int n, float (&ref)[3],
                                                 float (&sum)[3], float& v, int& vec) {
   const int lane = static_cast<int>(threadIdx.x & 31);
@@ -738,7 +788,7 @@ __device__ __forceinline__ void combine_records(const W1* rec, int n, float (&re
     const W1 r = rec[i];
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-      sum[q] += (r.s[q] == 0.f || r.ref[q] == ref[q]) ? r.s[q] : r.s[q] * ex2(r.ref[q] - ref[q]);
+      sum[q] += (r.s[q] == 0.f || r.ref[q] == ref[q]) ? r.s[q] : r.s[q] * ref_factor<NATS>(r.ref[q] - ref[q]);
     if (r.v == v) lo = min(lo, r.vec);
   }
   float z = 0.f;
@@ -911,12 +961,12 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
     got = mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
     float ref[3], sum[3], v;
     int vec;
-    combine_records(sh->recv(), nrec, ref, sum, v, vec);
+    combine_records<EDGE>(sh->recv(), nrec, ref, sum, v, vec);
     float lse[4];
-    lse[0] = draft ? lse_of(ref[0], sum[0]) : NAN;
-    lse[1] = draft ? lse_of(ref[1], sum[1]) : NAN;
-    lse[2] = !STOCH && draft ? lse_of(ref[2], sum[2]) : NAN;
-    lse[3] = STOCH ? lse_of(ref[2], sum[2]) : NAN;
+    lse[0] = draft ? record_lse<EDGE>(ref[0], sum[0]) : NAN;
+    lse[1] = draft ? record_lse<EDGE>(ref[1], sum[1]) : NAN;
+    lse[2] = !STOCH && draft ? record_lse<EDGE>(ref[2], sum[2]) : NAN;
+    lse[3] = STOCH ? record_lse<EDGE>(ref[2], sum[2]) : NAN;
     // (a token outside the vocabulary voids the element whatever the row does)
     const int path = draft && tok_ok ? row_path<STOCH>(P, lse, da, db, dt, u, pd) : kPathAccept;
     if (lane == 0) {
@@ -975,7 +1025,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
     // this warp's record: its block is one inverse-CDF group of the row.  The
     // fused mass (the bonus row's draw, and a draft row's where the row's
     // whole residual is zero) comes from the warp's pass-1 sum.
-    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(e.ref[2] - S2) : 0.f;
+    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(EDGE ? fmaf(e.ref[2], kLog2e, -S2) : e.ref[2] - S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

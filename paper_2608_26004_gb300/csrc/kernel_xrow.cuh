@@ -136,8 +136,7 @@ __device__ __forceinline__ bool x_pass1(const XSlice<T>& x, int p0, int p1, floa
   constexpr bool SUM3 = PROG == kStochDraft || PROG == kStochBonus || PROG == kGreedyDraft;
   constexpr bool ARG = !STOCH;
   const f2 L2 = pk(kLog2e, kLog2e);
-  const float bl = beta * kLog2e;
-  const f2 bL2 = pk(bl, bl), beta2 = pk(beta, beta);
+  const f2 beta2 = pk(beta, beta);
   float ra0 = -INFINITY, rb0 = -INFINITY, r30 = -INFINITY;
   const int jf = p0 + static_cast<int>(threadIdx.x & 31);  // any pairs do as references
   if (SUM3 && jf < p1) {
@@ -161,6 +160,7 @@ __device__ __forceinline__ bool x_pass1(const XSlice<T>& x, int p0, int p1, floa
   const f2 nA2 = pk(nA, nA), nB2 = pk(nB, nB), n32 = pk(n3, n3);
   f2 acc_a = 0ull, acc_b = 0ull, acc_3 = 0ull, fin = 0ull;
   float best = -INFINITY;
+  float ma = -INFINITY, mb = -INFINITY, m3 = -INFINITY;  // the largest values (to_largest)
   int jbest = INT_MAX;
   pair_steps<T, AB>(x, p0, p1, [&](int j, f2 a2, f2 b2, f2 t2) {
     f2 sc = t2;
@@ -170,11 +170,16 @@ __device__ __forceinline__ bool x_pass1(const XSlice<T>& x, int p0, int p1, floa
         acc_a = add2(acc_a, ex2_2(fma2(a2, L2, nA2)));
         acc_b = add2(acc_b, ex2_2(fma2(b2, L2, nB2)));
         fin = fma2(amb, 0ull, fin);  // 0 x (non-finite) is NaN
+        ma = max3_nan(ma, lo_of(a2), hi_of(a2));
+        mb = max3_nan(mb, lo_of(b2), hi_of(b2));
       }
-      if (STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, fma2(bL2, amb, n32))));
-      if (ARG) sc = fma2(beta2, amb, t2);
+      sc = fma2(beta2, amb, t2);
     }
-    if (SUM3 && !STOCH) acc_3 = add2(acc_3, ex2_2(fma2(t2, L2, n32)));
+    if (SUM3) {
+      const f2 x3 = STOCH ? sc : t2;
+      acc_3 = add2(acc_3, ex2_2(fma2(x3, L2, n32)));
+      m3 = max3_nan(m3, lo_of(x3), hi_of(x3));
+    }
     if (ARG) {
       // strictly larger wins, so the lane's earliest pair keeps a tie
       jbest = lo_of(sc) > best ? j : jbest;
@@ -197,6 +202,11 @@ __device__ __forceinline__ bool x_pass1(const XSlice<T>& x, int p0, int p1, floa
     e.s[0] = sa;
     e.s[1] = sb;
     e.s[2] = s3;
+    if (DRAFT) {
+      to_largest(e.s[0], e.ref[0], warp_max(ma));
+      to_largest(e.s[1], e.ref[1], warp_max(mb));
+    }
+    to_largest(e.s[2], e.ref[2], warp_max(m3));
   }
   e.v = 0.f;
   e.vec = 0;
@@ -239,9 +249,8 @@ __device__ __noinline__ void x_pass1_online(const XSlice<T>& x, int p0, int p1, 
     const float M = warp_max(m[q]);
     float sc = (s[q] == 0.f || m[q] == M) ? s[q] : s[q] * ex2((m[q] - M) * kLog2e);
     if (q == 0 && DRAFT && chk) sc += fin;  // 0, or NaN
-    e.ref[q] = ref_of(M);
+    e.ref[q] = M;
     e.s[q] = warp_sum(sc);
-    e.s[q] *= ref_residual(M, e.ref[q]);
   }
   if (!DRAFT) {
     e.ref[0] = e.ref[1] = -INFINITY;
@@ -451,12 +460,12 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
     got = mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
     float ref[3], sum[3], v;
     int vec;
-    combine_records(sh->recv(), nrec, ref, sum, v, vec);
+    combine_records<true>(sh->recv(), nrec, ref, sum, v, vec);
     float lse[4];
-    lse[0] = draft ? lse_of(ref[0], sum[0]) : NAN;
-    lse[1] = draft ? lse_of(ref[1], sum[1]) : NAN;
-    lse[2] = !STOCH && draft ? lse_of(ref[2], sum[2]) : NAN;
-    lse[3] = STOCH ? lse_of(ref[2], sum[2]) : NAN;
+    lse[0] = draft ? record_lse<true>(ref[0], sum[0]) : NAN;
+    lse[1] = draft ? record_lse<true>(ref[1], sum[1]) : NAN;
+    lse[2] = !STOCH && draft ? record_lse<true>(ref[2], sum[2]) : NAN;
+    lse[3] = STOCH ? record_lse<true>(ref[2], sum[2]) : NAN;
     const int path = draft && tok_ok ? row_path<STOCH>(P, lse, da, db, dt, u, pd) : kPathAccept;
     if (lane == 0) {
 #pragma unroll
@@ -489,7 +498,7 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
       jsum = x_jsd_wide<T>(x, p0, p1, A2, B2);
   }
   if (lane == 0 && (second || (STOCH && !draft))) {
-    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(e.ref[2] - S2) : 0.f;
+    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(fmaf(e.ref[2], kLog2e, -S2)) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + (static_cast<size_t>(row32) * nrec + rank * NW + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

@@ -271,3 +271,27 @@ def test_batches_of_several_sizes_share_a_workspace(torch, mode, first, second):
         want = run_gpu(batch, torch, mode=mode, full=recorded, tokens=recorded, logprobs=False)
         for name in ("accept_len", "next_token"):
             np.testing.assert_array_equal(res[name].cpu().numpy(), want[name])
+
+
+@pytest.mark.parametrize("dtype", [synth.BF16, synth.FP32])
+def test_a_token_that_holds_the_row_beside_a_low_reference(torch, dtype):
+    # One entry M near 0 anywhere in a row of -14: the warp's first step mostly
+    # sees the -14s.  What may round after M's term has entered the sum, each time
+    # relative to the whole sum: 3 steps of its block, 2 additions in its vector
+    # and 1 in its pair, 5 of the warp, 7 of the cluster's records, then the
+    # logarithm and the addition of M: 20 roundings, uniform within 2^-24, 3.4e-8
+    # RMS each and 1.6e-7 together.  (Not a bound on the largest error, for which
+    # the 20 may add up to 1.2e-6; M's exponent against a reference of -14, 20 log2
+    # units, rounds by 2.8e-7 RMS on its own.)
+    B, K, V = 24, 3, 33333
+    gen = torch.Generator().manual_seed(5)
+    dt = torch.float32 if dtype == synth.FP32 else torch.bfloat16
+    x = torch.full((3, B, K + 1, V), -14.0)
+    at = torch.randint(V, (3, B, K + 1, 1), generator=gen)
+    x.scatter_(-1, at, torch.rand(at.shape, generator=gen) * 1.4 - 0.7)
+    a, b, t = x.to(dt).cuda()
+    tokens = torch.zeros(B, K, dtype=torch.int32, device="cuda")
+    res = A.FuseVerify(B, K)(a, b, t, tokens, row_stats=True)
+    stats = res["row_stats"].double()
+    err = torch.stack([stats[..., q] - z.double().logsumexp(-1) for q, z in enumerate((a, b, t))])
+    assert err.square().mean().sqrt().item() <= 1.6e-7
