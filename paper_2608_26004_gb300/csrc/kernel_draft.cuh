@@ -142,7 +142,7 @@ struct DRow {
 
 // A partial vector: its elements inside the row, the others the type's lowest.
 template <bool EDGE>
-__device__ __noinline__ DRaw<__nv_bfloat16> dld_edge(const DRow<__nv_bfloat16, EDGE>& r, int v) {
+__device__ __noinline__ DRaw<__nv_bfloat16> dld_edge(DRow<__nv_bfloat16, EDGE> r, int v) {
   const unsigned short* p = reinterpret_cast<const unsigned short*>(r.base) + static_cast<long long>(v) * 8;
   unsigned w[4];
 #pragma unroll
@@ -154,7 +154,7 @@ __device__ __noinline__ DRaw<__nv_bfloat16> dld_edge(const DRow<__nv_bfloat16, E
   return {make_uint4(w[0], w[1], w[2], w[3])};
 }
 template <bool EDGE>
-__device__ __noinline__ DRaw<float> dld_edge(const DRow<float, EDGE>& r, int v) {
+__device__ __noinline__ DRaw<float> dld_edge(DRow<float, EDGE> r, int v) {
   const float* p = r.base + static_cast<long long>(v) * 4;
   float x[4];
 #pragma unroll

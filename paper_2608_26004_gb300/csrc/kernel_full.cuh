@@ -151,8 +151,8 @@ __device__ __forceinline__ bool full_pass1(uint4* ring, const Streams<T>& g, int
 
 // Fallback of full_pass1's sums, as row_pass1_online.
 template <typename T, bool EDGE>
-__device__ __noinline__ void full_pass1_online(const Streams<T>& g, int v0, int v1, float beta,
-                                               const EdgeVals& ed, WF& e) {
+__device__ __noinline__ WF full_pass1_online(Streams<T> g, int v0, int v1, float beta, EdgeVals ed,
+                                             WF e) {
   constexpr int NP = RawVec<T>::NP;
   constexpr int VE = 2 * NP;
   float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -186,6 +186,7 @@ __device__ __noinline__ void full_pass1_online(const Streams<T>& g, int v0, int 
     e.s[q] = warp_sum(sc);
     if (!EDGE) e.s[q] *= ref_residual(M, e.ref[q]);
   }
+  return e;
 }
 
 // The row's pass-1 result from the cluster's warp records (combine_records,
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
 
   WF e;
   const bool ovf = full_pass1<T, EDGE>(ring, g, v0, v1, P.beta, ed, s0 + i0, cut.nvec - 1, e);
-  if (__any_sync(0xffffffffu, ovf)) full_pass1_online<T, EDGE>(g, v0, v1, P.beta, ed, e);
+  if (__any_sync(0xffffffffu, ovf)) e = full_pass1_online<T, EDGE>(g, v0, v1, P.beta, ed, e);
   cp_async_wait<0>();
   // pass 2's first steps do not depend on the normalisers
   const bool jsd = P.divergence == ASYMSPEC_DIV_JSD, kl = P.divergence == ASYMSPEC_DIV_KL;

@@ -608,10 +608,14 @@ __device__ __forceinline__ bool row_pass1(uint4* ring, const Streams<T>& g, int 
 // Fallback of row_pass1's sums (a sum reached 2^100, or non-finite data):
 // each lane keeps a running maximum per stream over its vectors of the
 // warp's block, rescaling its sum when the maximum rises; the lanes then
-// merge.  The record's argmax stays as row_pass1 left it.
+// merge.  The record's argmax stays as row_pass1 left it.  (Called out of
+// line, so everything travels by value: a reference keeps the caller's record
+// and pointers in local memory for every warp, 20 MB of stores a launch at
+// B=64, K=7, V=128256 that reach HBM: stochastic 72.1 us a step against 66.4,
+// greedy 64.2 against 59.8, B=256, K=4, V=151936 fp32 367 against 332.)
 template <typename T, int PROG, bool EDGE>
-__device__ __noinline__ void row_pass1_online(const Streams<T>& g, int v0, int v1, float beta,
-                                              bool chk, const EdgeVals& ed, W1& e) {
+__device__ __noinline__ W1 row_pass1_online(Streams<T> g, int v0, int v1, float beta, bool chk,
+                                            EdgeVals ed, W1 e) {
   constexpr int NP = RawVec<T>::NP;
   constexpr int VE = 2 * NP;
   constexpr bool DRAFT = prog_draft(PROG);
@@ -662,6 +666,7 @@ __device__ __noinline__ void row_pass1_online(const Streams<T>& g, int v0, int v
     e.ref[0] = e.ref[1] = -INFINITY;
     e.s[0] = e.s[1] = 0.f;
   }
+  return e;
 }
 
 // ---------------------------------------------------------------- pass 2
@@ -710,8 +715,8 @@ __device__ __forceinline__ void row_pass2(uint4* ring, const Streams<T>& g, int 
 // exponents, an entry of no mass contributing nothing.  NaN where a or b is
 // not finite.
 template <typename T, bool EDGE>
-__device__ __noinline__ float row_jsd_wide(const Streams<T>& g, int v0, int v1, float A2, float B2,
-                                           const EdgeVals& ed) {
+__device__ __noinline__ float row_jsd_wide(Streams<T> g, int v0, int v1, float A2, float B2,
+                                           EdgeVals ed) {
   constexpr int NP = RawVec<T>::NP;
   constexpr int VE = 2 * NP;
   float j = 0.f;
@@ -918,7 +923,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
     if (PROG != kGreedyBonusT && PROG != kGreedyBonusS && __any_sync(0xffffffffu, ovf)) {
       // an entry far above the warp's reference (or non-finite data): redo
       // the block with running maxima
-      row_pass1_online<T, PROG, EDGE>(g, v0, v1, P.beta, chk, ed, e);
+      e = row_pass1_online<T, PROG, EDGE>(g, v0, v1, P.beta, chk, ed, e);
     }
   };
   if (STOCH) {

@@ -222,8 +222,7 @@ __device__ __forceinline__ bool x_pass1(const XSlice<T>& x, int p0, int p1, floa
 
 // Fallback of x_pass1's sums, as row_pass1_online.
 template <typename T, int PROG>
-__device__ __noinline__ void x_pass1_online(const XSlice<T>& x, int p0, int p1, float beta, bool chk,
-                                            W1& e) {
+__device__ __noinline__ W1 x_pass1_online(XSlice<T> x, int p0, int p1, float beta, bool chk, W1 e) {
   constexpr bool DRAFT = prog_draft(PROG);
   constexpr bool STOCH = PROG == kStochDraft || PROG == kStochBonus;
   float m[3] = {-INFINITY, -INFINITY, -INFINITY}, s[3] = {0.f, 0.f, 0.f}, fin = 0.f;
@@ -256,6 +255,7 @@ __device__ __noinline__ void x_pass1_online(const XSlice<T>& x, int p0, int p1, 
     e.ref[0] = e.ref[1] = -INFINITY;
     e.s[0] = e.s[1] = 0.f;
   }
+  return e;
 }
 
 // Pass 2 over the warp's pairs, as row_pass2.
@@ -285,7 +285,7 @@ __device__ __forceinline__ void x_pass2(const XSlice<T>& x, int p0, int p1, cons
 
 // The warp's JSD sum term by term, as row_jsd_wide.
 template <typename T>
-__device__ __noinline__ float x_jsd_wide(const XSlice<T>& x, int p0, int p1, float A2, float B2) {
+__device__ __noinline__ float x_jsd_wide(XSlice<T> x, int p0, int p1, float A2, float B2) {
   float j = 0.f;
   for (int i = p0 + static_cast<int>(threadIdx.x & 31); i < p1; i += 32) {
     const int d = __ldg(x.map_d + i);
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
     constexpr int PROG = decltype(prog)::value;
     const bool ovf = x_pass1<T, PROG>(x, p0, p1, P.beta, chk, e);
     if (PROG != kGreedyBonusT && PROG != kGreedyBonusS && __any_sync(0xffffffffu, ovf))
-      x_pass1_online<T, PROG>(x, p0, p1, P.beta, chk, e);
+      e = x_pass1_online<T, PROG>(x, p0, p1, P.beta, chk, e);
   };
   if (STOCH) {
     if (draft) pass1(std::integral_constant<int, kStochDraft>{});
