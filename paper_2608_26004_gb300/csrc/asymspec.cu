@@ -127,9 +127,9 @@ bool plan_tma(int V, int elt, int forced_C, Plan* pl) {
 // records) are spread.  With at least one wave of clusters of 8 (rows x 8 >=
 // 4 CTAs x SMs): the smallest C of kRowClusters whose resident clusters
 // hold at most kRowL2Budget of rows.  us a step, rows in flight:
-//   B=64, K=7, V=128256 bf16 stochastic: C=4 78.6, C=5 76.9 (90 MB), C=6 73.1 (75 MB), C=7 74.2,
-//     C=8 75.2 (57 MB), C=10 79.4; greedy: C=4 69.5, C=5 68.6, C=6 66.2, C=7 66.8, C=8 68.4
-//   B=256, K=4, V=151936 fp32 stochastic: C=10 386, C=12 363 (84 MB), C=16 381 (60 MB)
+//   B=64, K=7, V=128256 bf16 stochastic: C=4 70.8, C=5 67.9 (90 MB), C=6 66.5 (75 MB), C=7 67.8,
+//     C=8 69.0 (57 MB), C=10 73.6; greedy: C=4 62.1, C=5 60.8, C=6 60.6, C=7 60.8, C=8 62.6
+//   B=256, K=4, V=151936 fp32 stochastic: C=10 347, C=12 332 (84 MB), C=16 351 (60 MB)
 // Smaller batches take C = 8.  A warp's block takes at most kWalkRounds
 // steps (the decision kernel's draw takes one vector of a block per thread).  Only the
 // pass-1 records live in shared memory.  forced_C: the caller's
@@ -323,7 +323,7 @@ int make_plan(int B, int K, int V, int dtype, const asymspec_launch_opts* opts, 
   bool ok = false;
   // (decide_full's grid is (K+1, B): B up to 65535)
   // Greedy and recorded steps stream too (B=64, K=7, V=128256 bf16 greedy:
-  // 114 us of staged kernel against 65 us; B=8, K=5, V=151936 bf16 greedy with
+  // 114 us of staged kernel against 59 us; B=8, K=5, V=151936 bf16 greedy with
   // every row recorded: 48 us a step against 28).  The staged kernel's copy waits are
   // what the test hook shortens, so such calls that set it, or ask for
   // ASYMSPEC_KERNEL_TMA, keep the staged kernel.
