@@ -126,10 +126,16 @@ bool plan_tma(int V, int elt, int forced_C, Plan* pl) {
 // costs of a CTA (its launch, the first loads, the exchange of the pass-1
 // records) are spread.  With at least one wave of clusters of 8 (rows x 8 >=
 // 4 CTAs x SMs): the smallest C of kRowClusters whose resident clusters
-// hold at most kRowL2Budget of rows.  us a step, rows in flight:
+// hold at most kRowL2Budget of rows and whose CTAs fill the chip.  us a step,
+// rows in flight:
 //   B=64, K=7, V=128256 bf16 stochastic: C=4 70.8, C=5 67.9 (90 MB), C=6 66.5 (75 MB), C=7 67.8,
 //     C=8 69.0 (57 MB), C=10 73.6; greedy: C=4 62.1, C=5 60.8, C=6 60.6, C=7 60.8, C=8 62.6
 //   B=256, K=4, V=151936 fp32 stochastic: C=10 347, C=12 332 (84 MB), C=16 351 (60 MB)
+//   too few CTAs for the chip against enough, K=4, stochastic / greedy: V=128256 bf16 B=16 C=4
+//     23.3 / 16.9, C=8 20.6 / 16.5; B=19 C=4 23.8 / 20.2, C=7 21.7 / 18.3; B=22 C=4 25.6 / 22.0,
+//     C=6 23.1 / 20.5; V=64000 fp32 B=16 19.6 / 15.3, 18.2 / 14.9 and (the worst of 20) B=22
+//     C=4 22.8 / 18.0, C=6 23.5 / 18.6
+// (The recording kernel is not held to that: B=12, K=4, V=128256 bf16 greedy C=4 26.6, C=8 30.1.)
 // Smaller batches take C = 8.  A warp's block takes at most kWalkRounds
 // steps (the decision kernel's draw takes one vector of a block per thread).  Only the
 // pass-1 records live in shared memory.  forced_C: the caller's
@@ -183,7 +189,7 @@ bool plan_row(int V, int dtype, bool stoch, bool edge, bool full, int forced_C, 
       const void* fn = row_kernel(dtype, stoch, edge, full);
       const bool query = dev.ok && prepare_kernel(fn, dev.device) == cudaSuccess;
       for (int c : kRowClusters) {
-        if (!fits(c)) continue;
+        if (!fits(c) || (!full && rows * c < slots)) continue;
         // the clusters the device holds at once (an estimate without a device)
         long long resident = slots / c;
         Plan q = *pl;
