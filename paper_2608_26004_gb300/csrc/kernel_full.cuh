@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
   const RowCut<T, EDGE> cut(P, row32);
   const int Wv = P.W / VE, s0 = rank * Wv;  // the slice: vectors [s0, s0 + nv) of the row
   const int nv = max(0, min(Wv, cut.nvec - s0));
-  const int bw = row_block_vectors(nv, NW);
-  const int b0 = min(nv, warp * bw), b1 = min(nv, b0 + bw);
+  int b0, b1;  // the warp's block of the slice
+  row_block<!EDGE>(s0, nv, warp, b0, b1);
   const int v0 = EDGE ? max(b0, cut.in0 - s0) : b0;
   const int v1 = EDGE ? max(v0, min(b1, cut.in1 - s0)) : b1;
   const int i0 = v0 + lane;
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(STOCH ? kDrawThreads : 32) decide_full(const K
   }
   if constexpr (STOCH) {
     __syncthreads();
-    rr.sample = block_draw<T, EDGE>(P, row, sdraw, slse[0] * kLog2e, slse[1] * kLog2e);
+    rr.sample = block_draw<T, EDGE, !EDGE>(P, row, sdraw, slse[0] * kLog2e, slse[1] * kLog2e);
   }
   if (warp == 0)
     finish_row_warp<STOCH>(P, row, bi, k, rr, din.dtok, din.ad, din.bd, din.td, din.sc);

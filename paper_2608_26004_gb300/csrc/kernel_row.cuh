@@ -155,6 +155,28 @@ constexpr int kRowThreads = 256;  // threads per CTA of the row kernel
 constexpr int kRowMinBlocks = 4;  // CTAs per SM (64 registers a thread)
 static_assert(kRowThreads / 32 <= kRowMaxWarps, "one record slot per warp");
 
+// The block [b0, b1) of warp w in the slice of nv vectors that starts at the
+// row's vector s0: equal parts.  LINES (the recording kernel's aligned rows):
+// parts that start on the row's 128-byte lines, so that a step's 512 bytes lie in
+// four lines and not five, but for blocks of almost the most vectors a draw
+// takes, which are cut anywhere.  Recorded, greedy, V=128256 bf16: B=8, K=4 21.9 -> 20.1 us, B=64, K=7
+// 145.9 -> 139.3; V=64000 fp32 B=64, K=7 108.6 -> 107.5 (the worst of 16: B=20, K=5
+// stochastic 39.6 -> 39.9).  (fuse_verify_row's
+// blocks stay equal: lines took B=64, K=7 stochastic from 66.9 to 67.5.)
+template <bool LINES>
+__device__ __forceinline__ void row_block(int s0, int nv, int w, int& b0, int& b1) {
+  constexpr int NW = kRowThreads / 32;
+  const int part = row_block_vectors(nv, NW);
+  if (LINES && part <= kWalkRounds * 32 - 8) {
+    const int off = s0 & 7, bw = (row_block_vectors(nv + off, NW) + 7) & ~7;
+    b0 = min(nv, max(0, w * bw - off));
+    b1 = min(nv, max(0, (w + 1) * bw - off));
+  } else {
+    b0 = min(nv, w * part);
+    b1 = min(nv, b0 + part);
+  }
+}
+
 // A warp's pass-1 record: the references (whole numbers, in log2 units; EDGE:
 // nats) and sums of 2^(x log2 e - ref) of a, b and the fused score (stochastic) or t
 // (greedy); greedy: the largest fused score (t on an unfused bonus row) and
@@ -881,8 +903,8 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
   const RowCut<T, EDGE> cut(P, row32);
   const int Wv = P.W / VE, s0 = rank * Wv;  // the slice: vectors [s0, s0 + nv) of the row
   const int nv = max(0, min(Wv, cut.nvec - s0));
-  const int bw = row_block_vectors(nv, NW);
-  const int b0 = min(nv, warp * bw), b1 = min(nv, b0 + bw);
+  int b0, b1;  // the warp's block of the slice
+  row_block<false>(s0, nv, warp, b0, b1);
   // the block's whole vectors [v0, v1)
   const int v0 = EDGE ? max(b0, cut.in0 - s0) : b0;
   const int v1 = EDGE ? max(v0, min(b1, cut.in1 - s0)) : b1;
@@ -1244,7 +1266,7 @@ __device__ __forceinline__ int block_pick(const f2 (&m2)[NP], const Draw& dr) {
 // The row's draw: the masses of the group's vectors, one per thread, formed
 // exactly as the row kernel forms them; every thread returns the token (-1:
 // no mass).
-template <typename T, bool EDGE>
+template <typename T, bool EDGE, bool LINES = false>
 __device__ __forceinline__ int block_draw(const KParams& P, long long row, const Draw& dr, float A2,
                                           float S2) {
   constexpr int VE = 16 / static_cast<int>(sizeof(T));
@@ -1252,8 +1274,10 @@ __device__ __forceinline__ int block_draw(const KParams& P, long long row, const
   constexpr int NW = kRowThreads / 32;
   const RowCut<T, EDGE> cut(P, row);
   const int Wv = P.W / VE, rk = max(dr.g, 0) / NW, w = max(dr.g, 0) - rk * NW;
-  const int s0 = rk * Wv, nv = max(0, min(Wv, cut.nvec - s0)), bw = row_block_vectors(nv, NW);
-  const int g0 = s0 + min(nv, w * bw), g1 = s0 + min(nv, w * bw + bw);
+  const int s0 = rk * Wv, nv = max(0, min(Wv, cut.nvec - s0));
+  int b0, b1;
+  row_block<LINES>(s0, nv, w, b0, b1);
+  const int g0 = s0 + b0, g1 = s0 + b1;
   const int i = g0 + static_cast<int>(threadIdx.x);  // this thread's vector of the row
   const ResConst kc = res_const(P.beta, A2, 0.f, S2);
   f2 m2[NP];

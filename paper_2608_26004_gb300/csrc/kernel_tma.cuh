@@ -1153,9 +1153,7 @@ __device__ __noinline__ int group_walk(const T* ga, const T* gb, const T* gt, in
   return __shfl_sync(0xffffffffu, found, vc);
 }
 
-// The block of warp w in fuse_verify_row (kernel_row.cuh): vectors
-// [w bw, min(nv, (w + 1) bw)) of the slice, bw = ceil(nv / NW); the warp's
-// lane l takes vector w bw + 32 r + l in step r.
+// Vectors in a warp's block when nw warps share nv (kernel_row.cuh: row_block).
 __host__ __device__ __forceinline__ int row_block_vectors(int nv, int nw) {
   return (nv + nw - 1) / nw;
 }

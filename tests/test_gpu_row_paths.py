@@ -295,3 +295,18 @@ def test_a_token_that_holds_the_row_beside_a_low_reference(torch, dtype):
     stats = res["row_stats"].double()
     err = torch.stack([stats[..., q] - z.double().logsumexp(-1) for q, z in enumerate((a, b, t))])
     assert err.square().mean().sqrt().item() <= 1.6e-7
+
+
+@pytest.mark.parametrize("mode", [GREEDY, STOCH])
+@pytest.mark.parametrize("V,cluster", [
+    # vectors a CTA and where its slice starts in a line: one line and less,
+    (8 * 8, 1), (8 * 9, 1), (8 * 67, 2),
+    # slices that start off the lines,
+    (8 * 1001, 3), (8 * 4001, 6),
+    # and blocks of the last size cut on lines (504 vectors), one more, the largest
+    (8 * 4032, 1), (8 * 4033, 1), (8 * 4096, 1),
+])
+def test_recorded_rows_in_blocks_cut_on_lines(torch, V, cluster, mode):
+    batch = synth.generate(synth.Recipe(), 11, 3, 2, V, synth.BF16)
+    g = run_gpu(batch, torch, mode=mode, cluster_size=cluster)
+    compare(batch, g, run_oracle(batch, mode=mode), mode=mode)
