@@ -303,7 +303,10 @@ __device__ __noinline__ float x_jsd_wide(XSlice<T> x, int p0, int p1, float A2, 
 // t'_j = t[map_v[j]] for the slice's pairs, by the CTA: the verifier's row and
 // the inverse map in index order, U vectors of each in flight per thread.  A
 // map that passed the check gives every pair a distinct token, so every entry
-// is written.
+// is written.  (The inverse map is read with __ldcg: the map check writes it
+// while this kernel, its programmatic dependent, is already resident, and a
+// read-only load (__ldg) is defined only for memory that nothing writes during
+// the kernel.)
 template <typename T>
 __device__ __forceinline__ void build_t(const XRowParams& X, const T* src, T* out, int j0, int n) {
   constexpr int VE = 16 / static_cast<int>(sizeof(T));
@@ -325,7 +328,7 @@ __device__ __forceinline__ void build_t(const XRowParams& X, const T* src, T* ou
           v[q] = __ldg(reinterpret_cast<const uint4*>(src) + i);
 #pragma unroll
           for (int h = 0; h < VE / 4; ++h)
-            jv[q][h] = __ldg(reinterpret_cast<const int4*>(X.inv_v) + i * (VE / 4) + h);
+            jv[q][h] = __ldcg(reinterpret_cast<const int4*>(X.inv_v) + i * (VE / 4) + h);
         }
       }
 #pragma unroll
@@ -350,7 +353,7 @@ __device__ __forceinline__ void build_t(const XRowParams& X, const T* src, T* ou
         j[q] = -1;
         if (u0 + q * NT < X.V_v) {
           v[q] = src[u0 + q * NT];
-          j[q] = __ldg(X.inv_v + u0 + q * NT);
+          j[q] = __ldcg(X.inv_v + u0 + q * NT);
         }
       }
 #pragma unroll

@@ -76,3 +76,30 @@ def test_an_entry_far_above_its_warp(torch):  # noqa: F811
             got = run(torch, x, mode)
             compare(x, got, oracle(x, mode))
             assert got[3] == 0
+
+
+def test_another_map_on_the_same_workspace(torch):  # noqa: F811
+    # calls queued one behind another, each with a map of its own: what a call
+    # reads is the inverse map that its own check wrote
+    B, K, S, V = 2, 2, 30000, 40000
+    xs = [batch(B, K, S, V, V, synth.BF16, "any", 70 + i) for i in range(4)]
+    want = [run(torch, x, GREEDY) for x in xs]
+    keep = []
+    ws = torch.zeros(A.xvocab_workspace_bytes(B, K, S, V, V, A.BF16), dtype=torch.uint8, device="cuda")
+    for x in xs:
+        logits = [torch.from_numpy(v.view(np.int16)).view(torch.bfloat16).cuda()
+                  for v in (x.logits_full, x.logits_comp, x.logits_ver)]
+        ints = [torch.from_numpy(np.ascontiguousarray(v, np.int32)).cuda()
+                for v in (x.map_d, x.map_v, x.draft_tokens)]
+        keep.append((logits, ints, torch.full((2, B), -7, dtype=torch.int32, device="cuda")))
+    torch.cuda.synchronize()
+    for (a, b, t), (md, mv, d), out in keep:
+        st = A.fuse_verify_xvocab(a.data_ptr(), b.data_ptr(), V, t.data_ptr(), V, md.data_ptr(),
+                                  mv.data_ptr(), S, d.data_ptr(), 0, 0, B, K, A.BF16,
+                                  A.gate_params(mode=GREEDY), out[0].data_ptr(), out[1].data_ptr(),
+                                  0, ws.data_ptr(), ws.numel(), 0,
+                                  torch.cuda.current_stream().cuda_stream)
+        assert st == A.OK
+    torch.cuda.synchronize()
+    for (_, _, out), (L, N, _, _) in zip(keep, want):
+        assert np.array_equal(out.cpu().numpy(), np.stack([L, N]))
