@@ -171,6 +171,14 @@ __global__ void __launch_bounds__(kXInvThreads, 1) xvocab_gather_inv(XGatherPara
   const int S = max(0, min(part, P.S - j0)), V = P.V_v;
   const int tid = static_cast<int>(threadIdx.x), nt = static_cast<int>(blockDim.x);
   const T nan = x_nan<T>();
+  // A dependent of a kernel that starts it early has to wait for it, or what
+  // follows this grid could start before that kernel is done.  The last CTA
+  // does, at its end (in every CTA the wait would keep the next ones from
+  // starting beside that kernel).
+  auto wait_for_gather = [] {
+    if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1)
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+  };
   if (*P.map_err) {
     // the map check failed (a token out of range or in two pairs, which the
     // inverse map cannot express): read each pair's entry through map_v
@@ -178,6 +186,7 @@ __global__ void __launch_bounds__(kXInvThreads, 1) xvocab_gather_inv(XGatherPara
       const int u = __ldg(P.map_v + j0 + i);
       dst[i] = static_cast<unsigned>(u) < static_cast<unsigned>(V) ? src[u] : nan;
     }
+    wait_for_gather();
     return;
   }
   // a map that passed the check pairs every j with a distinct token in
@@ -222,6 +231,7 @@ __global__ void __launch_bounds__(kXInvThreads, 1) xvocab_gather_inv(XGatherPara
   const int nout = vec_out ? S / VE : 0;
   for (int i = tid; i < nout; i += nt) reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(out)[i];
   for (int i = nout * VE + tid; i < S; i += nt) dst[i] = out[i];
+  wait_for_gather();
 }
 
 // inv[v] = -1 for every token of both vocabularies; the map-error word is

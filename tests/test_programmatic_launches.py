@@ -21,3 +21,21 @@ def test_what_the_map_check_writes_is_not_read_as_read_only():
     assert {what for _, what in reads} == {"inv_v", "map_err"}
     assert all(load == "__ldcg" for load, _ in reads), reads
     assert len(reads) == len(re.findall(r"X\.(?:inv_v|map_err)\b", text))
+
+
+def test_every_programmatic_dependent_waits():
+    # a kernel launched with the attribute executes griddepcontrol.wait on every
+    # path that ends it (the wait may lie in a function it calls)
+    host = source("asymspec.cu")
+    assert host.count("programmaticStreamSerializationAllowed = 1") == 3
+    for name, kernel in (("kernel_tma.cuh", "decide_rows"), ("kernel_row.cuh", "decide_element"),
+                         ("kernel_full.cuh", "decide_full"), ("kernel_xrow.cuh", "fuse_verify_xrow"),
+                         ("kernel_xvocab.cuh", "xvocab_gather_inv")):
+        text = source(name)
+        body = text[text.index(" " + kernel + "("):].split("\ntemplate")[0]
+        first = re.search(r"griddepcontrol\.wait|\breturn;", body)
+        assert first and first.group().startswith("griddep"), kernel
+    # (the gather waits in its last CTA, through a lambda called before each exit)
+    body = source("kernel_xvocab.cuh").split(" xvocab_gather_inv(")[1].split("\ntemplate")[0]
+    assert len(re.findall(r"wait_for_gather\(\);\s*(?:return;|\})", body)) == 2
+    assert len(re.findall(r"\breturn;", body)) == 1
