@@ -50,30 +50,33 @@ def _run(cmd):
     return res.stderr
 
 
-def build_cuda(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale(CUDA_LIB, CUDA_SRC):
-        return CUDA_LIB
+def build_cuda(force: bool = False, verbose: bool = False, target: str = CUDA_LIB,
+               defines=()) -> str:
+    """The kernels' library (target, defines: a test's variant of it elsewhere)."""
+    if not force and not _stale(target, CUDA_SRC):
+        return target
     nvcc = nvcc_path()
     tag = f".tmp{os.getpid()}"
-    objs = [os.path.join(CSRC, os.path.basename(src)[:-3] + tag + ".o") for src in CUDA_SRC]
+    objs = [os.path.join(os.path.dirname(target) if defines else CSRC,
+                         os.path.basename(src)[:-3] + tag + ".o") for src in CUDA_SRC]
     base = [nvcc, "-gencode", GENCODE, "-O3", "-lineinfo", "-std=c++17", "-I" + INCLUDE,
-            "-Xcompiler", "-fPIC"]
+            "-Xcompiler", "-fPIC", *("-D" + d for d in defines)]
     if verbose:
         base.append("-Xptxas=-v")
     try:
         with ThreadPoolExecutor(len(CUDA_SRC)) as ex:
             logs = list(ex.map(_run, [base + ["-c", src, "-o", obj]
                                       for src, obj in zip(CUDA_SRC, objs)]))
-        tmp = CUDA_LIB + tag
+        tmp = target + tag
         _run([nvcc, "-shared", "-gencode", GENCODE, *objs, "-o", tmp])
-        os.replace(tmp, CUDA_LIB)
+        os.replace(tmp, target)
     finally:
         for obj in objs:
             if os.path.exists(obj):
                 os.remove(obj)
     if verbose:
         print("".join(logs))
-    return CUDA_LIB
+    return target
 
 
 def build_all(force: bool = False, verbose: bool = False) -> None:

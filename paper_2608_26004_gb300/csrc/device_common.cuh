@@ -441,15 +441,21 @@ struct KParams {
   int head0;            // fuse_verify_row, EDGE: elements from a 16-byte boundary to the logits
 };
 
-// What pass 1 leaves for the decision of a row: the normalisers, the
-// argmaxes, the data-error bits and the draft token's three logits.
+// What a row kernel leaves for the decision of a row: the normalisers, the
+// argmaxes and the data-error bits; from the staged kernel the draft token and
+// its three logits, from the streaming kernels what the row's second pass did
+// (kPath*) and the late word, which rank 0 clears when the cluster starts and
+// any CTA that gave up waiting for the cluster's records sets.
 struct __align__(16) RowStat {
   float lse[4];
   int is, it;
   unsigned bad;
-  int dtok;
+  int path;
+  union {
+    int dtok;
+    unsigned late;
+  };
   float da, db, dt;
-  int path;  // fuse_verify_row: what its second pass did (kPath*)
 };
 
 

@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
     fence_mbar_init();
     mbar_arrive_expect_tx(&sh->xbar, static_cast<unsigned>(nrec * sizeof(WF)));
   }
-  cluster_arrive_relaxed();
+  cluster_start(P, row32, rank);
   ring_prologue<T, true, true>(ring, g, i0, v1);
   const EdgeVals ed = load_edges<T, EDGE>(P, cut, row32, s0, b0, b1, true);
   cluster_wait();  // every CTA's barrier is initialised before any push
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
   }
   bool got = true;
   if (warp == 0) {
-    got = mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
+    got = wait_records(&sh->xbar, rank);
     float lse[4], vs, vt;
     int is, it;
     combine_full<EDGE>(recv, nrec, lse, vs, is, vt, it);
@@ -389,9 +389,9 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
         return hit ? vec * VE + __ffs(hit) - 1 - cut.head : INT_MAX;
       };
       const int es = element(is, vs, true), et = element(it, vt, false);
-      const unsigned bad = (got ? 0u : kBadTimeout) | (vs != vs ? kBadS : 0u) | (vt != vt ? kBadT : 0u);
+      const unsigned bad = (vs != vs ? kBadS : 0u) | (vt != vt ? kBadT : 0u);
       // the draft token's logits are read by the decision kernel itself
-      if (lane == 0) store_row_stat(P, row32, lse, es, et, bad, -1, 0.f, 0.f, 0.f, kPathFull);
+      if (lane == 0) store_stream_stat(P, row32, lse, es, et, bad, kPathFull);
     }
   }
   __syncthreads();
@@ -427,8 +427,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);
   }
-  // no CTA exits while a push to it may be in flight (as in fuse_verify_row)
-  if (warp == 0 && !got) mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
+  if (warp == 0 && !got) late_end(P, row32, &sh->xbar);
 }
 
 // Grid: (K + 1, B).  One warp decides in greedy mode; in stochastic mode the
@@ -456,7 +455,7 @@ __global__ void __launch_bounds__(STOCH ? kDrawThreads : 32) decide_full(const K
     rr.D = divergence_nats(P, x.j);
     rr.is = x.st.is;
     rr.it = x.st.it;
-    rr.bad = x.st.bad;
+    rr.bad = x.st.bad | x.st.late;
     rr.have_lse_t = true;
     if (STOCH) {
       const Draw dr = select_group(x.R, x.Q, bonus, din.sc.u_last, rr.mass);

@@ -63,8 +63,9 @@
 // Waits: one cluster barrier at the start (every CTA's mbarrier is
 // initialised before the first push), CTA barriers, its own cp.async groups,
 // and the record exchange's mbarrier, bounded by %globaltimer: a wait that
-// gives up reports ASYMSPEC_DATA_TIMEOUT for the row, and is waited for once
-// more (bounded) before the CTA exits, so that a late push finds it alive.
+// gives up, in any CTA of the cluster, reports ASYMSPEC_DATA_TIMEOUT for the
+// row (late_end), and is waited for once more (bounded) before the CTA exits,
+// so that a late push finds it alive.
 #pragma once
 
 #include "kernel_tma.cuh"
@@ -778,11 +779,41 @@ __device__ __forceinline__ void st_async16(const void* local, unsigned rank,
       "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(rb)
       : "memory");
 }
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+// Warp 0's wait for the records of the cluster; false: it gave up.
+__device__ __forceinline__ bool wait_records(unsigned long long* bar, int rank) {
+#ifdef ASYMSPEC_TEST_LATE_RANK  // a test build: the CTAs of one rank give up at once
+  if (rank == ASYMSPEC_TEST_LATE_RANK) return false;
+#endif
+  return mbar_wait_cluster_bounded(bar, 0, kCopyTimeoutNs);
+}
+// The end of a CTA whose warp 0 gave up.  Its normalisers, and so its path and its
+// masses, need not be the row's: it marks the row, whichever rank it has.  And no
+// CTA exits while a push to it may be in flight (once the barrier has completed
+// every push has landed): it waits once more, bounded, before it marks.
+__device__ __forceinline__ void late_end(const KParams& P, unsigned row, unsigned long long* bar) {
+  mbar_wait_cluster_bounded(bar, 0, kCopyTimeoutNs);
+  if ((threadIdx.x & 31) == 0)
+    atomicOr(&static_cast<RowStat*>(P.row_stat)[row].late, kBadTimeout);
+}
+// The start of a cluster: rank 0 clears the row's late word.  (Relaxed: a mark
+// follows only after the waits of late_end.  A release here, or a mark that every
+// CTA stores on every row, costs 64x7 bf16 V=128256 greedy 0.8 us of 59.5 and
+// 1x4 0.3 of 5.1; this form nothing.)
+__device__ __forceinline__ void cluster_start(const KParams& P, unsigned row, int rank) {
+  if (rank == 0 && threadIdx.x == 0) static_cast<RowStat*>(P.row_stat)[row].late = 0u;
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+// Rank 0: the row's normalisers, argmaxes, error bits and path (not the late word).
+__device__ __forceinline__ void store_stream_stat(const KParams& P, unsigned row,
+                                                  const float (&lse)[4], int is, int it,
+                                                  unsigned bad, int path) {
+  float4* st = reinterpret_cast<float4*>(static_cast<RowStat*>(P.row_stat) + row);
+  st[0] = make_float4(lse[0], lse[1], lse[2], lse[3]);
+  st[1] = make_float4(__int_as_float(is), __int_as_float(it), __uint_as_float(bad),
+                      __int_as_float(path));
 }
 // The row's pass-1 result from the n warp records of its cluster, by one
 // warp: the largest reference of each stream, every record's sum restated
@@ -926,7 +957,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
     fence_mbar_init();
     mbar_arrive_expect_tx(&sh->xbar, static_cast<unsigned>(nrec * sizeof(W1)));
   }
-  cluster_arrive_relaxed();
+  cluster_start(P, row32, rank);
   if (only_t) ring_prologue<T, false, true>(ring, g, i0, v1);
   else ring_prologue<T, true, true>(ring, g, i0, v1);
   const EdgeVals ed = load_edges<T, EDGE>(P, cut, row32, s0, b0, b1, !only_t);
@@ -985,7 +1016,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
       }
     }
     // every warp's record of the cluster is in this CTA once the barrier completes
-    got = mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
+    got = wait_records(&sh->xbar, rank);
     float ref[3], sum[3], v;
     int vec;
     combine_records<EDGE>(sh->recv(), nrec, ref, sum, v, vec);
@@ -1020,12 +1051,10 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
           if (hit) idx = vec * VE + __ffs(hit) - 1 - cut.head;
         }
       }
-      const unsigned bad = (got ? 0u : kBadTimeout) |
-                           (!STOCH && v != v ? (only_t ? kBadT : kBadS) : 0u);
+      const unsigned bad = !STOCH && v != v ? (only_t ? kBadT : kBadS) : 0u;
       // the draft token's logits are read by the decision kernel itself
       if (lane == 0)
-        store_row_stat(P, row32, lse, only_t ? INT_MAX : idx, only_t ? idx : INT_MAX, bad, -1, 0.f,
-                       0.f, 0.f, path);
+        store_stream_stat(P, row32, lse, only_t ? INT_MAX : idx, only_t ? idx : INT_MAX, bad, path);
     }
   }
   __syncthreads();
@@ -1057,10 +1086,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);
   }
-  // no CTA exits while a push to it may be in flight: once the barrier has
-  // completed every push has landed; after a wait that gave up, warp 0 waits
-  // once more (bounded) before the CTA may exit
-  if (warp == 0 && !got) mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
+  if (warp == 0 && !got) late_end(P, row32, &sh->xbar);
 }
 
 // ---------------------------------------------------------------- row decisions
@@ -1169,7 +1195,7 @@ __device__ __forceinline__ Draw select_group(const float (&Rm)[4], const float (
 
 // A row's statistics and its warps' records, as decided from (one warp; one
 // trip to the L2): the divergence sum (every lane) and the masses of groups
-// 4 lane .. 4 lane + 3.
+// 4 lane .. 4 lane + 3.  ng: the row's groups.
 struct RowRecords {
   RowStat st;
   float j, R[4], Q[4];
@@ -1182,7 +1208,7 @@ __device__ __forceinline__ RowRecords load_records(const KParams& P, long long r
   float4* dst = reinterpret_cast<float4*>(&x.st);
   dst[0] = __ldcg(src);
   dst[1] = __ldcg(src + 1);
-  dst[2] = __ldcg(src + 2);
+  x.st.late = __ldcg(&static_cast<const RowStat*>(P.row_stat)[row].late);
   float j = 0.f;
 #pragma unroll
   for (int h = 0; h < 4; ++h) {
@@ -1363,7 +1389,7 @@ __device__ __forceinline__ void decide_element(const KParams& P, const Rows& row
     rr.it = st.it;
     rr.sample = 0;  // the stop row's draw follows the scan
     rr.mass = NAN;
-    rr.bad = st.bad;
+    rr.bad = st.bad | st.late;
     rr.have_lse_t = !STOCH && !bonus;
     int4 rec = row_record<STOCH>(P, row, k, rr, din.dtok, din.ad, din.bd, din.td, din.sc, lane == 0);
     if (!bonus && st.path == kPathAccept) rec.x = 1;

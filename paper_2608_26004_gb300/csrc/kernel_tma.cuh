@@ -1176,18 +1176,18 @@ struct RowCtx {
 __device__ __forceinline__ void store_row_stat(const KParams& P, long long row,
                                                const float (&lse)[4], int is, int it,
                                                unsigned bad, int dtok, float ad, float bd,
-                                               float td, int path = 0) {
+                                               float td) {
   RowStat st;
 #pragma unroll
   for (int q = 0; q < 4; ++q) st.lse[q] = lse[q];
   st.is = is;
   st.it = it;
   st.bad = bad;
+  st.path = 0;
   st.dtok = dtok;
   st.da = ad;
   st.db = bd;
   st.dt = td;
-  st.path = path;
   static_cast<RowStat*>(P.row_stat)[row] = st;
 }
 

@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
     fence_mbar_init();
     mbar_arrive_expect_tx(&sh->xbar, static_cast<unsigned>(nrec * sizeof(W1)));
   }
-  cluster_arrive_relaxed();
+  cluster_start(P, row32, rank);
   build_t<T>(X, trow, tsh, j0, n);
   __syncthreads();
   cluster_wait();  // every CTA's barrier is initialised before any push
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
         dt = elem_ldg(trow + mv);
       }
     }
-    got = mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
+    got = wait_records(&sh->xbar, rank);
     float ref[3], sum[3], v;
     int vec;
     combine_records<true>(sh->recv(), nrec, ref, sum, v, vec);
@@ -476,11 +476,10 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
       sh->path = path;
     }
     if (rank == 0) {
-      const unsigned bad = (got ? 0u : kBadTimeout) |
-                           (!STOCH && v != v ? (only_t ? kBadT : kBadS) : 0u);
+      const unsigned bad = !STOCH && v != v ? (only_t ? kBadT : kBadS) : 0u;
       if (lane == 0)
-        store_row_stat(P, row32, lse, STOCH || only_t ? INT_MAX : vec,
-                       !STOCH && only_t ? vec : INT_MAX, bad, -1, 0.f, 0.f, 0.f, path);
+        store_stream_stat(P, row32, lse, STOCH || only_t ? INT_MAX : vec,
+                          !STOCH && only_t ? vec : INT_MAX, bad, path);
     }
   }
   __syncthreads();
@@ -506,8 +505,7 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
         P.pass2_rec + (static_cast<size_t>(row32) * nrec + rank * NW + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);
   }
-  // no CTA exits while a push to it may be in flight (as in fuse_verify_row)
-  if (warp == 0 && !got) mbar_wait_cluster_bounded(&sh->xbar, 0, kCopyTimeoutNs);
+  if (warp == 0 && !got) late_end(P, row32, &sh->xbar);
 }
 
 // The decisions over fuse_verify_xrow's rows; the emitted pair is committed as
