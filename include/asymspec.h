@@ -181,14 +181,13 @@ void asymspec_default_gate_params(asymspec_gate_params* p);
  * cluster size and dtype).  Layout, each part 256-byte aligned: 16 B of row
  * record per row and 4 B of ticket per element (all the generic kernel
  * needs); then, for ASYMSPEC_KERNEL_TMA with clusters of C CTAs, 48 B of
- * pass-1 results per row and 352 B per row and CTA of pass-2 record and
- * inverse-CDF group masses, which its decision kernel reads (its streaming
- * row kernels keep all they leave at the end of the workspace, clear of any
- * batch size's tickets).  With less than
- * the TMA part the automatic choice falls back to the generic kernel.  The tickets
- * must be zero before the first use (cudaMemset or
- * asymspec_workspace_reset); every call that completes leaves them zero
- * again, and every other part is written before it is read.  Two calls in
+ * pass-1 results per row and 576 B per row and CTA of pass-2 records and
+ * inverse-CDF group masses, which its decision kernel reads.  With less than
+ * the TMA part the automatic choice falls back to the generic kernel.  A call
+ * reads nothing from the workspace that it did not write itself (the generic
+ * kernel's tickets are cleared on `stream` first), so a workspace needs no
+ * zeroing and serves calls of any sizes it is large enough for, one after
+ * another; every call that completes leaves its tickets zero.  Two calls in
  * flight at the same time must not share a workspace. */
 size_t asymspec_workspace_bytes(int B, int K, int V);
 
@@ -216,7 +215,7 @@ int asymspec_fuse_verify(const void* logits_full, const void* logits_comp,
 /*
  * As asymspec_fuse_verify, with a caller-owned workspace and optional outputs:
  *   workspace, workspace_bytes: device scratch of asymspec_workspace_bytes()
- *       bytes, zeroed before first use (see above)
+ *       bytes (see above)
  *   out_row_stats:  [B, K+1, 8] fp32 device or NULL: per row LSE(a), LSE(b),
  *       LSE(t), LSE(s), D, gamma_eff, acceptance margin (greedy
  *       1 - ratio/gamma_eff, stochastic u - ratio/gamma_eff; NaN on row K) and
@@ -257,10 +256,9 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
  * before anything is enqueued.  Aligned rows run ASYMSPEC_KERNEL_TMA when
  * the array also holds its per-row results (48 + 576 C bytes a row for
  * clusters of C: about 890 rows at C = 8, 1190 at C = 6), else the generic
- * kernel.  Each call enqueues on `stream` a zero fill
- * of the B tickets (the only part that must start at zero), then the
- * launches of asymspec_fuse_verify_ex.  Nothing is allocated: no
- * cudaMalloc, cudaMallocAsync, cudaFree or library call that allocates.
+ * kernel.  Each call enqueues on `stream` what asymspec_fuse_verify_ex does.
+ * Nothing is allocated: no cudaMalloc, cudaMallocAsync, cudaFree or library
+ * call that allocates.
  *
  * Set-up: every call looks up the array's device address in the current
  * device's context with cudaGetSymbolAddress (return code checked,
@@ -301,8 +299,7 @@ int asymspec_fuse_verify_static(const void* logits_full, const void* logits_comp
  *   d_scratch, scratch_bytes: device memory of at least
  *       asymspec_host_scratch_bytes(B, K, V, dtype) bytes, 256-byte aligned:
  *       device copies of the inputs and outputs, then one workspace per
- *       chunk.  It needs no zeroing (each chunk's tickets are cleared on
- *       `stream` before its step).
+ *       chunk.  It needs no zeroing.
  * Host buffers should be page-locked (cudaMallocHost or cudaHostRegister)
  * for the copies to run asynchronously and overlap the kernels; pageable
  * buffers give the same results with the copies staged by the driver.
@@ -414,9 +411,8 @@ int asymspec_draft_sample(const void* logits, int rows, int V, int dtype, int mo
  *   out_next_index [B] int32 or NULL: the emitted pair index (-1 on a data
  *   error); workspace of
  *   asymspec_xvocab_workspace_bytes(B, K, S, V_d, V_v, dtype) bytes,
- *   256-byte aligned and zeroed before its first use
- *   (asymspec_workspace_reset; every call that completes leaves it fit for
- *   the next); out_error_word as for asymspec_fuse_verify_ex.  A map entry
+ *   256-byte aligned, which needs no zeroing; out_error_word as for
+ *   asymspec_fuse_verify_ex.  A map entry
  *   outside its vocabulary or a token in two pairs makes every batch element
  *   a data error (accept_len = next_token = -1, ASYMSPEC_DATA_BAD_MAP).
  *   Status codes are those of

@@ -322,13 +322,13 @@ def _stream(torch, dev) -> int:
 
 
 class FuseVerify:
-    """Holds a zeroed workspace for batches of up to B_max elements with K drafts.
+    """Holds a workspace for batches of up to B_max elements with K drafts.
 
     ``__call__`` takes CUDA tensors ([B, K+1, V] logits as float32 or
     bfloat16, int32 tokens, float32 probabilities and uniforms) and enqueues
     the step on the current stream.  Outputs are returned as tensors.  The
     workspace is sized for V_max vocabulary entries, or for the first call's
-    V when V_max is not given (and grown, zeroed, for a larger V).
+    V when V_max is not given (and grown for a larger V).
     """
 
     def __init__(self, B_max: int, K: int, device=None, V_max: int | None = None):

@@ -234,10 +234,14 @@ size_t cluster_ws_bytes(int B, int K) {
   return ws_records_bytes(B, K) + round_up(static_cast<size_t>(B) * sizeof(unsigned), 256);
 }
 
-// Workspace of the cluster TMA kernel for clusters of C CTAs: the records
-// and tickets first (same offsets), then what each row leaves for the
-// decision kernel: the row's pass-1 results, one pass-2 record per CTA and
-// each CTA's inverse-CDF group masses.
+// Workspace of the cluster kernels for clusters of C CTAs: the records and
+// tickets first (same offsets), then what each row leaves for the decision
+// kernel: the row's pass-1 results, one pass-2 record per CTA (staged) or warp
+// (streaming) and, from the staged kernel, each CTA's inverse-CDF group masses.
+// A workspace may serve calls of other sizes, and of other kernels, whose parts
+// lie over these: a call reads nothing but what it wrote itself.  The tickets,
+// which have to start at zero, are cleared by the call that uses them
+// (asymspec_fuse_verify_ex; fuse_verify_full clears its own).
 struct TmaLayout {
   size_t stat, p2rec, groups, total;
 };
@@ -255,25 +259,6 @@ TmaLayout tma_layout(int B, int K, int C, int group_stride = kGroupsMax) {
   L.groups = off;
   off += round_up(R * C * static_cast<size_t>(group_stride) * sizeof(float), 256);
   L.total = off;
-  return L;
-}
-
-// The streaming kernels' parts of a workspace that holds tma_layout(B, K, C):
-// at its end, where they take the room of the group masses too (those kernels
-// keep none).  A workspace may serve calls of other B, whose tickets must
-// still be zero then: they lie among its first bytes (after 16 (K + 1) a batch
-// element), which these parts leave alone.  fuse_verify_full clears its own.
-struct RowLayout {
-  size_t recs, tickets, stat, p2rec;
-};
-
-RowLayout row_layout(int B, int K, int C, size_t workspace_bytes) {
-  const size_t R = static_cast<size_t>(B) * (K + 1);
-  RowLayout L;
-  L.p2rec = (workspace_bytes - R * C * kRowMaxWarps * sizeof(X2)) / 256 * 256;
-  L.stat = L.p2rec - round_up(R * sizeof(RowStat), 256);
-  L.tickets = L.stat - round_up(static_cast<size_t>(B) * sizeof(unsigned), 256);
-  L.recs = L.tickets - ws_records_bytes(B, K);
   return L;
 }
 
@@ -787,18 +772,16 @@ int asymspec_fuse_verify_ex(const void* logits_full, const void* logits_comp,
   P.group_stride = pl.group_stride;
   if (pl.kernel == ASYMSPEC_KERNEL_TMA) {
     char* base = static_cast<char*>(workspace);
-    if (pl.row) {
-      const RowLayout L = row_layout(B, K, pl.C, workspace_bytes);
-      P.recs = reinterpret_cast<int4*>(base + L.recs);
-      P.tickets = reinterpret_cast<unsigned int*>(base + L.tickets);
-      P.row_stat = base + L.stat;
-      P.pass2_rec = reinterpret_cast<float*>(base + L.p2rec);
-    } else {
-      const TmaLayout L = tma_layout(B, K, pl.C, pl.group_stride);
-      P.row_stat = base + L.stat;
-      P.pass2_rec = reinterpret_cast<float*>(base + L.p2rec);
-      P.group_mass = reinterpret_cast<float*>(base + L.groups);
-    }
+    const TmaLayout L = tma_layout(B, K, pl.C, pl.group_stride);
+    P.row_stat = base + L.stat;
+    P.pass2_rec = reinterpret_cast<float*>(base + L.p2rec);
+    P.group_mass = reinterpret_cast<float*>(base + L.groups);
+  } else {
+    // Cleared by every call: another call's results may lie there.  (us a greedy
+    // step in calls, before -> after: B=1, K=4, V=4099 bf16 14.4 -> 15.1, B=8, K=5,
+    // V=1001 10.4 -> 12.4; 3 us in a graph.)
+    e = cudaMemsetAsync(P.tickets, 0, static_cast<size_t>(B) * sizeof(unsigned), cfg.stream);
+    if (e != cudaSuccess) return cuda_fail(e);
   }
   e = record_timing(opts, true, cfg.stream);
   if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, fn, args);
@@ -839,11 +822,6 @@ int asymspec_fuse_verify(const void* logits_full, const void* logits_comp,
   void* ws = nullptr;
   cudaError_t e = cudaMallocAsync(&ws, bytes, s);
   if (e != cudaSuccess) return cuda_fail(e);
-  e = cudaMemsetAsync(ws, 0, bytes, s);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(ws, s);
-    return cuda_fail(e);
-  }
   const int st = asymspec_fuse_verify_ex(logits_full, logits_comp, logits_ver, draft_tokens,
                                          draft_probs, uniforms, B, K, V, dtype, gate_params,
                                          out_accept_len, out_next_token, ws, bytes, nullptr,
@@ -866,12 +844,6 @@ int asymspec_fuse_verify_static(const void* logits_full, const void* logits_comp
   void* scratch = nullptr;
   int st = static_scratch(&scratch);
   if (st) return st;
-  // the tickets must start at zero; a call that did not complete may have
-  // left some set, so they are cleared on the caller's stream every time
-  cudaError_t e = cudaMemsetAsync(static_cast<char*>(scratch) + ws_records_bytes(B, K), 0,
-                                  static_cast<size_t>(B) * sizeof(unsigned),
-                                  static_cast<cudaStream_t>(stream));
-  if (e != cudaSuccess) return cuda_fail(e);
   return asymspec_fuse_verify_ex(logits_full, logits_comp, logits_ver, draft_tokens,
                                  draft_probs, uniforms, B, K, V, dtype, gate_params,
                                  out_accept_len, out_next_token, scratch, kStaticScratchBytes,
@@ -944,8 +916,6 @@ int asymspec_fuse_verify_host(const void* h_logits_full, const void* h_logits_co
     const size_t r0 = static_cast<size_t>(b0) * K1;
     char* ws = base + L.ws + static_cast<size_t>(c) * L.ws_each;
     e = cudaStreamWaitEvent(s, r->chunk[c], 0);
-    if (e == cudaSuccess)
-      e = cudaMemsetAsync(ws + ws_records_bytes(nb, K), 0, static_cast<size_t>(nb) * sizeof(unsigned), s);
     if (e != cudaSuccess) {
       cudaStreamSynchronize(r->copy);
       return cuda_fail(e);

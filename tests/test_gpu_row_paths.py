@@ -310,3 +310,37 @@ def test_recorded_rows_in_blocks_cut_on_lines(torch, V, cluster, mode):
     batch = synth.generate(synth.Recipe(), 11, 3, 2, V, synth.BF16)
     g = run_gpu(batch, torch, mode=mode, cluster_size=cluster)
     compare(batch, g, run_oracle(batch, mode=mode), mode=mode)
+
+
+@pytest.mark.parametrize("first,second", [
+    # (B, V, arguments) of two calls on one workspace, the one's records and
+    # results over the other's tickets:
+    ((64, 1001, {}), (4, 1001, {})),                                  # generic, both
+    ((4, 1001, {}), (64, 1001, {})),
+    ((8, 16392, dict(delta_source=A.DELTA_A)), (64, 1001, {})),       # staged, then generic
+    ((8, 16392, dict(row_tokens=True)), (64, 1001, {})),
+    ((64, 16392, {}), (4, 1001, {})),                                 # streaming, then generic
+    ((64, 1001, {}), (4, 16392, dict(row_stats=True))),
+    (None, (64, 1001, {})), (None, (4, 16392, dict(row_stats=True))), (None, (4, 16392, {})),
+    (None, (4, 16391, {})), (None, (4, 16392, dict(row_tokens=True))),
+])
+@pytest.mark.parametrize("own_size", [False, True])  # workspace_bytes of each call's own batch
+@pytest.mark.parametrize("mode", [GREEDY, STOCH])
+def test_whatever_lies_in_a_workspace(torch, mode, own_size, first, second):
+    K = 7
+    fv = A.FuseVerify(64, K, V_max=16392)
+    fv.workspace.fill_(255)  # (no call needs it zeroed)
+    whole = fv.nbytes
+    for B, V, args in (c for c in (first, second) if c):
+        batch = synth.generate(synth.Recipe(), 7, B, K, V, synth.BF16)
+        x = device_inputs(batch, torch)
+        out = {"accept_len": torch.full((B,), -7, dtype=torch.int32, device="cuda"),
+               "next_token": torch.full((B,), -7, dtype=torch.int32, device="cuda"),
+               "error_word": torch.zeros(1, dtype=torch.int32, device="cuda")}
+        fv.nbytes = A.workspace_bytes(B, K, V) if own_size else whole
+        fv(x["a"], x["b"], x["t"], x["tokens"], x["probs"], x["unif"], mode=mode, out=out, **args)
+    torch.cuda.synchronize()
+    o = run_oracle(batch, mode=mode, logprobs=False, delta_source=args.get("delta_source", A.DELTA_AB))
+    assert int(out["error_word"].item()) == 0
+    check_decisions(batch, np.arange(B), out["accept_len"].cpu().numpy(),
+                    out["next_token"].cpu().numpy(), o, mode)
