@@ -35,6 +35,10 @@
 //             group (recomputed against R) and the elements of the vector.
 //             If rounding leaves the target at or past a boundary with no
 //             owner, the last entry of positive mass is taken.
+// Finite logits of any size are taken.  What has a reference so far below zero that
+// x log2 e has no room for a fraction, or overflows (masks of the type's lowest
+// value), has no mass (greedy: thread_again); a row whose own reference lies there,
+// or as far above, is worked again by wide_row.
 // Non-finite data: every element also enters f = sum x 2^-40, finite
 // exactly when all elements are (2^-40 keeps 2^20 fp32 maxima finite).  A
 // row with a non-finite logit, or a uniform outside [0, 1), gets token -1
@@ -312,8 +316,25 @@ __device__ __forceinline__ float drescale(float mass, float ref, float R) {
 // error of the drawn token's probability against 64 bits, V = 32000 to 128256:
 // 2.3e-7 bf16, 2.6e-7 fp32 (references in nats 3.8e-7 and 4.3e-7, at the same speed).
 __device__ __forceinline__ float dref(float x) { return rintf(x * kLog2e); }
+// References (log2 units) from here on are too large for their exponents: below
+// it an exponent's rounding stays below 2^6, and a group's mass below kDGuard.
+constexpr float kDWideRef = 536870912.f;  // 2^29
 
 // ---------------------------------------------------------------- greedy slice
+
+// The thread's sum again, against its maximum m: it saw masks (or non-finite data)
+// before its first ordinary vector, or nothing else.
+template <typename T, bool EDGE>
+__device__ __noinline__ float thread_again(DRow<T, EDGE> a, int v0, int v1, float m) {
+  float s = 0.f;
+  if (!(-m * kLog2e < kDWideRef)) return s;
+  for (int v = v0 + static_cast<int>(threadIdx.x); v < v1; v += kDThreads) {
+    float x[DRaw<T>::VE];
+    dwiden(dld<T, EDGE>(a, v), x);
+    s += dmass(x, -m * kLog2e);
+  }
+  return s;
+}
 
 template <typename T, bool EDGE>
 __device__ __forceinline__ DSlice slice_greedy(const DRow<T, EDGE>& a, int v0, int v1, uint4* ring,
@@ -346,7 +367,8 @@ __device__ __forceinline__ DSlice slice_greedy(const DRow<T, EDGE>& a, int v0, i
       if (v < v1) take(raw[u], v, su[u]);
     }
   });
-  const float s = (su[0] + su[1]) + (su[2] + su[3]);
+  float s = (su[0] + su[1]) + (su[2] + su[3]);
+  if (!dfinite(s)) s = thread_again<T, EDGE>(a, v0, v1, m);
   // the CTA maximum, the lowest vector holding it, the sum rescaled to it
   const float w = dwarp_max(m);
   if (lane == 0) sh.red[warp] = w;
@@ -460,7 +482,8 @@ __device__ __forceinline__ DSlice slice_sample(const DRow<T, EDGE>& a, int v0, i
     tot = 0.f;
     DFin<T> unused;
     dring_start<T, EDGE>(ring, a, v0, v1);
-    slice_masses<T, EDGE, false>(a, v0, v1, ref, ring, gm, tot, unused);
+    // (a slice of nothing but masks: no mass)
+    slice_masses<T, EDGE, false>(a, v0, v1, -ref < kDWideRef ? ref : INFINITY, ring, gm, tot, unused);
     __syncthreads();  // every warp has read sh.red
   }
   const float wt = dwarp_sum(tot), wf = dwarp_sum(fin.value());
@@ -575,6 +598,44 @@ __device__ __forceinline__ void slice_walk(const DParams& P, const DRow<T, EDGE>
   P.probs[row] = pr;
 }
 
+// A whole row by one warp, masses against the row's maximum M formed as x - M
+// first: rows without a logit within 3.7e8 of zero.  best: the greedy draw.
+template <typename T, bool EDGE, bool STOCH>
+__device__ __forceinline__ void wide_row(DParams P, DRow<T, EDGE> a, int row, int best) {
+  const int lane = threadIdx.x & 31;
+  auto logit = [&](int i) { return to_f32(a.base[a.head + i]); };
+  float M = -INFINITY;
+  for (int i = lane; i < a.V; i += 32) M = fmaxf(M, logit(i));
+  M = dwarp_max(M);
+  auto mass = [&](int i) { return ex2((logit(i) - M) * kLog2e); };
+  const int seg = (a.V + 31) / 32, i0 = min(a.V, lane * seg), i1 = min(a.V, i0 + seg);
+  float s = 0.f;
+  for (int i = i0; i < i1; ++i) s += mass(i);
+  const float incl = dwarp_incl_scan(s, lane), S = __shfl_sync(0xffffffffu, incl, 31);
+  int tok = best;
+  float m = 1.f;  // the maximum's
+  if (STOCH) {
+    const float tau = P.unif[row] * S;
+    const unsigned over = __ballot_sync(0xffffffffu, s > 0.f && incl > tau);
+    const unsigned pos = __ballot_sync(0xffffffffu, s > 0.f);
+    if (lane != (over ? __ffs(over) - 1 : 31 - __clz(pos))) return;
+    float cum = incl - s;
+    for (int i = i0; i < i1; ++i) {
+      const float q = mass(i);
+      cum += q;
+      if (q > 0.f) {  // the last entry of positive mass, unless one passes the target
+        tok = i;
+        m = q;
+        if (cum > tau) break;
+      }
+    }
+  } else if (lane != 0) {
+    return;
+  }
+  P.tokens[row] = tok;
+  P.probs[row] = m / S;
+}
+
 // ------------------------------------------------------------------- the kernel
 
 // Grid: rows x C CTAs in clusters of C.  Shared memory: the ring, then
@@ -611,10 +672,15 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const __grid_constant_
       P.tokens[row] = ok ? idx : -1;
       P.probs[row] = ok ? 1.f / S : NAN;  // the maximum's own mass is 2^0
     }
+    if (rank == 0 && !(fabsf(R) * kLog2e < kDWideRef) && dfinite(F))
+      wide_row<T, EDGE, STOCH>(P, a, row, idx);
   } else {
     const float u = P.unif[row];
-    if (!(dfinite(F) && dfinite(R) && u >= 0.f && u < 1.f)) {
-      if (rank == 0 && lane == 0) {
+    if (!(dfinite(F) && u >= 0.f && u < 1.f && fabsf(R) < kDWideRef)) {
+      if (rank != 0) return;
+      if (dfinite(F) && u >= 0.f && u < 1.f) {
+        wide_row<T, EDGE, STOCH>(P, a, row, -1);
+      } else if (lane == 0) {
         P.tokens[row] = -1;
         P.probs[row] = NAN;
       }

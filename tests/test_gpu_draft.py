@@ -265,11 +265,56 @@ def test_draft_rows_off_the_vector_boundaries(torch, V, dtype, mode):
         logits = base
     u = rng.uniform(0, 1, rows).astype(np.float32)
     o = O.draft_sample(logits, u, dtype=dtype, mode=mode)
-    ok = np.arange(rows) != 2  # (its exponents overflow fp32 in sampling)
+    ok = np.arange(rows) != 2  # (V equal logits; in float64 too the LSE of such loses ln V)
     for offset in (0, 1, 3, 5):
         tok, pr = run(torch, logits, dtype, mode, u if mode == STOCH else None, offset)
-        if mode == GREEDY:
-            assert tok[2] == 0
+        assert abs(tok[2] - (0 if mode == GREEDY else int(u[2] * V))) <= (mode == STOCH)
+        np.testing.assert_allclose(pr[2], 1.0 / V, rtol=PROB_RTOL)
         good = ok & ~o.flagged
         assert np.array_equal(tok[good], o.tokens[good])
         np.testing.assert_allclose(pr[good], o.probs[good], rtol=PROB_RTOL)
+
+
+@pytest.mark.parametrize("mode", [GREEDY, STOCH], ids=["greedy", "stochastic"])
+@pytest.mark.parametrize("dtype", [synth.FP32, synth.BF16], ids=["fp32", "bf16"])
+@pytest.mark.parametrize("mask", ["lowest", -1e30, -1e9, 1e38])
+@pytest.mark.parametrize("V", [128, 32768, 33331])
+def test_draft_masked_rows(torch, V, mask, dtype, mode):
+    # masks at finite values far from the logits, the type's lowest among them:
+    # the end, the start, nearly all and all of a row (1e38: no mask, but logits
+    # far above the others); slices of one row with nothing but masks
+    rows = 4
+    rng = np.random.default_rng(V)
+    base = rng.normal(0, 2, (rows, V)).astype(np.float32)
+    low = -3.4028235e38 if dtype == synth.FP32 else -3.3895314e38
+    value = np.float32(low if mask == "lowest" else mask)
+    base[0, V // 3:] = value
+    base[1, :V - V // 5] = value
+    base[2, rng.random(V) < 0.97] = value
+    base[3] = value
+    logits = (base.view(np.uint32) >> 16).astype(np.uint16) if dtype == synth.BF16 else base
+    u = rng.uniform(0, 1, rows).astype(np.float32)
+    o = O.draft_sample(logits, u, dtype=dtype, mode=mode)
+    # the probability by its definition, differences from the maximum first
+    wide = O.widen(logits, dtype)
+    e = np.exp(wide - wide.max(1, keepdims=True))
+    for cluster in (0, 1, 8):
+        x = torch.from_numpy(logits.view(np.int16)).view(torch.bfloat16) \
+            if dtype == synth.BF16 else torch.from_numpy(logits)
+        tok, pr = A.draft_tokens(x.cuda(), torch.from_numpy(u).cuda() if mode == STOCH else None,
+                                 mode=mode, cluster_size=cluster)
+        tok, pr = tok.cpu().numpy(), pr.cpu().numpy()
+        want = e[np.arange(rows), tok] / e.sum(1)
+        np.testing.assert_allclose(pr, want, rtol=PROB_RTOL)
+        if mode == GREEDY:
+            assert np.array_equal(tok, wide.argmax(1))
+        else:  # (rows of equal logits: u V near a whole number may round to it)
+            tied = e.sum(1) == np.count_nonzero(e, axis=1)
+            cum = np.cumsum(e, 1)
+            t = u.astype(np.float64) * cum[:, -1]
+            near = np.abs(cum - t[:, None]).min(1) < 1e-6 * cum[:, -1]
+            good = ~o.flagged & ~tied & ~near
+            assert np.array_equal(tok[good], (cum <= t[:, None]).sum(1)[good])
+            r = np.arange(rows)
+            assert np.all(cum[r, tok] >= t - 1e-6 * cum[:, -1])
+            assert np.all(cum[r, tok] - e[r, tok] <= t + 1e-6 * cum[:, -1])
