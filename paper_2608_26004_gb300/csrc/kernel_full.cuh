@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(kRowThreads, kFullMinBlocks) fuse_verify_full(
       jsum = row_jsd_wide<T, EDGE>(g, v0, v1, A2, B2, ed);
   }
   if (lane == 0) {
-    const float qf = STOCH && e.s[3] > 0.f ? e.s[3] * ex2(EDGE ? fmaf(e.ref[3], kLog2e, -S2) : e.ref[3] - S2) : 0.f;
+    const float qf = STOCH ? block_mass<EDGE>(e.ref[3], e.s[3], S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

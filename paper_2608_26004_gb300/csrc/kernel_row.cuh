@@ -242,6 +242,18 @@ __device__ __forceinline__ float record_lse(float ref, float sum) {
   return NATS ? ref + logf(sum) : lse_of(ref, sum);
 }
 
+// The fused mass of a warp's block from its pass-1 sum: the group masses of a bonus
+// row's draw, and of a draft row's where the whole residual is zero.  A block below
+// 2^-100 has none: every entry of it, formed as the draw forms it (res_pair), may
+// be flushed to zero (below 2^-126), and a draw at u = 0 would find no token.  (At
+// most 2^12 entries a block and 2^7 blocks a row, so one that counts is kept, and
+// has an entry that is not flushed.)
+template <bool NATS>
+__device__ __forceinline__ float block_mass(float ref, float sum, float S2) {
+  const float m = sum > 0.f ? sum * ex2(NATS ? fmaf(ref, kLog2e, -S2) : ref - S2) : 0.f;
+  return m >= 7.888609052210118e-31f ? m : 0.f;
+}
+
 // What pass 2 does for a row (row_path): nothing, the residual masses alone,
 // or the divergence (and, in stochastic mode, the masses).
 enum : int { kPathFull = 0, kPathAccept = 1, kPathReject = 2 };
@@ -1078,10 +1090,8 @@ __global__ void __launch_bounds__(kRowThreads, kRowMinBlocks) fuse_verify_row(co
       jsum = row_jsd_wide<T, EDGE>(g, v0, v1, A2, B2, ed);
   }
   if (lane == 0 && (second || (STOCH && !draft))) {
-    // this warp's record: its block is one inverse-CDF group of the row.  The
-    // fused mass (the bonus row's draw, and a draft row's where the row's
-    // whole residual is zero) comes from the warp's pass-1 sum.
-    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(EDGE ? fmaf(e.ref[2], kLog2e, -S2) : e.ref[2] - S2) : 0.f;
+    // this warp's record: its block is one inverse-CDF group of the row
+    const float qf = STOCH ? block_mass<EDGE>(e.ref[2], e.s[2], S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + ((static_cast<size_t>(row32) * C + rank) * kRowMaxWarps + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParam
       jsum = x_jsd_wide<T>(x, p0, p1, A2, B2);
   }
   if (lane == 0 && (second || (STOCH && !draft))) {
-    const float qf = STOCH && e.s[2] > 0.f ? e.s[2] * ex2(fmaf(e.ref[2], kLog2e, -S2)) : 0.f;
+    const float qf = STOCH ? block_mass<true>(e.ref[2], e.s[2], S2) : 0.f;
     *reinterpret_cast<float4*>(
         P.pass2_rec + (static_cast<size_t>(row32) * nrec + rank * NW + warp) * 8) =
         make_float4(jsum, msum, qf, 0.f);

@@ -318,3 +318,18 @@ def test_draft_masked_rows(torch, V, mask, dtype, mode):
             r = np.arange(rows)
             assert np.all(cum[r, tok] >= t - 1e-6 * cum[:, -1])
             assert np.all(cum[r, tok] - e[r, tok] <= t + 1e-6 * cum[:, -1])
+
+
+@pytest.mark.parametrize("top", [0.0, -0.2])
+@pytest.mark.parametrize("cluster", [1, 8])
+def test_draft_at_zero_beside_flushed_masses(torch, cluster, top):
+    # u = 0, and the row's first entries around the smallest mass of fp32: a token
+    # of positive mass is drawn, not an error
+    bits = np.concatenate([np.arange(-128.0, -99.0, 0.125), np.arange(-126.6, -125.8, 0.01)])
+    logits = np.full((bits.size, 16384), -20.0, np.float32)
+    logits[:, :2048] = (bits * np.log(2.0))[:, None]
+    logits[:, 9000] = top
+    tok, pr = run(torch, logits, synth.FP32, STOCH, np.zeros(bits.size, np.float32),
+                  cluster_size=cluster)
+    assert np.all(tok >= 0) and np.all(pr > 0)
+    assert np.all((tok == 0) | (tok == 2048))

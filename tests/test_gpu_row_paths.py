@@ -344,3 +344,24 @@ def test_whatever_lies_in_a_workspace(torch, mode, own_size, first, second):
     assert int(out["error_word"].item()) == 0
     check_decisions(batch, np.arange(B), out["accept_len"].cpu().numpy(),
                     out["next_token"].cpu().numpy(), o, mode)
+
+
+@pytest.mark.parametrize("top", [0.0, -0.2])
+@pytest.mark.parametrize("full", ["row", True])
+@pytest.mark.parametrize("V", [16384, 16387])
+def test_a_draw_at_zero_beside_flushed_masses(torch, V, full, top):
+    # bonus rows drawn at u = 0, their first entries around the smallest mass of
+    # fp32: a token of positive mass is drawn, not an error
+    bits = np.concatenate([np.arange(-128.0, -99.0, 0.125), np.arange(-126.6, -125.8, 0.01)])
+    B = bits.size
+    t = np.full((B, 2, V), -20.0, np.float32)
+    t[..., 9000] = top
+    t[:, 1, :4096] = (bits * np.log(2.0))[:, None]
+    x = {n: torch.zeros(B, 2, V, device="cuda") for n in "ab"}
+    tokens = torch.full((B, 1), 9000, dtype=torch.int32, device="cuda")
+    r = A.FuseVerify(B, 1)(x["a"], x["b"], torch.from_numpy(t).cuda(), tokens,
+                           torch.full((B, 1), 1e-3, device="cuda"), torch.zeros(B, 2, device="cuda"),
+                           mode=STOCH, row_stats=full is True)
+    L, N = r["accept_len"].cpu().numpy(), r["next_token"].cpu().numpy()
+    assert int(r["error_word"].item()) == 0 and np.all(L == 1)
+    assert np.all((N == 0) | (N >= 2048) & (N <= 4096))
