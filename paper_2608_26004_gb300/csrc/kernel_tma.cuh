@@ -987,14 +987,6 @@ __device__ __forceinline__ void pass2_and_store(const T* ra, const T* rb, const 
   }
 }
 
-// The divergence of Eq. 3 from the summed pass-2 records (nats).
-template <unsigned G>
-__device__ __forceinline__ float divergence_of(const X2& tot) {
-  if (G & G_JSD) return 0.5f * kLn2 * (tot.j + tot.msum);
-  if (G & G_KL) return kLn2 * tot.kl;
-  return 0.f;
-}
-
 // ---------------------------------------------------------------- inverse-CDF walk
 
 // Masses of vector v of a slice held in global memory, as pass 2 computes them.
