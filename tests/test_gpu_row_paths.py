@@ -365,3 +365,37 @@ def test_a_draw_at_zero_beside_flushed_masses(torch, V, full, top):
     L, N = r["accept_len"].cpu().numpy(), r["next_token"].cpu().numpy()
     assert int(r["error_word"].item()) == 0 and np.all(L == 1)
     assert np.all((N == 0) | (N >= 2048) & (N <= 4096))
+
+
+@pytest.mark.parametrize("mode,div", [(STOCH, A.DIV_JSD), (STOCH, A.DIV_KL), (STOCH, A.DIV_NONE),
+                                      (GREEDY, A.DIV_JSD)])
+def test_more_elements_than_the_streaming_grid_holds(torch, mode, div):
+    # above 65535 elements the staged kernel's production programs run: the same
+    # decisions as on the streaming kernel (in halves), and as the oracle's on a few
+    B, K, V = 65540, 1, 64
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    a, b, t = (2 * torch.randn(B, K + 1, V, generator=gen, device="cuda") for _ in range(3))
+    b = a + 0.5 * b
+    a, b, t = (v.bfloat16() for v in (a, b, t))
+    tokens = a[:, :K].float().argmax(-1).int()
+    probs = a[:, :K].float().softmax(-1).max(-1).values
+    unif = torch.rand(B, K + 1, generator=gen, device="cuda")
+    assert A.plan(B, K, V, A.BF16, A.gate_params(mode=mode, divergence=div)).kernel == A.KERNEL_TMA
+
+    def step(s):
+        r = A.FuseVerify(s.stop - s.start, K)(a[s], b[s], t[s], tokens[s], probs[s], unif[s], mode=mode,
+                                              divergence=div)
+        assert int(r["error_word"].item()) == 0
+        return np.stack([r["accept_len"].cpu().numpy(), r["next_token"].cpu().numpy()])
+
+    whole = step(slice(0, B))
+    halves = np.concatenate([step(slice(0, B // 2)), step(slice(B // 2, B))], 1)
+    assert np.mean((whole != halves).any(0)) < 1e-3  # (near ties)
+    sel = np.r_[0:40, B - 40:B]
+    bits = [v[sel].contiguous().view(torch.int16).cpu().numpy().view(np.uint16) for v in (a, b, t)]
+    few = synth.generate(synth.Recipe(), 1, sel.size, K, V, synth.BF16)
+    few.logits_full[:], few.logits_comp[:], few.logits_ver[:] = bits
+    few.draft_tokens[:], few.draft_probs[:] = tokens[sel].cpu().numpy(), probs[sel].cpu().numpy()
+    few.uniforms[:] = unif[sel].cpu().numpy()
+    o = run_oracle(few, mode=mode, divergence=div, logprobs=False)
+    check_decisions(few, np.arange(sel.size), whole[0, sel], whole[1, sel], o, mode)
