@@ -83,10 +83,12 @@ def peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-def kernel_name(A, info) -> str:
-    """The row kernel a call launches (the roofline's kernel)."""
-    if info.kernel == A.KERNEL_TMA:  # both modes of the production program
-        return "fuse_verify_row"
+def kernel_name(A, info, elt) -> str:
+    """The row kernel a call launches (the roofline's kernel): the staged one
+    holds its slices of the three rows in shared memory."""
+    if info.kernel == A.KERNEL_TMA:
+        staged = not info.row_kernel and info.smem_bytes >= 3 * info.slice_elems * elt
+        return "fuse_verify_tma" if staged else "fuse_verify_row"
     return "fuse_verify_generic" if info.kernel == A.KERNEL_GENERIC else str(info.kernel)
 
 
@@ -666,7 +668,7 @@ def main():
                      "frac": achieved / hbm_peak, "peak_kind": peak_kind,
                      "traffic": measured_traffic(args.mode),
                      "algorithmic_bytes_per_launch": alg_bytes,
-                     "kernel": kernel_name(A, info),
+                     "kernel": kernel_name(A, info, 2),
                      "launch_us": kernel_ms * 1e3,
                      "launch_us_pct": percentiles(kern_us),
                      "timing": "CUDA events the library records around the fused row kernel "

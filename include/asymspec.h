@@ -71,8 +71,8 @@ extern "C" {
 #define ASYMSPEC_DATA_BAD_PROB 0x4u     /* stochastic: draft probability outside (0, 1] */
 #define ASYMSPEC_DATA_BAD_UNIFORM 0x8u  /* stochastic: uniform outside [0, 1) */
 #define ASYMSPEC_DATA_TIMEOUT 0x10u     /* a bulk copy into shared memory (staged row kernel) or the
-                                           exchange of the cluster's pass-1 records (production row
-                                           kernel) did not complete within its time limit (the
+                                           exchange of the cluster's pass-1 records (streaming row
+                                           kernels) did not complete within its time limit (the
                                            kernel gave up instead of hanging) */
 #define ASYMSPEC_DATA_BAD_MAP 0x20u     /* cross-family step: a map entry outside its vocabulary */
 
@@ -169,7 +169,9 @@ typedef struct {
                               (a cluster row kernel and its decision kernel) */
   int32_t row_kernel;      /* 1 if ASYMSPEC_KERNEL_TMA runs its production row kernel
                               (fuse_verify_row: the step without per-row outputs,
-                              delta = a - b) in stochastic mode, 0 otherwise */
+                              delta = a - b) in stochastic mode, 0 otherwise (a greedy
+                              step runs it too, unless ASYMSPEC_KERNEL_TMA or a test hook
+                              is asked for, but its plan says 0) */
 } asymspec_launch_info;
 
 /* Fills *p with the paper's defaults: gamma 0.5, beta 1.0, lambda 0.1,

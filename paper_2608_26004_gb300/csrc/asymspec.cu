@@ -136,10 +136,18 @@ bool plan_tma(int V, int elt, int forced_C, Plan* pl) {
 //     C=6 23.1 / 20.5; V=64000 fp32 B=16 19.6 / 15.3, 18.2 / 14.9 and (the worst of 20) B=22
 //     C=4 22.8 / 18.0, C=6 23.5 / 18.6
 // (The recording kernel is not held to that: B=12, K=4, V=128256 bf16 greedy C=4 26.6, C=8 30.1.)
-// Smaller batches take C = 8.  A warp's block takes at most kWalkRounds
-// steps (the decision kernel's draw takes one vector of a block per thread).  Only the
-// pass-1 records live in shared memory.  forced_C: the caller's
-// asymspec_launch_opts.
+// Smaller batches take C = 8: no size is best there, and 8 within 5 % of the best
+// where several are measured (us a step):
+//   B=8, K=5, V=151936 bf16 stochastic: C=5 18.2, 6 17.6, 7 18.3, 8 17.8, 10 18.0, 12 18.3, 16 17.4;
+//     greedy 13.8, 13.6, 14.4, 14.4, 15.1, 14.3, 14.9; recorded (greedy) 23.3, 26.8, 24.9, 23.9,
+//     27.0, 27.8, 31.1
+//   B=1, K=4, V=32000 fp32 greedy: C=4 5.3, 6 5.3, 8 5.1, 12 5.1, 16 5.1
+//   B=4, K=4, V=128256 bf16 stochastic: C=4 12.8, 6 10.9, 8 11.5, 12 10.7, 16 10.2 (the one it loses)
+// Rows too wide for C = 8 take the largest that fits (V=151936 fp32, B=4, K=4 stochastic: C=10
+// 14.8, 12 14.3, 16 14.9).  The rule does not count how full the last wave is.
+// A warp's block takes at most kWalkRounds steps (the decision kernel's draw takes one
+// vector of a block per thread).  Only the pass-1 records live in shared memory.
+// forced_C: the caller's asymspec_launch_opts.
 constexpr int kRowClusters[] = {4, 5, 6, 7, 8, 10, 12, 16};
 constexpr double kRowL2Budget = 86.0e6;
 
@@ -288,8 +296,8 @@ RowProgram row_program(const asymspec_gate_params& gp, bool full, bool tokens) {
 
 // Rows off the 16-byte boundaries stream too: the generic kernel reads them
 // element by element (greedy bf16, K=4: 98 us at B=32, V=100003 against 23
-// streaming; 16 against 7 at B=8, V=16385, the shortest measured).  Shorter
-// rows keep the generic kernel's single launch.
+// streaming; 16 against 7 at B=8, V=16385).  That is the shortest row measured, not
+// where the two cross: shorter rows keep the generic kernel, unmeasured.
 constexpr int kEdgeMinV = 16384;
 
 // How a call's rows lie in memory: every row on a 16-byte boundary; a, b and t

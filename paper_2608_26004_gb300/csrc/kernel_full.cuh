@@ -7,9 +7,11 @@
 // stochastic mode, the fused log-probabilities.  The staged kernel
 // (kernel_tma.cuh) held whole slices, two CTAs an SM: 384 CTAs of B=8, K=5,
 // V=151936 bf16 took two waves, 48 us a step; here three CTAs share an SM and
-// the loads of the next steps overlap the arithmetic.  What bounds it: the
-// issue of about 45 instructions per entry, then HBM (the log-probabilities
-// are 4 bytes written per entry against 6 read in bf16).
+// the loads of the next steps overlap the arithmetic.  What bounds it: at B=24
+// nothing alone (40 instructions per entry in greedy mode at 53 % of the issue
+// slots, the transcendental unit at 38 %, DRAM active half of the time; the
+// log-probabilities are 4 bytes written per entry against 6 read in bf16); a wave
+// or less, as B=8, has the latencies of fuse_verify_row.
 //
 // decide_full, one CTA per row: the row's divergence and record; in
 // stochastic mode every row's draw (the row tokens report it); the last row

@@ -23,8 +23,9 @@
 // and for rejected rows; the rest of the rows end after pass 1.  The results
 // are those of running it for every row.
 //
-// What bounds it: HBM (pass 1 is about 12 instructions per vocabulary entry,
-// a third of the issue slots at the copy bandwidth).  Layout:
+// What bounds it: HBM at B=64 (0.83 of the copy rate; 22 instructions per
+// vocabulary entry on the benchmark's rows, about half of the issue slots);
+// launch, ramp, exchange and decision where a batch is a wave or less.  Layout:
 //   * no slice is held in shared memory.  Each warp owns a contiguous block
 //     of the slice and reads it through a small ring in shared memory (kRing
 //     steps of 32 consecutive 16-byte vectors per stream, filled with
@@ -49,8 +50,10 @@
 //     a sum of small non-negative terms with no cancellation at the end (a
 //     block where e overflows is summed again term by term, row_jsd_wide);
 //   * the residual max(0, q_f - p) and fused score (t + beta (a - b)) log2 e
-//     are formed exactly as the decision kernel's inverse-CDF walk forms
-//     them (res_pair), so its group masses and the walk agree bit for bit.
+//     are formed exactly as the decision kernel's draw forms them (res_pair), so
+//     a group has residual mass only if an entry of it has.  The fused group
+//     masses (bonus rows; a draft row without residual) are the warps' pass-1
+//     sums and differ from the draw's by roundings (block_mass).
 //
 // EDGE: rows that do not start on a 16-byte boundary (V * element size not a
 // multiple of 16, or an offset base), with a, b and t at the same offset.
@@ -160,10 +163,10 @@ static_assert(kRowThreads / 32 <= kRowMaxWarps, "one record slot per warp");
 // row's vector s0: equal parts.  LINES (the recording kernel's aligned rows):
 // parts that start on the row's 128-byte lines, so that a step's 512 bytes lie in
 // four lines and not five, but for blocks of almost the most vectors a draw
-// takes, which are cut anywhere.  Recorded, greedy, V=128256 bf16: B=8, K=4 21.9 -> 20.1 us, B=64, K=7
-// 145.9 -> 139.3; V=64000 fp32 B=64, K=7 108.6 -> 107.5 (the worst of 16: B=20, K=5
-// stochastic 39.6 -> 39.9).  (fuse_verify_row's
-// blocks stay equal: lines took B=64, K=7 stochastic from 66.9 to 67.5.)
+// takes, which are cut anywhere.  Recorded, greedy, V=128256 bf16: B=8, K=4 21.9 ->
+// 20.1 us, B=64, K=7 145.9 -> 139.3; V=64000 fp32 B=64, K=7 108.6 -> 107.5 (the
+// worst of 16: B=20, K=5 stochastic 39.6 -> 39.9).  (fuse_verify_row's blocks stay
+// equal: lines took B=64, K=7 stochastic from 66.9 to 67.5.)
 template <bool LINES>
 __device__ __forceinline__ void row_block(int s0, int nv, int w, int& b0, int& b1) {
   constexpr int NW = kRowThreads / 32;
@@ -858,7 +861,9 @@ __device__ __forceinline__ void combine_records(const W1* rec, int n, float (&re
     const W1 r = rec[i];
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-      sum[q] += (r.s[q] == 0.f || r.ref[q] == ref[q]) ? r.s[q] : r.s[q] * ref_factor<NATS>(r.ref[q] - ref[q]);
+      sum[q] += (r.s[q] == 0.f || r.ref[q] == ref[q])
+                    ? r.s[q]
+                    : r.s[q] * ref_factor<NATS>(r.ref[q] - ref[q]);
     if (r.v == v) lo = min(lo, r.vec);
   }
   float z = 0.f;

@@ -17,15 +17,15 @@
 //     block of pairs being its inverse-CDF group.
 // The decision kernel commits the emitted pair as its verifier token.
 //
-// What bounds it: per CTA of that shape (C = 2) about 18 us of building t'
-// (the scattered 16-bit stores take 3.7 bank cycles a warp, and the loads
-// before them are waited for in bursts) and 11 us of pass 1 (a warp's load of
-// 32 scattered entries holds the L1 for about four cycles: 12.7 cycles per 32
-// pairs); HBM's share of its bytes is 10 us.  Tried: a and b in token order with wide loads
-// and a word per eight tokens that says which are paired (pass 1 10 % slower:
-// more instructions, and the unpaired tokens are worked too); C = 1 (215 us:
-// the slice leaves the L1 no room to keep the sectors that neighbouring lanes
-// share); 512-thread CTAs, two an SM (227 us, the same).
+// What bounds it: latency and the L1, not HBM (B=24, K=7 of those rows: DRAM
+// active 26 % of the time, the L1 at 61 % of its peak; 46 % of the shared-memory
+// wavefronts are bank conflicts, of the scattered 16-bit stores that build t'; a
+// warp waits 4.6 issue slots per instruction on global loads, two of 16 bits per
+// pair).  Tried: a and b in token order with wide loads and a word per eight
+// tokens that says which are paired (pass 1 10 % slower: more instructions, and
+// the unpaired tokens are worked too); C = 1 (215 us: the slice leaves the L1 no
+// room to keep the sectors that neighbouring lanes share); 512-thread CTAs, two an
+// SM (227 us, the same).
 #pragma once
 
 #include "kernel_row.cuh"
@@ -368,8 +368,9 @@ __host__ __device__ constexpr int xrow_shared_bytes(int C) {
   return static_cast<int>(sizeof(RowShared) + C * kXRowWarps * sizeof(W1));
 }
 
-// Grid: C B (K+1) CTAs of kXRowThreads threads in clusters of C, one CTA an SM.  P.V = S; P.tokens holds pair indices.  Leaves what
-// fuse_verify_row leaves, C kXRowWarps records a row.
+// Grid: C B (K+1) CTAs of kXRowThreads threads in clusters of C, one CTA an SM.
+// P.V = S; P.tokens holds pair indices.  Leaves what fuse_verify_row leaves, C
+// kXRowWarps records a row.
 template <typename T, bool STOCH>
 __global__ void __launch_bounds__(kXRowThreads, 1) fuse_verify_xrow(const KParams P,
                                                                     const XRowParams X) {
