@@ -322,6 +322,15 @@ constexpr float kDWideRef = 536870912.f;  // 2^29
 
 // ---------------------------------------------------------------- greedy slice
 
+// The log2 units a greedy thread's masses are formed against: its maximum m times
+// log2 e, rounded (a rescale takes the difference of two such, and greedy_mass takes
+// the rounding out at the end: for m = 1e5 it is 2^-9 of a mass).
+__device__ __forceinline__ float dlog2(float m) { return __fmul_rn(m, kLog2e); }
+// A sum of masses against dlog2(m), restated against m.
+__device__ __forceinline__ float greedy_mass(float s, float m) {
+  return s * ex2(fmaf(-m, kLog2e, dlog2(m)));
+}
+
 // The thread's sum again, against its maximum m: it saw masks (or non-finite data)
 // before its first ordinary vector, or nothing else.
 template <typename T, bool EDGE>
@@ -331,9 +340,9 @@ __device__ __noinline__ float thread_again(DRow<T, EDGE> a, int v0, int v1, floa
   for (int v = v0 + static_cast<int>(threadIdx.x); v < v1; v += kDThreads) {
     float x[DRaw<T>::VE];
     dwiden(dld<T, EDGE>(a, v), x);
-    s += dmass(x, -m * kLog2e);
+    s += dmass(x, -dlog2(m));
   }
-  return s;
+  return greedy_mass(s, m);
 }
 
 template <typename T, bool EDGE>
@@ -350,13 +359,13 @@ __device__ __forceinline__ DSlice slice_greedy(const DRow<T, EDGE>& a, int v0, i
     dwiden(raw, x);
     const float vm = dvmax(x);
     if (vm > m) {  // strict: the lowest vector of this thread keeps the maximum
-      const float f = ex2((m - vm) * kLog2e);
+      const float f = ex2(__fsub_rn(dlog2(m), dlog2(vm)));
 #pragma unroll
       for (int u = 0; u < kDUnroll; ++u) su[u] *= f;
       m = vm;
       bvec = v;
     }
-    s += dmass(x, -m * kLog2e);
+    s += dmass(x, -dlog2(m));
     fin.add(raw);
   };
   dring_start<T, EDGE>(ring, a, v0, v1);
@@ -367,7 +376,7 @@ __device__ __forceinline__ DSlice slice_greedy(const DRow<T, EDGE>& a, int v0, i
       if (v < v1) take(raw[u], v, su[u]);
     }
   });
-  float s = (su[0] + su[1]) + (su[2] + su[3]);
+  float s = greedy_mass((su[0] + su[1]) + (su[2] + su[3]), m);
   if (!dfinite(s)) s = thread_again<T, EDGE>(a, v0, v1, m);
   // the CTA maximum, the lowest vector holding it, the sum rescaled to it
   const float w = dwarp_max(m);

@@ -277,12 +277,12 @@ def test_draft_rows_off_the_vector_boundaries(torch, V, dtype, mode):
 
 @pytest.mark.parametrize("mode", [GREEDY, STOCH], ids=["greedy", "stochastic"])
 @pytest.mark.parametrize("dtype", [synth.FP32, synth.BF16], ids=["fp32", "bf16"])
-@pytest.mark.parametrize("mask", ["lowest", -1e30, -1e9, 1e38])
+@pytest.mark.parametrize("mask", ["lowest", -1e30, -1e9, -1e7, -1e5, 1e4, 1e38])
 @pytest.mark.parametrize("V", [128, 32768, 33331])
 def test_draft_masked_rows(torch, V, mask, dtype, mode):
     # masks at finite values far from the logits, the type's lowest among them:
-    # the end, the start, nearly all and all of a row (1e38: no mask, but logits
-    # far above the others); slices of one row with nothing but masks
+    # the end, the start, nearly all and all of a row (1e4 and 1e38: no masks, but
+    # logits far above the others); slices of one row with nothing but masks
     rows = 4
     rng = np.random.default_rng(V)
     base = rng.normal(0, 2, (rows, V)).astype(np.float32)
